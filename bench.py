@@ -51,10 +51,10 @@ METRIC = "dd-Rgemm/Rsyrk GFlops vs roofline; sliced vs plain at bound; p50/p99 s
 UNIT = "dd-GFlop/s"
 # nominal FP64 rate of GB300 (1.25 TFLOP/s counting an FMA as two flops) ->
 # 625 G FP64 instructions per second; a dd multiply-add in the GEMM kernels
-# costs 12.75 of them (1 DMUL + 3 DFMA + 8 DADD, FastTwoSum every 4 steps)
+# costs 9.75 of them (1 DMUL + 3 DFMA + 5 DADD, FastTwoSum every 4 steps)
 NOMINAL_FP64_INSTR = 1.25e12 / 2
-FP64_OPS_PER_MAC = 12.75
-QD_OPS_PER_MAC = 117.5   # qd multiply-add: 113 FP64 operations + 4.5 for the level pass
+FP64_OPS_PER_MAC = 9.75
+QD_OPS_PER_MAC = 73.25   # qd multiply-add: 71 FP64 operations + 2.25 for the level pass
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from single ncu
 # captures of the current kernels (the summaries under profiles/ give the
 # commands): the plain Rgemm NN launch at 4096 and the band kernel of the
@@ -364,7 +364,7 @@ def plain_section(mp, torch, size, problems, r64, rmac=None):
     """The plain FP64 path on the step's three problems, one call each timed
     with CUDA events (after the split-precision runs on the same inputs).
     Fractions: of 2 R64 / 15 (the survey's accounting, R64 the measured FP64
-    FMA rate), of the FP64 pipe at the kernel's 12.75 instructions per
+    FMA rate), of the FP64 pipe at the kernel's 9.75 instructions per
     multiply-add, and of the measured rate of the kernel's own multiply-add
     mix with operands in registers (mp_dd_peak_ddmac)."""
     nn, tn, syrk, dnn, dtn, dsy = problems
@@ -852,7 +852,7 @@ def routines_section(mp, torch, size):
     out[f"Rgetrf_{n}"]["info"] = int(info.item())
     del A, B, C, A0
     out.update(potrf_section(mp, torch, n, info))
-    # quad-double Rgemm (117.5 FP64 instructions per qd multiply-add)
+    # quad-double Rgemm (73.25 FP64 instructions per qd multiply-add)
     nq = min(n, 1024)
     gq = datagen.rng(5)
     Aq, Bq, Cq = (dev(datagen.qd_matrix(gq, nq, nq)) for _ in range(3))

@@ -15,12 +15,53 @@ struct dd {
     double hi, lo;
 };
 
-// Knuth TwoSum: s + e == a + b exactly, s = fl(a + b).  6 FP64 operations.
-__device__ __forceinline__ void two_sum(double a, double b, double &s, double &e) {
-    s = __dadd_rn(a, b);
-    double bv = __dsub_rn(s, a);
-    double av = __dsub_rn(s, bv);
-    e = __dadd_rn(__dsub_rn(a, av), __dsub_rn(b, bv));
+// Rounded sum and difference: the intrinsics on the device, plain binary64
+// on the host (where the check of two_sum compiles this header).
+__host__ __device__ __forceinline__ double add_rn(double a, double b) {
+#if defined(__CUDA_ARCH__)
+    return __dadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+__host__ __device__ __forceinline__ double sub_rn(double a, double b) {
+#if defined(__CUDA_ARCH__)
+    return __dsub_rn(a, b);
+#else
+    return a - b;
+#endif
+}
+
+// The leading 32 bits of |x|, shifted left by one: they order like the
+// exponents of finite numbers, and like the magnitudes up to the trailing
+// 32 significand bits.
+__host__ __device__ __forceinline__ unsigned int lead_bits(double x) {
+#if defined(__CUDA_ARCH__)
+    return (unsigned int)__double2hiint(x) << 1;
+#else
+    unsigned long long u;
+    __builtin_memcpy(&u, &x, 8);
+    return (unsigned int)(u >> 32) << 1;
+#endif
+}
+
+// TwoSum: s + e == a + b exactly, s = fl(a + b).  Knuth's form takes 6 FP64
+// operations because it does not know which operand is the larger.  Here the
+// leading words are compared and the operands exchanged on the integer pipe
+// (7 instructions), after which Dekker's form needs 3: it is exact whenever
+// the exponent of the first operand is at least that of the second.  e is the
+// rounding error of s in either form, so the result is the same number bit
+// for bit (the sign of a zero e aside; when s overflows, e is an infinity
+// here and a NaN there, and the next renormalisation makes both NaN).
+// An FP64 instruction occupies its partition of the SM for ~76 cycles and an
+// integer one for 2, and every dd kernel is bound by the FP64 pipe: a dd
+// multiply-add falls from 12.75 to 9.75 FP64 instructions, and the multiply-
+// add mix of the plain kernel measured 85.9 before and 113.9 dd-GFlop/s now.
+__host__ __device__ __forceinline__ void two_sum(double a, double b, double &s, double &e) {
+    const bool swap = lead_bits(b) > lead_bits(a);
+    const double big = swap ? b : a, small = swap ? a : b;
+    s = add_rn(a, b);
+    e = sub_rn(small, sub_rn(s, big));
 }
 
 // Dekker FastTwoSum (|a| >= |b| or a == 0): s + e == a + b.  3 operations.
@@ -40,7 +81,7 @@ __device__ __forceinline__ void prod_terms(dd a, dd b, double &p, double &e) {
 }
 
 // acc += (p + e), renormalised: TwoSum on the leading parts, the low parts
-// added, FastTwoSum.  11 FP64 operations; absolute error at most ~2u^2
+// added, FastTwoSum.  8 FP64 operations; absolute error at most ~2u^2
 // (|acc| + |p|) per step (u = 2^-53).
 __device__ __forceinline__ void acc_add(dd &acc, double p, double e) {
     double s, t;
@@ -49,7 +90,7 @@ __device__ __forceinline__ void acc_add(dd &acc, double p, double e) {
     fast_two_sum(s, t, acc.hi, acc.lo);
 }
 
-// One dd multiply-add: acc += a * b (15 FP64 operations).
+// One dd multiply-add: acc += a * b (12 FP64 operations).
 __device__ __forceinline__ void mac(dd &acc, dd a, dd b) {
     double p, e;
     prod_terms(a, b, p, e);
@@ -61,7 +102,7 @@ __device__ __forceinline__ void mac(dd &acc, dd a, dd b) {
 // part are added into acc.lo, and the FastTwoSum is left to renorm(), which
 // the GEMM kernels call after every kRenormEvery steps of k (at l = 3, 7, 11,
 // ... counted from the start of k, so every kernel renormalises at the same
-// places).  4 + 6 + 2 = 12 FP64 operations per step, 12.75 with the
+// places).  4 + 3 + 2 = 9 FP64 operations per step, 9.75 with the
 // renormalisation.  Between renormalisations |acc.lo| stays within a few
 // ulps of acc.hi, so each step's rounding error is at most ~(G+4) u^2
 // (|acc| + |a b|) with G = 4: within the Rgemm bound 4 k 2^-104 (...).  A
@@ -103,7 +144,7 @@ __device__ __forceinline__ dd add(dd a, dd b) {
 }
 
 // Sloppy dd addition (TwoSum on the leading parts, low parts added,
-// FastTwoSum): 11 FP64 operations, absolute error at most ~2u^2 (|a| + |b|)
+// FastTwoSum): 8 FP64 operations, absolute error at most ~2u^2 (|a| + |b|)
 // (the relative error can be large under cancellation).  Used where the
 // accuracy target is the absolute bound 4 k 2^-104 (|alpha||A||B| +
 // |beta||C|), e.g. the final alpha/beta combination.

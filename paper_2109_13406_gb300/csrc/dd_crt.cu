@@ -432,8 +432,8 @@ struct CrtArgs {
 // alpha v + beta c in dd with one rounding chain: the two leading products
 // split exactly (product and FMA error), their sum by TwoSum, every
 // lower-order term added into the error word, one FastTwoSum.  Absolute error
-// within about 3u^2 (|alpha v| + |beta c|), u = 2^-53; 20 FP64 operations
-// against 25 for two dd products and a dd sum.
+// within about 3u^2 (|alpha v| + |beta c|), u = 2^-53; 17 FP64 operations
+// against 22 for two dd products and a dd sum.
 __device__ __forceinline__ dd axpby_dd(dd alpha, dd v, dd beta, dd c) {
     const double p1 = __dmul_rn(alpha.hi, v.hi), e1 = __fma_rn(alpha.hi, v.hi, -p1);
     const double p2 = __dmul_rn(beta.hi, c.hi), e2 = __fma_rn(beta.hi, c.hi, -p2);

@@ -10,7 +10,7 @@
 // products, TwoSum into the accumulator, and a FastTwoSum renormalisation
 // every 4 steps of k (dd_arith.cuh).
 //
-// On GB300 the FP64 pipe is the bottleneck by a wide margin (12.75 FP64
+// On GB300 the FP64 pipe is the bottleneck by a wide margin (9.75 FP64
 // instructions per dd multiply-add), so the kernel is organised to keep that
 // pipe busy and nothing else (large plain products go to the TMA-staged form
 // of this kernel, dd_gemm_tma.cu, whose per-entry arithmetic is identical): each CTA owns a 16R x 16R tile of C (R = 4, 2

@@ -16,8 +16,8 @@
 // products of order u^4 and below (within 7 u^4 |a b|), so the result
 // stays within the qd bound 4 k 2^-209 (|alpha||A||B| + |beta||C|).  Every
 // 4 steps one bottom-up TwoSum pass (L2+L3, L1+L2, L0+L1) brings level t
-// back to order u^t |acc|; the pass is exact.  113 FP64 operations per
-// step plus 4.5 for the pass.
+// back to order u^t |acc|; the pass is exact.  71 FP64 operations per
+// step plus 2.25 for the pass (113 and 4.5 with Knuth's six-operation TwoSum).
 //
 // Tiles: 16R x 16R of C per CTA (R = 2 or 1, the larger one when the tiles
 // still fill the SMs), R x R qd accumulators per thread, the four planes of

@@ -9,6 +9,8 @@ compiled as host code with nvcc.
   value when Z has at most 128 significant bits, and |hi + lo - Z 2^s| stays
   within (2^-106 + 2^-126) |Z 2^s| (plus the subnormal spacing), with
   overflow to a correctly signed infinity.
+* two_sum (dd_arith.cuh), which orders its operands by their leading words:
+  equal to Knuth's TwoSum over the whole binary64 range (hostcheck/two_sum.cu).
 """
 from __future__ import annotations
 
@@ -50,6 +52,15 @@ def test_triangle_items_match_the_skipping_raster(tmp_path):
     assert r.returncode == 0, r.stdout + r.stderr
     cases, bad = (int(x) for x in r.stdout.split()[1::2])
     assert cases > 3000 and bad == 0
+
+
+def test_two_sum_equals_knuths(tmp_path):
+    exe = str(tmp_path / "two_sum")
+    _build(os.path.join(HERE, "hostcheck", "two_sum.cu"), exe, shared=False)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    pairs, bad = (int(x) for x in r.stdout.split()[1::2])
+    assert pairs == 8000000 and bad == 0
 
 
 def test_words_to_dd_rounding(tmp_path):
