@@ -78,6 +78,9 @@ constexpr int kGroupFull = 8, kGroupTri = 4;
 // the extra arithmetic per drained value slows the MMAs.)
 constexpr int kEpiCols = 64;
 constexpr int kEpiColsWide = 128;
+// Digit products of fewer tiles than this take one work item per (band,
+// tile), the others one per tile (item_coords).
+constexpr int64_t kSplitTiles = 912;
 
 // Two tile widths: 128 x 128 (6-stage ring of 32 KB, 8 epilogue warps) and
 // 128 x 256 (4 stages of 48 KB, 8 epilogue warps, all 512 TMEM columns);
@@ -101,10 +104,20 @@ struct BandCfg {
 
 }  // namespace
 
-// Tile width used for an m x n product: the wide tile once there are enough
-// tiles to fill the GPU twice over.
+// Tile width of the digit products.  A 128 x 128 tile reads 128 bytes of
+// shared memory per clock for its MMAs, all there is, and takes as long as a
+// 128 x 256 tile (96 bytes per clock): 16.5 against 17.1 us per digit pair of
+// k = 3000, so the wide tile does the same columns in about half the time
+// (2048^3: 2255 us against 1197; 3000^3: 6586 against 3498).  The narrow one
+// stays where the wide would not fill n_pad (an odd count of 128-column
+// tiles; up to 255 tiles, where a wider padding could outgrow the built-in
+// scratch array) and up to 20 tiles, where the longest band sets the time
+// either way (items per band, see item_coords) and the narrow tile's is 7 %
+// shorter.
 int band_tn(int64_t m, int64_t n) {
-    return (ceil_div(m, TM) * ceil_div(n, 256) >= 304) ? 256 : 128;
+    const int64_t nt = ceil_div(n, 128), tiles = ceil_div(m, TM) * nt;
+    if (nt % 2 == 0) return tiles > 20 ? 256 : 128;
+    return nt > 1 && tiles >= 256 ? 256 : 128;
 }
 
 namespace {
@@ -307,25 +320,27 @@ __device__ __forceinline__ void tile_coords(int tile, int tiles_m, int tiles_n, 
     tm = local / gn;
 }
 
-// Work item -> output tile and the bands [b0, b1) it accumulates.  Digit
-// pairs (sliced form): one item per tile, all S bands, so each tile's int32
-// sums are finished in one visit.  Residues (diagonal mode): one item per
-// (modulus, tile) with the modulus slowest, so the CTAs resident at one time
-// share one modulus's operand panels in L2.
+// Work item -> output tile and the bands [b0, b1) it accumulates.
+// Residues (diagonal mode): one item per (modulus, tile) with the modulus
+// slowest, so the CTAs resident at one time share one modulus's operand
+// panels in L2.  Digit pairs (sliced form): band b sums b + 1 products.  Below
+// kSplitTiles tiles one item per (band, tile), the longest bands first, so
+// that few tiles fill the SMs and the short bands even out their ends; above,
+// one item per tile with all S bands, which keeps the CTAs on the same panels
+// for longer.  Band phase per call, one item per tile / per band:
+// 256^3 157 / 28 us, 512^3 296 / 62 us, 2048^3 1192 / 1073 us, 4096^3 (512
+// tiles) 9.42 / 8.94 ms, 5000^3 (800 tiles) 18.5 / 17.0 ms, 6000^3 (1128
+// tiles) 28.5 / 29.9 ms, 8192^3 71.8 / 93.0 ms.
 // Tiles entirely outside the requested triangle (Rsyrk form) get an empty
 // band range, so every role skips them alike.
 template <int TN, bool PAIR>
 __device__ __forceinline__ void item_coords(const BandArgs &p, int S, int item, int num_tiles,
                                             int rank, const int *tri_s, int &tm, int &tn,
                                             int &b0, int &b1) {
-    int tile = item;
-    b0 = 0;
-    b1 = S;
-    if (p.diag) {
-        b0 = item / num_tiles;
-        b1 = b0 + 1;
-        tile = item % num_tiles;
-    }
+    const int unit = item / num_tiles;
+    const int tile = item - unit * num_tiles;
+    b0 = p.diag ? unit : p.split ? S - 1 - unit : 0;
+    b1 = p.diag || p.split ? b0 + 1 : S;
     if (tri_s != nullptr) {
         // tile-th tile inside the triangle: the last (group, row unit) whose
         // cumulative count is at most tile, then the column within it
@@ -534,7 +549,7 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
 
     const int num_tiles = TRI ? p.tri_tiles : (PAIR ? p.tiles_m / 2 : p.tiles_m) * p.tiles_n;
     const int KB = p.kb_count;
-    const int num_items = p.diag ? num_tiles * S : num_tiles;
+    const int num_items = p.diag || p.split ? num_tiles * S : num_tiles;
 
     if (warp == 0) {
         // ---------------- TMA producer
@@ -1243,6 +1258,7 @@ int run_sliced(const GemmArgs &p, int slices, void *ws, size_t ws_bytes, cudaStr
     ba.P = P;
     ba.R = nullptr;
     ba.diag = 0;
+    ba.split = (int64_t)ba.tiles_m * ba.tiles_n < kSplitTiles;
     ba.status = &hdr->status;
     ba.plan = plan;
     if ((rc = launch_band(tmA, tmB, ba, TN, st, &tmB_half))) return rc;
@@ -1397,7 +1413,7 @@ int launch_band(const CUtensorMap &tmA, const CUtensorMap &tmB, const BandArgs &
     // work items (see item_coords; S: the most bands the plan may choose)
     const int units = pair ? b.tiles_m / 2 : b.tiles_m;
     const int tiles = b.tri_cum != nullptr ? b.tri_tiles : units * b.tiles_n;
-    const int items = b.diag ? tiles * b.S : tiles;
+    const int items = b.diag || b.split ? tiles * b.S : tiles;
     const bool tt = b.tri_cum != nullptr;
     if (pair) {
         const int clusters = items < pair_clusters() ? items : pair_clusters();

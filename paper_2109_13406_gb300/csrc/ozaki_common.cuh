@@ -93,6 +93,7 @@ struct BandArgs {
     uint8_t *R;   // [S][n_pad][m_pad] (diagonal mode)
     int *status;
     int diag;
+    int split;    // triangle mode: work items of one band each (else all bands of a tile)
     int tri;      // diagonal / magnitude mode: 1 / 2 = only the upper / lower triangle
     int moduli[kMaxBands];
     SplitPlan plan;

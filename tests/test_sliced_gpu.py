@@ -146,3 +146,29 @@ def test_wide_tiles_4096x4096_k256_bands_and_result(cuda_lib):
     assert np.array_equal(got_bands, P)
     rr, cc = sample_blocks(m, n, bs=16, count=8)
     assert check_against_exact(c, got, rr, cc) <= 1.0
+
+
+@pytest.mark.parametrize("shape", [(700, 640, 70), (700, 900, 70), (2600, 257, 33),
+                                   (7296, 3840, 40), (7290, 4090, 40)])
+def test_work_items_and_tile_widths(cuda_lib, shape):
+    """Products on either side of the rules for the tile width (30 narrow, 48
+    wide tiles, an odd count of 128-column tiles) and for the work items (855
+    tiles: one per band and tile; 912: one per tile): band sums at sampled
+    entries, the first and the last among them, bit-exact against the integer
+    oracle, the result within the bound."""
+    m, n, k = shape
+    S = 14
+    c = datagen.gemm_case(410 + k, "N", "N", m, n, k)
+    got, ws = run_sliced(cuda_lib, c, S)
+    L = cuda_lib.mp_dd_sliced_layout(m, n, k, S)
+    g = datagen.rng(411)
+    rows = np.concatenate([[0, m - 1], g.integers(0, m, 10)])
+    cols = np.concatenate([[0, n - 1], g.integers(0, n, 10)])
+    DA, _ = oz.split_matrix(*(x[rows] for x in oz.op_rows(c.A, False, m, k)), S)
+    DB, _ = oz.split_matrix(*(x[cols] for x in oz.op_cols(c.B, False, k, n)), S)
+    P = oz.band_products(DA, DB)
+    mp_, np_ = L["m_pad"], L["n_pad"]
+    bands = ws_view(ws, L["bands"], S * np_ * mp_, np.int32).reshape(S, np_, mp_)
+    assert np.array_equal(bands[:, cols][:, :, rows].transpose(0, 2, 1).astype(np.int64), P)
+    rr, cc = sample_blocks(m, n, bs=16, count=4)
+    assert check_against_exact(c, got, rr, cc) <= 1.0
