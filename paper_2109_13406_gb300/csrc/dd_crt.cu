@@ -927,14 +927,11 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     const int a_rc = p.ta ? 0 : 1, b_rc = p.tb ? 1 : 0;
     int rc;
     sliced_timing_mark(0, st);
-    if ((rc = launch_absmax(p.ah, p.lda, a_rc, p.m, p.k, rmax, st))) return rc;
-    if (!sym && (rc = launch_absmax(p.bh, p.ldb, b_rc, p.n, p.k, cmax, st))) return rc;
-    if ((rc = launch_magnitude(p.ah, p.lda, a_rc, p.m, p.k, L.m_pad, L.k_pad, rmax,
-                               w + L.off_ma, hdr, &init, st)))
-        return rc;
-    if (!sym && (rc = launch_magnitude(p.bh, p.ldb, b_rc, p.n, p.k, L.n_pad, L.k_pad, cmax,
-                                       w + L.off_mb, hdr, nullptr, st)))
-        return rc;
+    const SplitOperand oa{p.ah, p.al, p.lda, a_rc, p.m, L.m_pad, rmax, w + L.off_ma, 0};
+    const SplitOperand ob{p.bh, p.bl, p.ldb, b_rc, p.n, L.n_pad, cmax, w + L.off_mb, 0};
+    // (the Rsyrk form has one operand: its maxima and planes serve as both)
+    if ((rc = launch_absmax(oa, sym ? nullptr : &ob, p.k, st))) return rc;
+    if ((rc = launch_magnitude(oa, sym ? nullptr : &ob, p.k, L.k_pad, hdr, init, st))) return rc;
     int *tri_table = (p.tri && sym) ? reinterpret_cast<int *>(w + L.off_tri) : nullptr;
     if ((rc = launch_certificate(p, w + L.off_ma, w + L.off_mb, L.m_pad, L.n_pad, L.k_pad, TN,
                                  rmax, cmax, hdr, st, tri_table)))

@@ -143,8 +143,19 @@ __host__ __device__ inline void tri_range(const TriGeom &g, int grp, int u, int 
 // elem: 0 = fp16, 1 = bf16 elements.
 int make_tmap(CUtensorMap *m, void *base, int64_t rows, int64_t k_pad, int box_rows,
               int elem = 0);
-int launch_absmax(const double *X, int64_t ld, int row_contig, int64_t rows, int64_t k,
-                  unsigned long long *out, cudaStream_t st);
+// One operand of a call as rows x k (op(A), or op(B)^T): element (r, l) at
+// [r + l ld] (row_contig) or [l + r ld].
+struct SplitOperand {
+    const double *hi, *lo;
+    int64_t ld;
+    int row_contig;
+    int64_t rows, rows_pad;
+    unsigned long long *max;   // row maxima of |hi| (bit patterns)
+    void *mag;                 // magnitude plane [rows_pad][k_pad] bf16
+    unsigned blocks;           // its blocks of the launch (set by the launchers)
+};
+// Row maxima of the call's operands (b == nullptr: one) in one launch.
+int launch_absmax(const SplitOperand &a, const SplitOperand *b, int64_t k, cudaStream_t st);
 // tmB_half: the op(B) map with TN / 2-row boxes; given for a product that may
 // run on CTA pairs (NULL: single CTAs).
 int launch_band(const CUtensorMap &tmA, const CUtensorMap &tmB, const BandArgs &ba, int TN,
@@ -155,12 +166,11 @@ int band_tn(int64_t m, int64_t n);
 // Magnitude planes and the certificate (dd_sliced.cu).  form: 1 slices, 2
 // residues; widths[c] / counts[c] / cst[c] the candidates (ascending width)
 // and their per-product error constants.  make_plan also fills the header
-// image that the first magnitude launch writes (init != nullptr).
+// image that the magnitude launch writes.
 SplitPlan make_plan(SplitHeader *hdr_image, unsigned int *dmin_dev, int form, int64_t k,
                     int ncand, const int *widths, const int *counts, const double *cst);
-int launch_magnitude(const double *X, int64_t ld, int row_contig, int64_t rows, int64_t k,
-                     int64_t rows_pad, int64_t k_pad, const unsigned long long *rmax, void *M,
-                     SplitHeader *hdr, const SplitHeader *init, cudaStream_t st);
+int launch_magnitude(const SplitOperand &a, const SplitOperand *b, int64_t k, int64_t k_pad,
+                     SplitHeader *hdr, const SplitHeader &init, cudaStream_t st);
 // The magnitude product and its reduction into the header (MA [m_pad][k_pad],
 // MB [n_pad][k_pad] bf16).
 struct GemmArgs;
