@@ -54,148 +54,19 @@ __host__ __device__ constexpr int modulus(int i) {
     return m[i];
 }
 
-// 256^(kMaxDigits-1-u) mod p_i as exact floats (< 256), and 1/p_i.  Digit t
-// of a D-digit expansion has the weight w[i][kMaxDigits - D + t].
-struct ModWeights {
-    float w[kMaxMod][kMaxDigits];
-    float inv[kMaxMod];
-};
-
-constexpr ModWeights make_mod_weights() {
-    ModWeights mw{};
-    for (int i = 0; i < kMaxMod; ++i) {
-        const int p = modulus(i);
-        int v = 1;
-        for (int t = kMaxDigits - 1; t >= 0; --t) {
-            mw.w[i][t] = (float)v;
-            v = (v * 256) % p;
-        }
-        mw.inv[i] = 1.0f / (float)p;
-    }
-    return mw;
+// 256^t mod p_b.
+__host__ __device__ constexpr int pow256_mod(int t, int b) {
+    int v = 1 % modulus(b);
+    for (int u = 0; u < t; ++u) v = (v * 256) % modulus(b);
+    return v;
 }
 
-__constant__ ModWeights c_mod_weights = make_mod_weights();
-
-// The same weights, each duplicated into both halves of a float2, with the
-// packed constants of the quotient step: the residue kernel works on two
-// entries at once with the packed fp32 instructions (f32x2), whose lanes are
-// the same IEEE operations as the scalar ones.
-struct ModWeights2 {
-    float2 w[kMaxMod][kMaxDigits];
-    float2 inv[kMaxMod];
-    float2 negp[kMaxMod];
-};
-
-constexpr ModWeights2 make_mod_weights2() {
-    ModWeights2 m{};
-    const ModWeights s = make_mod_weights();
-    for (int i = 0; i < kMaxMod; ++i) {
-        for (int t = 0; t < kMaxDigits; ++t) m.w[i][t] = float2{s.w[i][t], s.w[i][t]};
-        m.inv[i] = float2{s.inv[i], s.inv[i]};
-        m.negp[i] = float2{-(float)modulus(i), -(float)modulus(i)};
-    }
-    return m;
-}
-
-__constant__ ModWeights2 c_mod_weights2 = make_mod_weights2();
-
-// Residues of an op(X) whose rows are contiguous in memory, on the FP32
-// pipe: 4 threads per (row, 16 consecutive k), 4 entries each, one 8-byte store
-// per residue plane and thread (a quad of lanes writes one 32-byte sector).
-// Residues from the balanced digits d_t of X on the FP32 pipe:
-// s = sum_t d_t (256^(D-1-t) mod p) is an integer below 16 * 128 * 255 < 2^24,
-// so every partial sum is exact in fp32, and r = s - p rint(s / p) is the
-// residue in [-(p-1)/2, (p-1)/2] for odd p: the fp32 quotient is within
-// |s / p| 2^-23 < 1e-3 of s / p, while s / p, an integer over an odd p, is
-// never within 1 / (2 p) > 0.0019 of a half-integer.  For p = 256 the
-// lowest digit, in [-128, 127], is the residue.  The first N planes are
-// written (N and D from the call's certificate).
-template <int NP, int DG>
-__device__ __forceinline__ void residue_rows_body(
-    const double *__restrict__ Xh, const double *__restrict__ Xl, int64_t ld, int row_contig,
-    int64_t rows, int64_t k, int64_t rows_pad, int64_t k_pad,
-    const unsigned long long *__restrict__ rmax, __half *__restrict__ R, int N) {
-    const int64_t r = (int64_t)blockIdx.x * (blockDim.x / 4) + threadIdx.x / 4;
-    if (r >= rows_pad) return;
-    const int64_t l0 = (int64_t)blockIdx.y * 16 + 4 * (threadIdx.x & 3);
-    const int e = r < rows ? scale_exponent(rmax[r]) : 0;
-    const int shift = 8 * DG - e;
-    // digits of the entry pairs (l0, l0 + 1) and (l0 + 2, l0 + 3), packed
-    float2 d2[2][DG];
-    int lowest[4];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        int dg[2][DG];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int64_t l = l0 + 2 * h + u;
-            double hi = 0.0, lo = 0.0;
-            if (r < rows && l < k) {
-                const int64_t off = row_contig ? (r + l * ld) : (l + r * ld);
-                hi = Xh[off];
-                lo = Xl[off];
-            }
-            dd_digits<DG>(hi, lo, shift, dg[u]);
-            lowest[2 * h + u] = dg[u][DG - 1];
-        }
-        // d as a float without a conversion instruction: the bits of
-        // 2^23 + 128 + d (exact, d in [-128, 128]) minus 2^23 + 128
-#pragma unroll
-        for (int t = 0; t < DG; ++t)
-            d2[h][t] = __fadd2_rn(float2{__int_as_float(0x4B000000 + 128 + dg[0][t]),
-                                         __int_as_float(0x4B000000 + 128 + dg[1][t])},
-                                  float2{-8388736.0f, -8388736.0f});
-    }
-    // plane 0 (p = 256): the lowest digits, exact in fp16
-    {
-        const __half2 h01 = __floats2half2_rn((float)lowest[0], (float)lowest[1]);
-        const __half2 h23 = __floats2half2_rn((float)lowest[2], (float)lowest[3]);
-        *reinterpret_cast<uint2 *>(R + r * k_pad + l0) =
-            make_uint2(*reinterpret_cast<const uint32_t *>(&h01),
-                       *reinterpret_cast<const uint32_t *>(&h23));
-    }
-    const float2 magic{12582912.0f, 12582912.0f}, nmagic{-12582912.0f, -12582912.0f};
-#pragma unroll
-    for (int i = 1; i < 2 * NP; ++i) {
-        if (i >= N) break;
-        uint32_t packed[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float2 s2{0.0f, 0.0f};
-#pragma unroll
-            for (int t = 0; t < DG; ++t)
-                s2 = __ffma2_rn(d2[h][t], c_mod_weights2.w[i][kMaxDigits - DG + t], s2);
-            // rint(s / p) by the 1.5 2^23 shift (|s / p| < 2^22), then the residue
-            const float2 qn = __fadd2_rn(__ffma2_rn(s2, c_mod_weights2.inv[i], magic), nmagic);
-            const float2 res = __ffma2_rn(c_mod_weights2.negp[i], qn, s2);
-            const __half2 hv = __float22half2_rn(res);
-            packed[h] = *reinterpret_cast<const uint32_t *>(&hv);
-        }
-        *reinterpret_cast<uint2 *>(R + ((int64_t)i * rows_pad + r) * k_pad + l0) =
-            make_uint2(packed[0], packed[1]);
-    }
-}
-
-template <int NP>
-__global__ void __launch_bounds__(128) residue_rows_kernel(
-    const double *__restrict__ Xh, const double *__restrict__ Xl, int64_t ld, int row_contig,
-    int64_t rows, int64_t k, int64_t rows_pad, int64_t k_pad,
-    const unsigned long long *__restrict__ rmax, __half *__restrict__ R, const SplitPlan plan) {
-    const PlanPick pk = plan_choice(plan);
-    if (pk.c < 0) return;
-    const int N = pk.count;
-    switch (pk.width) {
-        case 8 * 14:
-            residue_rows_body<NP, 14>(Xh, Xl, ld, row_contig, rows, k, rows_pad, k_pad, rmax, R, N);
-            break;
-        case 8 * 15:
-            residue_rows_body<NP, 15>(Xh, Xl, ld, row_contig, rows, k, rows_pad, k_pad, rmax, R, N);
-            break;
-        default:
-            residue_rows_body<NP, 16>(Xh, Xl, ld, row_contig, rows, k, rows_pad, k_pad, rmax, R, N);
-            break;
-    }
+// The fp16 bits of an integer in [0, 255] (exact).
+__host__ __device__ constexpr unsigned half_bits(int v) {
+    if (v == 0) return 0u;
+    int e = 0;
+    while ((v >> (e + 1)) != 0) ++e;
+    return ((unsigned)(e + 15) << 10) | (((unsigned)v << (10 - e)) & 0x3FFu);
 }
 
 // Residues on the tensor cores.  For an entry X (the scaled integer of
@@ -215,14 +86,26 @@ __global__ void __launch_bounds__(128) residue_rows_kernel(
 // sit in n-tiles of 8; the first N planes are written (N and D from the
 // call's certificate).
 //
-// A warp computes 32 entries: each lane forms X' of one entry, and the quad
-// exchanges words so that lane (g, q) holds bytes 2q, 2q+1, 2q+8, 2q+9 of
-// its four entries (the A fragments of two m16 tiles); its accumulators
-// then hold two moduli of four consecutive k, stored as one 8-byte write
-// per modulus.  Entries: rows r, columns l of op(X); with l contiguous in
-// memory (row_contig = 0) a warp takes 32 consecutive l of one row, else 4
-// consecutive l of 8 consecutive rows.
+// A warp computes 64 consecutive k of one row.  Each lane forms X' of two
+// entries and leaves its words in shared memory, from where lane (g, q) of the
+// warp's quads takes the bytes 2q, 2q+1, 2q+8, 2q+9 of the entries 8g .. 8g+7
+// (the A fragments of four m16 tiles); its accumulators then hold two moduli
+// of those eight consecutive k, stored as one 16-byte write per modulus (a
+// whole 128-byte line per modulus and warp).  Rows that are contiguous in
+// memory reach a block as a 16 x 64 tile, read along the rows and turned in
+// shared memory, so both layouts share the rest; the next entries are loaded
+// before the present ones are computed.  Both operands of a call go in one
+// launch of as many blocks as are resident.
+//
+// What bounds it: 16 bytes read and 64 written per entry (1.58 ms of HBM time
+// for both operands of an 8192 product) against instruction issue and the
+// shared-memory wavefronts of the tables (32 k per warp and 8-byte stores ran
+// the wavefronts at 74 % of their peak; they are at 84 % now).  Both operands of
+// an 8192 product: 2.03 ms, 0.78 of the copy rate; an FP32 kernel for the
+// row-contiguous operand and this one with 128-bit shifts left to the
+// compiler and a byte exchange by shuffles took 3.44 ms.
 constexpr int kResNT = (kMaxMod - 1 + 7) / 8;   // n-tiles of moduli 1 .. 39
+constexpr int kResThreads = 256, kResWarps = kResThreads / 32, kResBlocks = 3;
 
 // D = A B + C for one m16n8k16 tile: fp16 A (row) and B (col), fp32 C / D.
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint2 b,
@@ -235,167 +118,274 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
           "f"(c[2]), "f"(c[3]));
 }
 
-struct ResLane {     // per n-tile and lane: B fragment, accumulator starts,
-    uint32_t b0, b1; // and the reduction constants of the lane's 2 moduli
+struct alignas(16) ResLane {   // per n-tile and lane: B fragment, accumulator starts,
+    unsigned b0, b1;           // and the reduction constants of the lane's 2 moduli
     float init0, init1;
-    float4 inv, negp;   // {1/p0, 1/p0, 1/p1, 1/p1}, {-p0, -p0, -p1, -p1}
+    float inv[2], negp[2];     // {1/p0, 1/p1}, {-p0, -p1}
 };
 
-__device__ __forceinline__ uint32_t res_weight(int b, int t, int N, int DG) {
-    // 256^t mod p_b (0 past N or past the digit count); plane 0 is not here
-    return (b < N && t < DG) ? (uint32_t)c_mod_weights.w[b][kMaxDigits - 1 - t] : 0u;
-}
+// For D = 14, 15, 16 digit bytes; the moduli past a call's N are computed
+// with the others and not stored.
+struct ResTables {
+    ResLane t[kMaxDigits - kMinDigits + 1][kResNT * 32];
+};
 
-__device__ void res_setup(int N, int DG, ResLane *tab) {
-    for (int x = threadIdx.x; x < kResNT * 32; x += blockDim.x) {
-        const int lane = x % 32, nt = x / 32, g = lane >> 2, q = lane & 3;
-        const int bm = 1 + 8 * nt + g;   // B column g
-        auto h = [&](int t) {
-            return (uint32_t)__half_as_ushort(__uint2half_rn(res_weight(bm, t, N, DG)));
-        };
-        ResLane L;
-        L.b0 = h(2 * q) | (h(2 * q + 1) << 16);
-        L.b1 = h(2 * q + 8) | (h(2 * q + 9) << 16);
-        float init[2], inv[2], negp[2];
-        for (int e = 0; e < 2; ++e) {
-            const int m = 1 + 8 * nt + 2 * q + e;   // C column 2q + e
-            init[e] = inv[e] = negp[e] = 0.0f;
-            if (m < N) {
-                const int pm = modulus(m);
-                uint32_t ws = 0;
-                for (int t = 0; t < DG; ++t) ws += res_weight(m, t, N, DG);
-                const uint32_t bias = (128u * res_weight(m, DG - 1, N, DG)) % (uint32_t)pm;
-                init[e] = -1024.0f * (float)ws - (float)bias;   // exact: below 2^23
-                inv[e] = c_mod_weights.inv[m];
-                negp[e] = -(float)pm;
-            }
-        }
-        L.init0 = init[0];
-        L.init1 = init[1];
-        L.inv = make_float4(inv[0], inv[0], inv[1], inv[1]);
-        L.negp = make_float4(negp[0], negp[0], negp[1], negp[1]);
-        tab[x] = L;
-    }
-}
-
-template <int DG>
-__device__ __forceinline__ void residue_warp(
-    const double *__restrict__ Xh, const double *__restrict__ Xl, int64_t ld, int row_contig,
-    int64_t rows, int64_t k, int64_t rows_pad, int64_t k_pad,
-    const unsigned long long *__restrict__ rmax, __half *__restrict__ R, int N,
-    const ResLane *tab) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-    const int64_t lchunks = row_contig ? k_pad / 4 : k_pad / 32;
-    const int64_t items = row_contig ? (rows_pad / 8) * lchunks : rows_pad * lchunks;
-    const int ntiles = (N - 1 + 7) / 8;
-    const uint32_t sel = (q & 1) ? 0x4342u : 0x4140u;   // halfword q&1 as two fp16 1024 + x
-    const float2 magic{12582912.0f, 12582912.0f}, nmagic{-12582912.0f, -12582912.0f};
-    for (int64_t item = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; item < items;
-         item += (int64_t)gridDim.x * (blockDim.x / 32)) {
-        // this lane's entry and the four entries (same row, consecutive l) it stores
-        const int64_t a = item / lchunks, c = item - a * lchunks;
-        const int64_t row = row_contig ? 8 * a + g : a;
-        const int64_t lbase = row_contig ? 4 * c : 32 * c + 4 * g;
-        const int64_t l = lbase + q;
-        double hi = 0.0, lo = 0.0;
-        int e = 0;
-        if (row < rows) {
-            e = scale_exponent(rmax[row]);
-            if (l < k) {
-                const int64_t off = row_contig ? (row + l * ld) : (l + row * ld);
-                hi = Xh[off];
-                lo = Xl[off];
-            }
-        }
-        const int shift = 8 * DG - e;
-        const unsigned __int128 Xb = (unsigned __int128)(scaled_round(hi, shift) +
-                                                         scaled_round(lo, shift)) +
-                                     ((unsigned __int128)1 << (8 * DG - 1));
-        const uint32_t w0 = (uint32_t)Xb, w1 = (uint32_t)(Xb >> 32), w2 = (uint32_t)(Xb >> 64),
-                       w3 = (uint32_t)(Xb >> 96);
-        // words q/2 and 2 + q/2 of the quad's four entries
-        uint32_t lw[4], hw[4];
-#pragma unroll
-        for (int E = 0; E < 4; ++E) {
-            const int src = (lane & ~3) | E;
-            const uint32_t x0 = __shfl_sync(0xFFFFFFFFu, w0, src);
-            const uint32_t x1 = __shfl_sync(0xFFFFFFFFu, w1, src);
-            const uint32_t x2 = __shfl_sync(0xFFFFFFFFu, w2, src);
-            const uint32_t x3 = __shfl_sync(0xFFFFFFFFu, w3, src);
-            lw[E] = (q >> 1) ? x1 : x0;
-            hw[E] = (q >> 1) ? x3 : x2;
-        }
-        // plane 0 (p = 256): the lowest byte of X, signed; lane q = 0 holds it for all four
-        if (q == 0) {
-            const __half2 h01 = __floats2half2_rn((float)(int8_t)(lw[0] & 0xFFu),
-                                                  (float)(int8_t)(lw[1] & 0xFFu));
-            const __half2 h23 = __floats2half2_rn((float)(int8_t)(lw[2] & 0xFFu),
-                                                  (float)(int8_t)(lw[3] & 0xFFu));
-            *reinterpret_cast<uint2 *>(R + row * k_pad + lbase) =
-                make_uint2(*reinterpret_cast<const uint32_t *>(&h01),
-                           *reinterpret_cast<const uint32_t *>(&h23));
-        }
-        // A fragments of tile t: row g = entry 2t, row g + 8 = entry 2t + 1
-        uint32_t A[2][4];
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            A[t][0] = __byte_perm(lw[2 * t], 0x64646464u, sel);
-            A[t][1] = __byte_perm(lw[2 * t + 1], 0x64646464u, sel);
-            A[t][2] = __byte_perm(hw[2 * t], 0x64646464u, sel);
-            A[t][3] = __byte_perm(hw[2 * t + 1], 0x64646464u, sel);
-        }
-#pragma unroll
-        for (int nt = 0; nt < kResNT; ++nt) {
-            if (nt >= ntiles) break;
-            const ResLane L = tab[nt * 32 + lane];
-            const float c0[4] = {L.init0, L.init1, L.init0, L.init1};
-            float acc[2][4];
-            const uint2 bf = make_uint2(L.b0, L.b1);
-#pragma unroll
-            for (int t = 0; t < 2; ++t) mma_16816(acc[t], A[t], bf, c0);
-            const float2 inv0{L.inv.x, L.inv.y}, inv1{L.inv.z, L.inv.w};
-            const float2 np0{L.negp.x, L.negp.y}, np1{L.negp.z, L.negp.w};
-#pragma unroll
-            for (int e2 = 0; e2 < 2; ++e2) {   // the lane's moduli 1 + 8nt + 2q + e2
-                const int m = 1 + 8 * nt + 2 * q + e2;
-                uint32_t packed[2];
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    const float2 s2{acc[t][e2], acc[t][2 + e2]};   // entries 2t, 2t + 1
-                    const float2 qn =
-                        __fadd2_rn(__ffma2_rn(s2, e2 ? inv1 : inv0, magic), nmagic);
-                    const float2 rr = __ffma2_rn(e2 ? np1 : np0, qn, s2);
-                    const __half2 hv = __float22half2_rn(rr);
-                    packed[t] = *reinterpret_cast<const uint32_t *>(&hv);
+constexpr ResTables make_res_tables() {
+    ResTables T{};
+    for (int D = kMinDigits; D <= kMaxDigits; ++D)
+        for (int nt = 0; nt < kResNT; ++nt)
+            for (int lane = 0; lane < 32; ++lane) {
+                const int g = lane >> 2, q = lane & 3;
+                ResLane L{};
+                const int bm = 1 + 8 * nt + g;   // B column g
+                auto h = [&](int t) {
+                    return bm < kMaxMod && t < D ? half_bits(pow256_mod(t, bm)) : 0u;
+                };
+                L.b0 = h(2 * q) | (h(2 * q + 1) << 16);
+                L.b1 = h(2 * q + 8) | (h(2 * q + 9) << 16);
+                float init[2] = {0.0f, 0.0f};
+                for (int e = 0; e < 2; ++e) {
+                    const int m = 1 + 8 * nt + 2 * q + e;   // C column 2q + e
+                    if (m >= kMaxMod) continue;
+                    int ws = 0;
+                    for (int t = 0; t < D; ++t) ws += pow256_mod(t, m);
+                    const int bias = (128 * pow256_mod(D - 1, m)) % modulus(m);
+                    init[e] = (float)(-1024 * ws - bias);   // exact: below 2^23
+                    L.inv[e] = 1.0f / (float)modulus(m);
+                    L.negp[e] = -(float)modulus(m);
                 }
-                if (m < N)
-                    *reinterpret_cast<uint2 *>(R + ((int64_t)m * rows_pad + row) * k_pad + lbase) =
-                        make_uint2(packed[0], packed[1]);
+                L.init0 = init[0];
+                L.init1 = init[1];
+                T.t[D - kMinDigits][nt * 32 + lane] = L;
             }
+    return T;
+}
+
+__device__ const ResTables g_res_tables = make_res_tables();
+
+struct ResOperand {
+    const double *hi, *lo;
+    int64_t ld;
+    int row_contig;
+    int64_t rows, rows_pad;
+    const unsigned long long *max;
+    __half *R;
+    unsigned blocks;   // its blocks of the launch
+};
+
+struct ResShared {
+    ResLane tab[kResNT * 32];
+    // words (0, 2, 1, 3) of the warp's 64 integers, eight to a row of 36
+    // words: 16-byte stores and 8-byte reads without bank conflicts
+    uint32_t x[kResWarps][8 * 36];
+    double hi[64][17], lo[64][17];   // row-contiguous tiles, [l][row]
+};
+
+// Residues of the 64 entries (row, 64 c + lane) and (row, 64 c + 32 + lane)
+// from the lane's two X'; base: the address of plane 0's entry (row, 64 c + 8
+// g), ps: entries of a plane.
+__device__ __forceinline__ void residue_warp(const unsigned __int128 (&Xb)[2], __half *base,
+                                             int64_t ps, int N, const ResLane *tab,
+                                             uint32_t *xw) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const float2 magic{12582912.0f, 12582912.0f}, nmagic{-12582912.0f, -12582912.0f};
+    __syncwarp();   // the previous entries' words have been read
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int at = lane + 32 * u;
+        *reinterpret_cast<uint4 *>(xw + (at >> 3) * 36 + (at & 7) * 4) =
+            make_uint4((uint32_t)Xb[u], (uint32_t)(Xb[u] >> 64), (uint32_t)(Xb[u] >> 32),
+                       (uint32_t)(Xb[u] >> 96));
+    }
+    __syncwarp();
+    // A fragments of tile t: row g = entry 8g + 2t, row g + 8 = entry 8g + 2t + 1,
+    // each byte as the fp16 1024 + x
+    const uint32_t sel = (q & 1) ? 0x4342u : 0x4140u;
+    uint32_t A[4][4];
+    uint32_t low[4] = {0u, 0u, 0u, 0u};   // the lowest bytes of the entries, lane q = 0
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            // words q/2 and 2 + q/2 of the entry
+            const uint2 w = *reinterpret_cast<const uint2 *>(xw + g * 36 + (2 * t + h) * 4 +
+                                                             (q >> 1) * 2);
+            A[t][h] = __byte_perm(w.x, 0x64646464u, sel);
+            A[t][2 + h] = __byte_perm(w.y, 0x64646464u, sel);
+            low[t] |= (w.x & 0xFFu) << (16 * h);
         }
+    // plane 0 (p = 256): the lowest byte x of X, signed: with its top bit
+    // turned, fp16 1024 + (x ^ 128) less 1152
+    if (q == 0) {
+        uint32_t o[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const uint32_t b = (low[t] ^ 0x00800080u) | 0x64006400u;
+            const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&b),
+                                      __floats2half2_rn(1152.0f, 1152.0f));
+            o[t] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+        *reinterpret_cast<uint4 *>(base) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+    __half *dst = base + (1 + 2 * q) * ps;
+#pragma unroll
+    for (int nt = 0; nt < kResNT; ++nt, dst += 8 * ps) {
+        if (1 + 8 * nt >= N) break;
+        const ResLane &L = tab[nt * 32 + lane];
+        const float4 start = *reinterpret_cast<const float4 *>(&L.b0);
+        const float4 red = *reinterpret_cast<const float4 *>(L.inv);
+        const float2 iv{red.x, red.y}, np{red.z, red.w};
+        const float c0[4] = {start.z, start.w, start.z, start.w};
+        const uint2 bf = make_uint2(__float_as_uint(start.x), __float_as_uint(start.y));
+        uint32_t o0[4], o1[4];   // the lane's two moduli, entries 2t and 2t + 1
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            float acc[4];
+            mma_16816(acc, A[t], bf, c0);
+            float2 r[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 s2{acc[2 * h], acc[2 * h + 1]};
+                const float2 qn = __fadd2_rn(__ffma2_rn(s2, iv, magic), nmagic);
+                r[h] = __ffma2_rn(np, qn, s2);
+            }
+            const __half2 h0 = __floats2half2_rn(r[0].x, r[1].x);
+            const __half2 h1 = __floats2half2_rn(r[0].y, r[1].y);
+            o0[t] = *reinterpret_cast<const uint32_t *>(&h0);
+            o1[t] = *reinterpret_cast<const uint32_t *>(&h1);
+        }
+        if (1 + 8 * nt + 2 * q < N)
+            *reinterpret_cast<uint4 *>(dst) = make_uint4(o0[0], o0[1], o0[2], o0[3]);
+        if (2 + 8 * nt + 2 * q < N)
+            *reinterpret_cast<uint4 *>(dst + ps) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
     }
 }
 
-__global__ void __launch_bounds__(256) residue_kernel(
-    const double *__restrict__ Xh, const double *__restrict__ Xl, int64_t ld, int row_contig,
-    int64_t rows, int64_t k, int64_t rows_pad, int64_t k_pad,
-    const unsigned long long *__restrict__ rmax, __half *__restrict__ R, const SplitPlan plan) {
-    __shared__ ResLane tab[kResNT * 32];
+// X + 2^(8 DG - 1) of a dd entry at scale e.  The lo part of a normalised dd
+// at 112 bits is below 2^59: 64-bit arithmetic, whenever that holds.
+__device__ __forceinline__ unsigned __int128 biased_integer(double hi, double lo, int DG, int e) {
+    const int shift = 8 * DG - e;
+    const int E = (int)(((uint32_t)__double2hiint(lo) >> 20) & 0x7FF);
+    __int128 L;
+    if (E - 1075 + shift <= 9) {   // |lo 2^shift| < 2^62
+        const unsigned long long bits = (unsigned long long)__double_as_longlong(lo);
+        unsigned long long m =
+            (bits & ((1ull << 52) - 1)) | ((unsigned long long)(E ? 1 : 0) << 52);
+        const int sh = (E ? E : 1) - 1075 + shift;
+        if (sh < 0) {
+            const int rs = -sh < 60 ? -sh : 60;
+            m = (m + ((1ull << (rs - 1)) - 1) + ((m >> rs) & 1)) >> rs;
+        } else {
+            m <<= sh;
+        }
+        const long long v = (long long)m;
+        L = (bits >> 63) ? -v : v;
+    } else {
+        L = scaled_round(lo, shift);
+    }
+    return (unsigned __int128)(scaled_round(hi, shift) + L) +
+           ((unsigned __int128)1 << (8 * DG - 1));
+}
+
+__global__ void __launch_bounds__(kResThreads, kResBlocks) residue_kernel(
+    const ResOperand a, const ResOperand b, int64_t k, int64_t k_pad, const SplitPlan plan) {
+    __shared__ ResShared sh;
     const PlanPick pk = plan_choice(plan);
     if (pk.c < 0) return;
     const int N = pk.count, DG = pk.width / 8;
-    res_setup(N, DG, tab);
+    const bool first = blockIdx.x < a.blocks;
+    const double *Xh = first ? a.hi : b.hi, *Xl = first ? a.lo : b.lo;
+    const int64_t ld = first ? a.ld : b.ld, rows = first ? a.rows : b.rows;
+    const int64_t rows_pad = first ? a.rows_pad : b.rows_pad;
+    const int row_contig = first ? a.row_contig : b.row_contig;
+    const unsigned long long *rmax = first ? a.max : b.max;
+    __half *R = first ? a.R : b.R;
+    const unsigned bid = first ? blockIdx.x : blockIdx.x - a.blocks;
+    const unsigned nblk = first ? a.blocks : b.blocks;
+    for (int x = threadIdx.x; x < kResNT * 32; x += kResThreads)
+        sh.tab[x] = g_res_tables.t[DG - kMinDigits][x];
     __syncthreads();
-    switch (DG) {
-        case 14:
-            residue_warp<14>(Xh, Xl, ld, row_contig, rows, k, rows_pad, k_pad, rmax, R, N, tab);
-            break;
-        case 15:
-            residue_warp<15>(Xh, Xl, ld, row_contig, rows, k, rows_pad, k_pad, rmax, R, N, tab);
-            break;
-        default:
-            residue_warp<16>(Xh, Xl, ld, row_contig, rows, k, rows_pad, k_pad, rmax, R, N, tab);
-            break;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+    const int64_t ps = rows_pad * k_pad;
+    const int64_t cols = k_pad / 64;             // 64-entry chunks of a row
+    uint32_t *xw = sh.x[warp];
+    // items in order, chunk fastest: (row, chunk) per warp, or (16 rows,
+    // chunk) per block; the stride is kept as whole rows and a remainder
+    const int64_t stride = row_contig ? (int64_t)nblk : (int64_t)nblk * kResWarps;
+    const int64_t start = row_contig ? (int64_t)bid : (int64_t)bid * kResWarps + warp;
+    const int64_t end = row_contig ? rows_pad / 16 : rows_pad;
+    int64_t i = start / cols, c = start - i * cols;
+    const int64_t si = stride / cols, sc = stride - si * cols;
+    if (!row_contig) {
+        double hi[2], lo[2];
+        int e = 0;
+        auto fetch = [&](int64_t row, int64_t ch) {
+            const int64_t l = 64 * ch + lane;
+            const double *ph = Xh + l + row * ld, *pl = Xl + l + row * ld;
+            e = 0;
+            if (row < rows) e = scale_exponent(__ldg(rmax + row));
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const bool ok = row < rows && l + 32 * u < k;
+                hi[u] = ok ? __ldg(ph + 32 * u) : 0.0;
+                lo[u] = ok ? __ldg(pl + 32 * u) : 0.0;
+            }
+        };
+        if (i < end) fetch(i, c);
+        while (i < end) {
+            const unsigned __int128 Xb[2] = {biased_integer(hi[0], lo[0], DG, e),
+                                             biased_integer(hi[1], lo[1], DG, e)};
+            __half *base = R + i * k_pad + 64 * c + 8 * (lane >> 2);
+            i += si;
+            c += sc;
+            if (c >= cols) {
+                c -= cols;
+                ++i;
+            }
+            if (i < end) fetch(i, c);
+            residue_warp(Xb, base, ps, N, sh.tab, xw);
+        }
+        return;
+    }
+    double fh[4], fl[4];
+    const int tr = threadIdx.x % 16, tl = threadIdx.x / 16;
+    auto fetch = [&](int64_t rt, int64_t ch) {
+        const int64_t row = 16 * rt + tr;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t l = 64 * ch + tl + 16 * u;
+            const bool ok = row < rows && l < k;
+            fh[u] = ok ? __ldg(Xh + row + l * ld) : 0.0;
+            fl[u] = ok ? __ldg(Xl + row + l * ld) : 0.0;
+        }
+    };
+    if (i < end) fetch(i, c);
+    while (i < end) {
+        __syncthreads();   // the previous tile has been read
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            sh.hi[tl + 16 * u][tr] = fh[u];
+            sh.lo[tl + 16 * u][tr] = fl[u];
+        }
+        __syncthreads();
+        const int64_t ti = i, tc = c;
+        i += si;
+        c += sc;
+        if (c >= cols) {
+            c -= cols;
+            ++i;
+        }
+        if (i < end) fetch(i, c);
+#pragma unroll 1
+        for (int u = 0; u < 2; ++u) {
+            const int rr = warp + kResWarps * u;
+            const int64_t row = 16 * ti + rr;
+            const int e = row < rows ? scale_exponent(__ldg(rmax + row)) : 0;
+            const unsigned __int128 Xb[2] = {
+                biased_integer(sh.hi[lane][rr], sh.lo[lane][rr], DG, e),
+                biased_integer(sh.hi[lane + 32][rr], sh.lo[lane + 32][rr], DG, e)};
+            residue_warp(Xb, R + row * k_pad + 64 * tc + 8 * (lane >> 2), ps, N, sh.tab, xw);
+        }
     }
 }
 
@@ -789,45 +779,29 @@ CrtLayout crt_layout(int64_t m, int64_t n, int64_t k, bool sym = false) {
     return L;
 }
 
-template <int NP>
-void launch_residues_rows(const double *Xh, const double *Xl, int64_t ld, int rc, int64_t rows,
-                        int64_t k, int64_t rows_pad, int64_t k_pad,
-                        const unsigned long long *rmax, __half *R, const SplitPlan &plan,
-                        cudaStream_t st) {
-    dim3 grid((unsigned)ceil_div(rows_pad, 32), (unsigned)(k_pad / 16));
-    residue_rows_kernel<NP><<<grid, 128, 0, st>>>(Xh, Xl, ld, rc, rows, k, rows_pad, k_pad, rmax, R,
-                                             plan);
-}
-
-// Residues for up to Nmax moduli (the plan's widest candidate): one warp
-// per 32 entries, blocks resident at once, looping.
-int launch_residues(int Nmax, const double *Xh, const double *Xl, int64_t ld, int rc,
-                    int64_t rows, int64_t k, int64_t rows_pad, int64_t k_pad,
-                    const unsigned long long *rmax, __half *R, const SplitPlan &plan,
-                    cudaStream_t st) {
-    if (rc) {   // rows contiguous: the FP32 kernel (full-sector stores along k)
-        if (k_pad / 16 > 65535) return fail(MP_DD_ERR_TOO_LARGE, "k too large for residues");
-        switch (Nmax / 2) {
-#define MPDD_RES_CASE(NP)                                                                      \
-    case NP:                                                                                   \
-        launch_residues_rows<NP>(Xh, Xl, ld, rc, rows, k, rows_pad, k_pad, rmax, R, plan, st); \
-        break;
-            MPDD_RES_CASE(14) MPDD_RES_CASE(15) MPDD_RES_CASE(16) MPDD_RES_CASE(17)
-            MPDD_RES_CASE(18) MPDD_RES_CASE(19) MPDD_RES_CASE(20)
-#undef MPDD_RES_CASE
-            default:
-                return fail(MP_DD_ERR_TOO_LARGE, "residue count %d outside [28, 40]", Nmax);
-        }
-        return check_launch("residue_rows_kernel");
+// Residues of the call's operands (b == nullptr: one) in one launch of the
+// blocks resident at once, shared out by the operands' padded rows.
+int launch_residues(const SplitOperand &a, __half *ra, const SplitOperand *b, __half *rb, int64_t k,
+                    int64_t k_pad, const SplitPlan &plan, cudaStream_t st) {
+    ResOperand x{a.hi, a.lo, a.ld, a.row_contig, a.rows, a.rows_pad, a.max, ra, 0}, y{};
+    if (b) y = ResOperand{b->hi, b->lo, b->ld, b->row_contig, b->rows, b->rows_pad, b->max, rb, 0};
+    const int64_t slots = (int64_t)sm_count() * kResBlocks;
+    auto items = [&](const ResOperand &o) {   // block items
+        return o.row_contig ? o.rows_pad / 16 * (k_pad / 64)
+                            : ceil_div(o.rows_pad * (k_pad / 64), kResWarps);
+    };
+    const int64_t ia = items(x), ib = items(y), rows = x.rows_pad + y.rows_pad;
+    int64_t na = ia, nb = ib;
+    if (ia + ib > slots) {
+        na = slots * x.rows_pad / rows;
+        if (na < 1) na = 1;
+        if (na > ia) na = ia;
+        nb = slots - na < ib ? slots - na : ib;
+        if (b && nb < 1) nb = 1;
     }
-    if (Nmax < 2 || Nmax > kMaxMod)
-        return fail(MP_DD_ERR_TOO_LARGE, "residue count %d outside [2, %d]", Nmax, kMaxMod);
-    const int64_t warps = rows_pad * k_pad / 32;
-    int64_t blocks = ceil_div(warps, 8);
-    if (blocks > (int64_t)sm_count() * 8) blocks = (int64_t)sm_count() * 8;
-    if (blocks < 1) blocks = 1;
-    residue_kernel<<<(unsigned)blocks, 256, 0, st>>>(Xh, Xl, ld, rc, rows, k, rows_pad, k_pad,
-                                                     rmax, R, plan);
+    x.blocks = (unsigned)na;
+    y.blocks = (unsigned)nb;
+    residue_kernel<<<(unsigned)(na + nb), kResThreads, 0, st>>>(x, y, k, k_pad, plan);
     return check_launch("residue_kernel");
 }
 
@@ -936,14 +910,7 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     if ((rc = launch_certificate(p, w + L.off_ma, w + L.off_mb, L.m_pad, L.n_pad, L.k_pad, TN,
                                  rmax, cmax, hdr, st, tri_table)))
         return rc;
-    if ((rc = launch_residues(L.N, p.ah, p.al, p.lda, a_rc, p.m, p.k, L.m_pad, L.k_pad, rmax,
-                              RA, plan, st)))
-        return rc;
-    if (!sym) {   // (the Rsyrk form reuses the maxima and planes of op(A))
-        if ((rc = launch_residues(L.N, p.bh, p.bl, p.ldb, b_rc, p.n, p.k, L.n_pad, L.k_pad,
-                                  cmax, RB, plan, st)))
-            return rc;
-    }
+    if ((rc = launch_residues(oa, RA, sym ? nullptr : &ob, RB, p.k, L.k_pad, plan, st))) return rc;
 
     sliced_timing_mark(1, st);
     CUtensorMap tmA, tmB;
