@@ -190,6 +190,66 @@ BF_HD void to_dd(const BF &x, double &hi, double &lo) {
     lo = make_double(ml, x.e - 127 + (127 - lz) - 52, lsg);
 }
 
+// The nearest dd of Z 2^s for a two's complement Z of NW words (|Z| below
+// 2^(32 NW - 1)): the same result, bit for bit, as from_words and to_dd on
+// the magnitude.  The usual case (Z's leading bit in its upper two words, no
+// carry of the negation into the leading words, a remainder with its leading
+// bit among the first 32, exponents well inside the normal range) is written
+// out: the five leading words are taken as they are or one word lower, the
+// sign is an exclusive or, and both significands are assembled by adding the
+// exponent field to the rounded bits.  About 75 integer instructions; the
+// general path selects among all words and shifts by any count.
+template <int NW>
+BF_HD void signed_words_to_dd(const uint32_t (&S)[NW], int s, double &hi, double &lo) {
+    const uint32_t mask = (S[NW - 1] >> 31) ? 0xFFFFFFFFu : 0u;
+    const bool low = S[NW - 1] == mask;          // the top word is empty
+    uint32_t below = 0;                          // the words under the leading five
+#pragma unroll
+    for (int t = 0; t + 6 < NW; ++t) below |= S[t];
+    if (NW >= 6 && !low) below |= S[NW - 6];
+    const uint32_t w4 = (low ? S[NW - 2] : S[NW - 1]) ^ mask;
+    const uint32_t w3 = (low ? S[NW - 3] : S[NW - 2]) ^ mask;
+    const uint32_t w2 = (low ? S[NW - 4] : S[NW - 3]) ^ mask;
+    const uint32_t w1 = (low ? S[NW - 5] : S[NW - 4]) ^ mask;
+    const uint32_t w0 = (low ? S[NW - 6] : S[NW - 5]) ^ mask;
+    const int lz = clz32(w4);
+    const int e = 32 * (NW - 1) + 31 - (low ? 32 : 0) - lz + s;
+    const uint32_t m3 = fshl(w3, w4, lz), m2 = fshl(w2, w3, lz), m1 = fshl(w1, w2, lz),
+                   m0 = fshl(w0, w1, lz);
+    // hi: bits 127 .. 75, rounded by bit 74 and the rest
+    const uint32_t r2 = m2 & 0x7FFu;
+    const uint32_t ml = (m3 << 21) | (m2 >> 11);
+    const bool up = (r2 >> 10) && (((r2 & 0x3FFu) | m1 | m0) != 0 || (ml & 1u));
+    // lo: the remainder, or 2^75 minus it when rounded up
+    const uint64_t r10 = ((uint64_t)m1 << 32) | m0;
+    const uint64_t l10 = up ? 0 - r10 : r10;
+    const uint32_t l2 = up ? 0x800u - r2 - (r10 != 0) : r2;
+    const uint32_t l1 = (uint32_t)(l10 >> 32), l0 = (uint32_t)l10;
+    const uint32_t a2 = (l2 << 21) | (l1 >> 11), a1 = (l1 << 21) | (l0 >> 11), a0 = l0 << 21;
+    if (w4 == 0 || (mask != 0 && below == 0) || a2 == 0 || e < -900 || e > 1000) {
+        uint32_t z[NW];                          // the magnitude
+        uint32_t c = mask & 1u;
+#pragma unroll
+        for (int t = 0; t < NW; ++t) {
+            const uint64_t v = (uint64_t)(S[t] ^ mask) + c;
+            z[t] = (uint32_t)v;
+            c = (uint32_t)(v >> 32);
+        }
+        to_dd(from_words<NW>(z, mask & 1u, s), hi, lo);
+        return;
+    }
+    const uint64_t mh = ((uint64_t)(m3 >> 11) << 32) | ml;   // 2^52 <= mh < 2^53
+    hi = bitsd((((uint64_t)(uint32_t)(e + 1022) << 52) + mh + (up ? 1 : 0)) |
+               ((uint64_t)(mask & 1u) << 63));
+    const int lz2 = clz32(a2);
+    const uint32_t n2 = fshl(a1, a2, lz2), n1 = fshl(a0, a1, lz2), n0 = a0 << lz2;
+    const uint32_t nl = (n2 << 21) | (n1 >> 11);
+    const bool up2 = ((n1 >> 10) & 1u) && (((n1 & 0x3FFu) | n0) != 0 || (nl & 1u));
+    const uint64_t nh = ((uint64_t)(n2 >> 11) << 32) | nl;
+    lo = bitsd((((uint64_t)(uint32_t)(e - 53 - lz2 + 1022) << 52) + nh + (up2 ? 1 : 0)) |
+               ((uint64_t)((mask & 1u) ^ (up ? 1u : 0u)) << 63));
+}
+
 #undef BF_HD
 
 }  // namespace bigf

@@ -393,14 +393,15 @@ __global__ void __launch_bounds__(kResThreads, kResBlocks) residue_kernel(
 
 // Reconstruction constants of one moduli count N.
 struct CrtTables {
-    uint32_t P[kWords];                   // product of the moduli
     // Byte t of the CRT weights w_b = (P / p_b) ((P / p_b)^-1 mod p_b) of the
     // four moduli b = 4g .. 4g+3, packed in one word (zero past N): the dp4a
     // operand of digit t of the sums.
     uint32_t wp[kMaxMod / 4][4 * kWords];
-    // The same for qfix_b = RN(2^24 ((P / p_b)^-1 mod p_b) / p_b), w_b / P in
-    // fixed point (three bytes).
+    // Byte t of qfix_b = RN(2^24 ((P / p_b)^-1 mod p_b) / p_b), w_b / P in
+    // fixed point, of the moduli b = 4g .. 4g+3.
     uint32_t qp[kMaxMod / 4][3];
+    // 16-bit digits of 2^(32 kWords) - P, P the product of the moduli.
+    uint32_t negp[2 * kWords];
 };
 
 struct CrtArgs {
@@ -438,127 +439,59 @@ __device__ __forceinline__ dd axpby_dd(dd alpha, dd v, dd beta, dd c) {
     return r;
 }
 
-// The CRT sums of two adjacent entries (i, j), (i + 1, j) from the N
-// products reduced mod p_b: S = sum_b c_b w_b over NW 32-bit words and the
-// fixed-point quotient column Q = sum_b c_b qfix_b.  The residues of both
-// entries come in one 2-byte load per modulus and are packed four moduli to
-// a register, so each byte digit t of the sums is one dp4a per four moduli
-// (the digit sums stay below 40 255^2 < 2^22, exact in 32 bits) before the
-// digits are carried into words.  T is a reference into the kernel's
-// parameter block: the packed weights are constant-bank operands.
-constexpr int kCrtGroups = kMaxMod / 4;
-
-// The residues of entries (i, i + 1), i even (2-byte aligned): word h holds
-// moduli 2h and 2h + 1 as bytes e0b e1b e0b' e1b' (zero past N).
-__device__ __forceinline__ void crt_load_pair(const CrtArgs &p, int N, int64_t i, int64_t j,
-                                              uint32_t (&v)[kMaxMod / 2]) {
-    const uint8_t *res = p.res + j * p.m_pad + i;
-    const int64_t plane = p.n_pad * p.m_pad;
-#pragma unroll
-    for (int h = 0; h < kMaxMod / 2; ++h) {
-        const uint32_t lo = 2 * h < N
-            ? (uint32_t)__ldg(reinterpret_cast<const unsigned short *>(res + 2 * h * plane)) : 0u;
-        const uint32_t hi = 2 * h + 1 < N
-            ? (uint32_t)__ldg(reinterpret_cast<const unsigned short *>(res + (2 * h + 1) * plane))
-            : 0u;
-        v[h] = lo | (hi << 16);
-    }
-}
-
-template <int NW>
-__device__ __forceinline__ void crt_sums(const CrtTables &T, int N,
-                                         const uint32_t (&v)[kMaxMod / 2],
-                                         uint32_t (&S0)[NW], uint32_t (&S1)[NW], uint64_t &Q0,
-                                         uint64_t &Q1) {
-    constexpr int G = kCrtGroups;
-    uint32_t R0[G], R1[G];
+// The reconstructed integer of one entry from its N products reduced mod p_b
+// (four to a register): Z = sum_b c_b w_b - q P over NW 32-bit words in two's
+// complement.  q is the integer nearest to S / P = sum_b c_b (inv_b / p_b),
+// S = sum_b c_b w_b: |Z| < k 2^(2W-2) <= P / 4 puts S / P at least 1/4 from a
+// half-integer, while the fixed-point column (each qfix_b within 2^-25 of
+// inv_b / p_b, 16 bits of the sum kept) is within N 255 2^-25 + 2^-15 <
+// 0.0005 of it.  Then each byte digit of S is a column summed by one dp4a per
+// four moduli (below 40 255^2 < 2^22), two columns and q times the 16-bit
+// digit of -P make a half word (below 2^31), and one carry runs up the words.
+// T is a reference into the kernel's parameter block: its words are
+// constant-bank operands.  (16-bit columns with dp2a, half as many to carry,
+// were slower: the constant has to be dp2a's 16-bit operand, which the
+// instruction does not read from the constant bank.)
+//
+// What bounds the kernel: the ~17 FP64 operations of a general alpha / beta
+// epilogue (2.15 ms at 8192 x 8192), beside ~330 multiply-add-class integer
+// instructions at 64 lanes per clock and SM (1.1 ms) and as many issue slots
+// of others.  A separate subtraction of q P, a full negation and general
+// 128-bit shifts made ~1120 instructions per entry (747 now): at 8192 x 8192
+// 3.43 ms before and 2.42 now with general alpha and beta, 2.83 and 1.63 with
+// alpha = 1 and beta = 0.
+template <int NW, int G>
+__device__ __forceinline__ void crt_integer(const CrtTables &T, const uint32_t (&R)[G],
+                                            uint32_t (&Z)[NW]) {
+    uint32_t q0 = 0, q1 = 0, q2 = 0;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-        // v[2g] = e0b0 e1b0 e0b1 e1b1, v[2g + 1] = e0b2 e1b2 e0b3 e1b3
-        R0[g] = __byte_perm(v[2 * g], v[2 * g + 1], 0x6420);   // entry i: moduli 4g .. 4g+3
-        R1[g] = __byte_perm(v[2 * g], v[2 * g + 1], 0x7531);   // entry i + 1
+        q0 = __dp4a(R[g], T.qp[g][0], q0);
+        q1 = __dp4a(R[g], T.qp[g][1], q1);
+        q2 = __dp4a(R[g], T.qp[g][2], q2);
     }
-    const int groups = (N + 3) / 4;
-    uint64_t c0 = 0, c1 = 0;
+    const uint32_t q = ((q0 >> 8) + q1 + (q2 << 8) + (1u << 15)) >> 16;
+    uint32_t c = 0;
 #pragma unroll
-    for (int k = 0; k < NW; ++k) {
-        uint32_t d0[4] = {0u, 0u, 0u, 0u}, d1[4] = {0u, 0u, 0u, 0u};
+    for (int t = 0; t < NW; ++t) {
+        uint32_t d[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            if (g >= groups) break;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                d0[u] = __dp4a(R0[g], T.wp[g][4 * k + u], d0[u]);
-                d1[u] = __dp4a(R1[g], T.wp[g][4 * k + u], d1[u]);
-            }
+            for (int u = 0; u < 4; ++u) d[u] = __dp4a(R[g], T.wp[g][4 * t + u], d[u]);
         }
-        // word k: d[0] + d[1] 2^8 + d[2] 2^16 + d[3] 2^24 + the carry
-        const uint64_t v0 = c0 + (d0[0] + (d0[1] << 8)) + ((uint64_t)(d0[2] + (d0[3] << 8)) << 16);
-        const uint64_t v1 = c1 + (d1[0] + (d1[1] << 8)) + ((uint64_t)(d1[2] + (d1[3] << 8)) << 16);
-        S0[k] = (uint32_t)v0;
-        S1[k] = (uint32_t)v1;
-        c0 = v0 >> 32;
-        c1 = v1 >> 32;
+        const uint32_t x = q * T.negp[2 * t] + (d[1] * 256u + d[0]);
+        const uint32_t y = q * T.negp[2 * t + 1] + (d[3] * 256u + d[2]);
+        // word t: x + 2^16 y + the carry (below 2^31 + 2^16 + 2^47)
+        const uint64_t v = (uint64_t)y * 65536u + (x + c);
+        Z[t] = (uint32_t)v;
+        c = (uint32_t)(v >> 32);
     }
-    uint32_t q0[3] = {0u, 0u, 0u}, q1[3] = {0u, 0u, 0u};
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        if (g >= groups) break;
-#pragma unroll
-        for (int u = 0; u < 3; ++u) {
-            q0[u] = __dp4a(R0[g], T.qp[g][u], q0[u]);
-            q1[u] = __dp4a(R1[g], T.qp[g][u], q1[u]);
-        }
-    }
-    Q0 = q0[0] + ((uint64_t)q0[1] << 8) + ((uint64_t)q0[2] << 16);
-    Q1 = q1[0] + ((uint64_t)q1[1] << 8) + ((uint64_t)q1[2] << 16);
 }
 
-// One output entry from its sums: the symmetric representative of S mod P,
-// then the alpha/beta epilogue rounded once to dd.
-// NW: 32-bit words of the sums (P < 2^(32 (NW - 1)), and the sum of N
-// residues < 256 times the weights < P stays below 2^(32 NW)).
-// ch, cl: C(i, j) when the epilogue reads it; rbits, cbits: the row and
-// column maxima of op(A) and op(B) (loaded ahead by the caller).
-template <int NW>
-__device__ __forceinline__ void crt_entry(const CrtArgs &p, const CrtTables &T, int W,
-                                          uint32_t (&S)[NW], uint64_t Q, int64_t i, int64_t j,
-                                          double ch, double cl, unsigned long long rbits,
-                                          unsigned long long cbits) {
-    // The symmetric representative is Z = S - q P with q the integer
-    // nearest to S / P = sum_b c_b (inv_b / p_b): |Z| < k 2^(2W-2) <= P / 4,
-    // and Q 2^-24 is within N 255 2^-25 < 0.0004 of S / P (each qfix_b
-    // within 2^-25 of inv_b / p_b), so rounding it gives q.
-    const uint64_t q = (Q + (1ull << 23)) >> 24;
-    // Z = S - q P in two's complement over NW words (exact: |Z| < 2^(32 NW - 1))
-    {
-        uint64_t mc = 0, borrow = 0;
-#pragma unroll
-        for (int t = 0; t < NW; ++t) {
-            const uint64_t prod = q * T.P[t] + mc;
-            mc = prod >> 32;
-            const uint64_t d = (uint64_t)S[t] - (uint32_t)prod - borrow;
-            S[t] = (uint32_t)d;
-            borrow = (d >> 63) & 1;
-        }
-    }
-    // magnitude and sign
-    const bool negative = (S[NW - 1] & 0x80000000u) != 0;
-    if (negative) {
-        uint64_t c2 = 1;
-#pragma unroll
-        for (int t = 0; t < NW; ++t) {
-            const uint64_t v = (uint64_t)(uint32_t)~S[t] + c2;
-            S[t] = (uint32_t)v;
-            c2 = v >> 32;
-        }
-    }
-    const int sc = scale_exponent(rbits) + scale_exponent(cbits) - 2 * W;
-    // v = Z 2^sc rounded once to dd by integer operations (no FP64), then
-    // the alpha / beta epilogue in dd arithmetic
-    dd v;
-    bigf::to_dd(bigf::from_words<NW>(S, negative ? 1u : 0u, sc), v.hi, v.lo);
-    const int64_t off = i + j * p.ldc;
+// The alpha / beta epilogue of one entry: v its product, (ch, cl) the old C
+// where the epilogue reads it.
+__device__ __forceinline__ void crt_store(const CrtArgs &p, dd v, int64_t off, double ch, double cl) {
     dd r;
     switch (p.ab_mode) {
         case 1:   // alpha = +-1, beta = 0: the product itself
@@ -578,74 +511,111 @@ __device__ __forceinline__ void crt_entry(const CrtArgs &p, const CrtTables &T, 
 }
 
 // Entry pairs (i, i + 1) of column j, i even (m_pad is even, so the pair's
-// residues exist even when i + 1 = m).  (Requesting the next pair's loads
-// ahead measured slower: the extra registers cost more occupancy than the
-// overlap gains.)
-template <int NW>
+// residues exist even when i + 1 = m): one 2-byte load per modulus brings both
+// entries' residues, packed four moduli to a register.  (Requesting the next
+// pair's loads ahead measured slower: the extra registers cost more occupancy
+// than the overlap gains.)
+// G: groups of four moduli, 4 (G - 1) < N <= 4 G or the weights past N zero.
+template <int NW, int G>
 __device__ __forceinline__ void crt_pair(const CrtArgs &p, const CrtTables &T, int N, int W,
                                          int64_t i, int64_t j) {
     const bool in0 = !((p.tri == 1 && i > j) || (p.tri == 2 && i < j));
     const bool in1 = i + 1 < p.m && !((p.tri == 1 && i + 1 > j) || (p.tri == 2 && i + 1 < j));
     if (!in0 && !in1) return;
-    uint32_t v[kMaxMod / 2];
-    crt_load_pair(p, N, i, j, v);
-    uint32_t S0[NW], S1[NW];
-    uint64_t Q0, Q1;
-    crt_sums<NW>(T, N, v, S0, S1, Q0, Q1);
+    uint32_t R0[G], R1[G];
+    {
+        const int64_t at = j * p.m_pad + i, plane = p.n_pad * p.m_pad;
+        uint32_t v[2 * G];
+#pragma unroll
+        for (int h = 0; h < 2 * G; ++h) {   // N is even: moduli 2h and 2h + 1
+            v[h] = 0;
+            if (h < 2 * (G - 1) || 2 * h < N) {
+                const uint8_t *res = p.res + (int64_t)(2 * h) * plane + at;
+                const uint32_t lo = __ldg(reinterpret_cast<const unsigned short *>(res));
+                const uint32_t hi = __ldg(reinterpret_cast<const unsigned short *>(res + plane));
+                v[h] = lo | (hi << 16);
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            R0[g] = __byte_perm(v[2 * g], v[2 * g + 1], 0x6420);   // entry i: moduli 4g .. 4g+3
+            R1[g] = __byte_perm(v[2 * g], v[2 * g + 1], 0x7531);   // entry i + 1
+        }
+    }
     const bool use_c = p.ab_mode == 2 || (p.ab_mode == 0 && !p.beta_zero);
-    const unsigned long long cb = __ldg(p.cmax + j);
+    const int64_t off = i + j * p.ldc;
+    const int ec = scale_exponent(__ldg(p.cmax + j)) - 2 * W;
+    double c0h = 0.0, c0l = 0.0, c1h = 0.0, c1l = 0.0;
+    if (use_c && in0) {
+        c0h = p.ch[off];
+        c0l = p.cl[off];
+    }
+    if (use_c && in1) {
+        c1h = p.ch[off + 1];
+        c1l = p.cl[off + 1];
+    }
     if (in0) {
-        const int64_t off = i + j * p.ldc;
-        crt_entry<NW>(p, T, W, S0, Q0, i, j, use_c ? p.ch[off] : 0.0, use_c ? p.cl[off] : 0.0,
-                      __ldg(p.rmax + i), cb);
+        uint32_t Z[NW];
+        crt_integer<NW, G>(T, R0, Z);
+        dd v;
+        bigf::signed_words_to_dd<NW>(Z, scale_exponent(__ldg(p.rmax + i)) + ec, v.hi, v.lo);
+        crt_store(p, v, off, c0h, c0l);
     }
     if (in1) {
-        const int64_t off = i + 1 + j * p.ldc;
-        crt_entry<NW>(p, T, W, S1, Q1, i + 1, j, use_c ? p.ch[off] : 0.0,
-                      use_c ? p.cl[off] : 0.0, __ldg(p.rmax + i + 1), cb);
+        uint32_t Z[NW];
+        crt_integer<NW, G>(T, R1, Z);
+        dd v;
+        bigf::signed_words_to_dd<NW>(Z, scale_exponent(__ldg(p.rmax + i + 1)) + ec, v.hi, v.lo);
+        crt_store(p, v, off + 1, c1h, c1l);
     }
 }
 
-template <int NW>
+template <int NW, int G>
 __device__ __forceinline__ void crt_loop(const CrtArgs &p, const CrtTables &T, int N, int W) {
+    // pair index = j * mh + ih, kept as (ih, j); the stride likewise
     const int64_t mh = (p.m + 1) / 2;
-    const int64_t total = mh * p.n;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (total <= 0xFFFFFFFFll) {   // 32-bit index arithmetic
-        const uint32_t m32 = (uint32_t)mh;
-        for (; idx < total; idx += stride) {
-            const uint32_t u = (uint32_t)idx, jj = u / m32, ih = u - jj * m32;
-            crt_pair<NW>(p, T, N, W, 2 * (int64_t)ih, jj);
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int64_t j = idx / mh, ih = idx - j * mh;
+    const int64_t sj = stride / mh, si = stride - sj * mh;
+    while (j < p.n) {
+        crt_pair<NW, G>(p, T, N, W, 2 * ih, j);
+        ih += si;
+        j += sj;
+        if (ih >= mh) {
+            ih -= mh;
+            ++j;
         }
-        return;
     }
-    for (; idx < total; idx += stride) crt_pair<NW>(p, T, N, W, 2 * (idx % mh), idx / mh);
 }
 
-// NW0..NW2: words of the sums for the three candidate widths.
-template <int NW0, int NW1, int NW2>
-__global__ void __launch_bounds__(256) crt_kernel(const __grid_constant__ CrtArgs p) {
+// Words and groups of four moduli of the three candidate widths for every k
+// the form takes: at 112 bits 8 words and N = 30 or 32 up to k = 32768, 9 words
+// and N = 34 beyond; at 120 bits 9 words and N = 34 or 36; at 128 bits 9 or 10
+// words and N = 36 or 38 (more words or groups than needed give the same
+// result: their weights are zero).  They are compile-time constants: with a
+// test of the count in every word's loop a quarter of the instructions were
+// tests and branches.
+template <int NW0, int G0>
+__global__ void __launch_bounds__(256, 4) crt_kernel(const __grid_constant__ CrtArgs p) {
     if (p.info != nullptr && *p.info != 0) return;   // an earlier step failed
     const PlanPick pk = plan_choice(p.plan);
     if (pk.c < 0) return;                            // the plain kernel computes C
-    if (pk.c == 0) crt_loop<NW0>(p, p.tab[0], pk.count, pk.width);
-    else if (pk.c == 1) crt_loop<NW1>(p, p.tab[1], pk.count, pk.width);
-    else crt_loop<NW2>(p, p.tab[2], pk.count, pk.width);
+    if (pk.c == 0) crt_loop<NW0, G0>(p, p.tab[0], pk.count, pk.width);
+    else if (pk.c == 1) crt_loop<9, 9>(p, p.tab[1], pk.count, pk.width);
+    else crt_loop<10, 10>(p, p.tab[2], pk.count, pk.width);
 }
 
 // ------------------------------------------------------------------ host
 
-// 256-thread blocks of the three crt_kernel instantiations resident per SM
+// 256-thread blocks of the two crt_kernel instantiations resident per SM
 // (occupancy query, once per instantiation; 1 if the query fails).
 int crt_resident_blocks(int which) {
-    static int cached[3] = {0, 0, 0};
-    static std::once_flag once[3];
+    static int cached[2] = {0, 0};
+    static std::once_flag once[2];
     std::call_once(once[which], [which] {
         int b = 0;
-        const void *f = which == 0 ? (const void *)crt_kernel<8, 9, 10>
-                        : which == 1 ? (const void *)crt_kernel<9, 9, 10>
-                                     : (const void *)crt_kernel<9, 10, 10>;
+        const void *f = which == 0 ? (const void *)crt_kernel<8, 8> : (const void *)crt_kernel<9, 9>;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, 256, 0) != cudaSuccess) {
             cudaGetLastError();
             b = 0;
@@ -811,7 +781,15 @@ int crt_tables(int N, CrtTables &T, int *nwords) {
     Big P{1};
     for (int i = 0; i < N; ++i) P = big_mul_small(P, modulus(i));
     if ((int)P.size() > kWords - 1) return fail(MP_DD_ERR_TOO_LARGE, "moduli product too wide");
-    for (int t = 0; t < kWords; ++t) T.P[t] = t < (int)P.size() ? P[t] : 0;
+    {   // 2^(32 kWords) - P
+        uint64_t borrow = 0;
+        for (int t = 0; t < kWords; ++t) {
+            const uint64_t d = 0 - (uint64_t)(t < (int)P.size() ? P[t] : 0u) - borrow;
+            T.negp[2 * t] = (uint32_t)d & 0xFFFFu;
+            T.negp[2 * t + 1] = ((uint32_t)d >> 16) & 0xFFFFu;
+            borrow = (d >> 63) & 1;
+        }
+    }
     for (int i = 0; i < N; ++i) {
         uint32_t mi_mod = 0;
         Big Mi = big_div_small(P, modulus(i), nullptr);
@@ -955,29 +933,26 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     int nw[kMaxCand] = {0, 0, 0};
     for (int c = 0; c < ncand; ++c)
         if ((rc = crt_tables(counts[c], ca.tab[c], &nw[c]))) return rc;
-    for (int c = ncand; c < kMaxCand; ++c) nw[c] = nw[ncand - 1];   // (never chosen)
-    // the word counts that occur for k < 2^17: 8 at 112 bits (9 for the
-    // largest k), 9 at 120 bits, 9 or 10 at 128 bits; a kernel with more
-    // words than needed gives the same result (the weights are zero-padded)
-    if (nw[0] > 9 || nw[1] > 10 || nw[2] > 10)
-        return fail(MP_DD_ERR_TOO_LARGE, "CRT word counts %d/%d/%d beyond the kernel's", nw[0],
-                    nw[1], nw[2]);
+    const int which = nw[0] <= 8 && counts[0] <= 32 ? 0 : 1;
+    const int words[kMaxCand] = {which == 0 ? 8 : 9, 9, 10};
+    for (int c = 0; c < ncand; ++c)   // (see crt_kernel)
+        if (nw[c] > words[c] || counts[c] > 4 * words[c] || counts[c] < 4 * words[c] - 4)
+            return fail(MP_DD_ERR_TOO_LARGE, "CRT words %d / moduli %d beyond the kernel's", nw[c],
+                        counts[c]);
     // one thread per entry pair, looping.  Full products: as many blocks as
-    // are resident at once (three per SM at 80 registers; eight per SM left
+    // are resident at once (four per SM; eight per SM left
     // the last two-thirds wave with a third of the slots idle: 3.65-3.68
     // against 3.70-3.73 ms at 8192).  Triangles: eight per SM, which the
     // block scheduler balances over the uneven work of the skipped entries
     // (resident blocks only: 2.61 against 2.41-2.45 ms).
     const int64_t pairs = ceil_div(p.m, 2) * p.n;
-    const int which = nw[0] <= 8 && nw[1] <= 9 ? 0 : (nw[1] <= 9 ? 1 : 2);
     int64_t blocks = ceil_div(pairs, 256);
     const int64_t cap = (int64_t)sm_count() * (p.tri ? 8 : crt_resident_blocks(which));
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     const unsigned nb = (unsigned)blocks;
-    if (which == 0) crt_kernel<8, 9, 10><<<nb, 256, 0, st>>>(ca);
-    else if (which == 1) crt_kernel<9, 9, 10><<<nb, 256, 0, st>>>(ca);
-    else crt_kernel<9, 10, 10><<<nb, 256, 0, st>>>(ca);
+    if (which == 0) crt_kernel<8, 8><<<nb, 256, 0, st>>>(ca);
+    else crt_kernel<9, 9><<<nb, 256, 0, st>>>(ca);
     if ((rc = check_launch("crt_kernel"))) return rc;
     rc = launch_plain_fallback(p, plan, st);
     sliced_timing_mark(3, st);

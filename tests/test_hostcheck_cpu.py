@@ -88,3 +88,33 @@ def test_words_to_dd_rounding(tmp_path):
         assert err <= abs(x) * (Fraction(2) ** -106 + Fraction(2) ** -126) + Fraction(2) ** -1074
         if Z.bit_length() <= 128 and abs(x) > Fraction(2) ** -900:
             assert out[0] == float(x)
+
+
+def test_signed_words_to_dd_is_the_general_rounding(tmp_path):
+    """The reconstruction kernel's rounding of a two's complement Z equals
+    from_words and to_dd on its magnitude bit for bit: leading bits in every
+    word, zero and all-one words below, exponents past the normal range."""
+    so = str(tmp_path / "words_dd.so")
+    _build(os.path.join(HERE, "hostcheck", "words_dd.cu"), so, shared=True)
+    lib = ctypes.CDLL(so)
+    U8 = ctypes.c_uint32 * 8
+    D2 = ctypes.c_double * 2
+    for f in (lib.words_to_dd, lib.signed_words_to_dd):
+        f.argtypes = [U8, ctypes.c_uint32, ctypes.c_int, D2]
+    g = random.Random(12)
+    fill = [0, 0xFFFFFFFF, 0x80000000, 1, 0x7FF, 0x400, 0x800]
+    for it in range(60000):
+        nbits = g.choice([0, 1, 53, 54, 96, 107, 127, 128, 160, 192, 193, 223, 224, 225, 230, 240, 254, 255])
+        z = [g.choice(fill) if g.random() < 0.3 else g.getrandbits(32) for _ in range(8)]
+        Z = sum(w << (32 * t) for t, w in enumerate(z)) & ((1 << nbits) - 1)
+        if nbits:
+            Z |= 1 << (nbits - 1)
+        if g.random() < 0.2:
+            Z = (Z >> (nbits // 2)) << (nbits // 2)
+        s = g.choice([g.randint(-300, 50), g.randint(-1300, -1000), g.randint(700, 1100)])
+        neg = int(Z != 0 and g.random() < 0.5)
+        words = U8(*[(Z >> (32 * t)) & 0xFFFFFFFF for t in range(8)])
+        a, b = D2(), D2()
+        lib.words_to_dd(words, neg, s, a)
+        lib.signed_words_to_dd(words, neg, s, b)
+        assert bytes(a) == bytes(b), (hex(Z), neg, s, list(a), list(b))
