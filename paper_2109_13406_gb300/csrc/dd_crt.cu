@@ -417,6 +417,7 @@ struct CrtArgs {
     double *ch, *cl;
     int64_t ldc;
     int tri;                              // 0: all of C; 1 / 2: upper / lower triangle
+    int single;                           // one entry per thread, no loop
     const int64_t *info;                  // optional: non-zero -> leave C as is
 };
 
@@ -570,12 +571,50 @@ __device__ __forceinline__ void crt_pair(const CrtArgs &p, const CrtTables &T, i
     }
 }
 
+// One entry (i, j): the pair's 2-byte loads (shared with the neighbouring
+// lane), the entry's bytes picked out of them.
+template <int NW, int G>
+__device__ __forceinline__ void crt_one(const CrtArgs &p, const CrtTables &T, int N, int W,
+                                        int64_t i, int64_t j) {
+    if ((p.tri == 1 && i > j) || (p.tri == 2 && i < j)) return;
+    uint32_t R[G];
+    const int64_t at = j * p.m_pad + (i & ~(int64_t)1), plane = p.n_pad * p.m_pad;
+    const uint32_t sel = (i & 1) ? 0x7531u : 0x6420u;
+    uint32_t v[2 * G];
+#pragma unroll
+    for (int h = 0; h < 2 * G; ++h) {
+        v[h] = 0;
+        if (h < 2 * (G - 1) || 2 * h < N) {
+            const uint8_t *res = p.res + (int64_t)(2 * h) * plane + at;
+            const uint32_t lo = __ldg(reinterpret_cast<const unsigned short *>(res));
+            const uint32_t hi = __ldg(reinterpret_cast<const unsigned short *>(res + plane));
+            v[h] = lo | (hi << 16);
+        }
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) R[g] = __byte_perm(v[2 * g], v[2 * g + 1], sel);
+    const bool use_c = p.ab_mode == 2 || (p.ab_mode == 0 && !p.beta_zero);
+    const int64_t off = i + j * p.ldc;
+    const double ch = use_c ? p.ch[off] : 0.0, cl = use_c ? p.cl[off] : 0.0;
+    const int sc = scale_exponent(__ldg(p.rmax + i)) + scale_exponent(__ldg(p.cmax + j)) - 2 * W;
+    uint32_t Z[NW];
+    crt_integer<NW, G>(T, R, Z);
+    dd v2;
+    bigf::signed_words_to_dd<NW>(Z, sc, v2.hi, v2.lo);
+    crt_store(p, v2, off, ch, cl);
+}
+
 template <int NW, int G>
 __device__ __forceinline__ void crt_loop(const CrtArgs &p, const CrtTables &T, int N, int W) {
-    // pair index = j * mh + ih, kept as (ih, j); the stride likewise
-    const int64_t mh = (p.m + 1) / 2;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p.single) {   // the grid has a thread for every entry
+        const int64_t j = idx / p.m;
+        if (j < p.n) crt_one<NW, G>(p, T, N, W, idx - j * p.m, j);
+        return;
+    }
+    // pair index = j * mh + ih, kept as (ih, j); the stride likewise
+    const int64_t mh = (p.m + 1) / 2;
     int64_t j = idx / mh, ih = idx - j * mh;
     const int64_t sj = stride / mh, si = stride - sj * mh;
     while (j < p.n) {
@@ -948,7 +987,12 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     const int64_t pairs = ceil_div(p.m, 2) * p.n;
     int64_t blocks = ceil_div(pairs, 256);
     const int64_t cap = (int64_t)sm_count() * (p.tri ? 8 : crt_resident_blocks(which));
-    if (blocks > cap) blocks = cap;
+    // few entries: one per thread halves the latency of a thread's chain (64 x
+    // 2048: 17.3 us in pairs, 15.4 so; 512 x 512, already two blocks per SM
+    // and more: 21.4 either way)
+    ca.single = p.m * p.n <= 2 * 256 * (int64_t)sm_count() * crt_resident_blocks(which);
+    if (ca.single) blocks = ceil_div(p.m * p.n, 256);
+    else if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     const unsigned nb = (unsigned)blocks;
     if (which == 0) crt_kernel<8, 8><<<nb, 256, 0, st>>>(ca);

@@ -526,6 +526,32 @@ struct Margin {
     }
 };
 
+// 16 accumulator columns of one exact fp32 run (integers of magnitude at most
+// 2^24) reduced to [0, p) and stored as bytes, one column every m_pad bytes:
+// x - p rint(x / p), the quotient within 2^-6 of x / p, so the remainder is
+// above -p and below p; p is added to a negative one, and the byte read off
+// the low bits of 2^23 plus it.  Two columns per packed instruction, ~4 a
+// column; the int32 path's conversion (at 16 lanes per clock) and division
+// with an unknown divisor took ~30, which made the products of small k
+// wait for this epilogue (band phase of a 2048 x 2048 Rsyrk with k = 256: 108 us
+// before, 75 now; 512^3: 27 and 23; 64 x 2048 x 192: 20.5 and 16.4).
+__device__ __forceinline__ void store_residues(const uint32_t (&r)[16], float pm, float iv,
+                                               uint8_t *dst, int64_t m_pad) {
+    const float2 iv2{iv, iv}, np2{-pm, -pm}, magic{12582912.0f, 12582912.0f},
+        nmagic{-12582912.0f, -12582912.0f};
+#pragma unroll
+    for (int j = 0; j < 16; j += 2) {
+        const float2 x{__uint_as_float(r[j]), __uint_as_float(r[j + 1])};
+        const float2 qn = __fadd2_rn(__ffma2_rn(x, iv2, magic), nmagic);
+        float2 c = __ffma2_rn(np2, qn, x);
+        c.x += c.x < 0.0f ? pm : 0.0f;
+        c.y += c.y < 0.0f ? pm : 0.0f;
+        const float2 o = __fadd2_rn(c, float2{8388608.0f, 8388608.0f});
+        dst[(int64_t)j * m_pad] = (uint8_t)__float_as_uint(o.x);
+        dst[(int64_t)(j + 1) * m_pad] = (uint8_t)__float_as_uint(o.y);
+    }
+}
+
 // MAG: the certificate's magnitude product (bf16 operands, fp32 sums, the
 // margin d_ij of every entry reduced to its minimum); otherwise the integer
 // band products with the band count taken from the call's plan.
@@ -747,6 +773,16 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
         const int col0 = ((warp - 2) / 4) * EC;       // first accumulator column
         const int row = q * 32 + lane;          // row of the tile this thread owns
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+        // this warp has read accumulator `buf`
+        auto release = [&](uint32_t buf) {
+            tc_fence_before();
+            if (PAIR) {   // one arrival per warp on the leader's barrier
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(cluster_map(&acce[buf], 0));
+            } else {
+                mbar_arrive(&acce[buf]);
+            }
+        };
         uint32_t chunk = 0;
         bool ok = true;
         for (int item = item0; item < num_items && ok; item += item_step) {
@@ -777,11 +813,35 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
                     mg.finish(p);
                     continue;
                 }
+                const int steps = (p.diag ? 1 : b + 1) * KB;
+                const int nchunks = (steps + chunk_kb<MAG>() - 1) / chunk_kb<MAG>();
+                if (p.diag && nchunks == 1) {
+                    // one exact run (k <= 1024): reduced mod p as it is read
+                    const uint32_t buf = chunk & 1, use = chunk >> 1;
+                    ++chunk;
+                    const float pm = (float)p.moduli[b];
+                    const float iv = __frcp_rn(pm);
+                    uint8_t *dst = p.R + ((int64_t)b * p.n_pad + (int64_t)tn * TN + col0) * p.m_pad +
+                                   (int64_t)tm * TM + row;
+                    if (!mbar_wait(&accf[buf], use & 1, abort_flag)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+#pragma unroll
+                    for (int cc = 0; cc < EC / 16; ++cc) {
+                        uint32_t r[16];
+                        tmem_ld_32x32b_x16(tmem + lane_base + buf * TN + col0 + cc * 16, r);
+                        tmem_ld_wait();
+                        if (cc + 1 == EC / 16) release(buf);
+                        store_residues(r, pm, iv, dst, p.m_pad);
+                        dst += 16 * p.m_pad;
+                    }
+                    continue;
+                }
                 int32_t acc[EC];
 #pragma unroll
                 for (int j = 0; j < EC; ++j) acc[j] = 0;
-                const int steps = (p.diag ? 1 : b + 1) * KB;
-                const int nchunks = (steps + chunk_kb<MAG>() - 1) / chunk_kb<MAG>();
                 for (int c = 0; c < nchunks; ++c, ++chunk) {
                     const uint32_t buf = chunk & 1, use = chunk >> 1;
                     if (!mbar_wait(&accf[buf], use & 1, abort_flag)) {
@@ -798,24 +858,25 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
                         for (int j = 0; j < 16; ++j)
                             acc[cc * 16 + j] += __float2int_rn(__uint_as_float(r[j]));
                     }
-                    tc_fence_before();
-                    if (PAIR) {   // one arrival per warp on the leader's barrier
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_cluster(cluster_map(&acce[buf], 0));
-                    } else {
-                        mbar_arrive(&acce[buf]);
-                    }
+                    release(buf);
                 }
                 if (!ok) break;
                 const int64_t off = ((int64_t)b * p.n_pad + (int64_t)tn * TN + col0) * p.m_pad +
                                     (int64_t)tm * TM + row;
                 if (p.diag) {
-                    const int pm = p.moduli[b];
+                    // acc mod p: u = acc + (a multiple of p from 2^31 on) is
+                    // in [0, 2^32), and floor(u ceil(2^32 / p) / 2^32) is
+                    // floor(u / p) or one more
+                    const uint32_t pm = (uint32_t)p.moduli[b];
+                    const uint32_t mul = 0xFFFFFFFFu / pm + 1u;
+                    const uint32_t bias = (0x80000000u / pm + 1u) * pm;
                     uint8_t *dst = p.R + off;
 #pragma unroll
                     for (int j = 0; j < EC; ++j) {
-                        int r = acc[j] % pm;
-                        dst[(int64_t)j * p.m_pad] = (uint8_t)(r < 0 ? r + pm : r);
+                        const uint32_t u = (uint32_t)acc[j] + bias;
+                        uint32_t r = u - __umulhi(u, mul) * pm;
+                        if ((int32_t)r < 0) r += pm;
+                        dst[(int64_t)j * p.m_pad] = (uint8_t)r;
                     }
                 } else {
                     int32_t *dst = p.P + off;

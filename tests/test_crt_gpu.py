@@ -268,3 +268,55 @@ def test_crt_non_finite_c_entries(cuda_lib):
     rows, cols = np.nonzero(keep)
     clean = datagen.gemm_case(748, "N", "N", m, n, k)
     assert check_against_exact(clean, got, rows, cols) <= 1.0
+
+
+@pytest.mark.parametrize("k", [64, 1024, 1025])
+def test_crt_products_on_either_side_of_one_run(cuda_lib, k):
+    """Up to k = 1024 the products are reduced mod p from one exact fp32 run,
+    beyond it from int32 sums.  Half the rows hold the entries whose products
+    mod 256 are all 2^14, so the runs end at +-2^24 and 2^14 k; the planes are
+    bit-exact against the oracle, over several tiles with ragged edges."""
+    mp = cuda_lib
+    m, n = 140, 270
+    c = datagen.gemm_case(750 + k, "N", "N", m, n, k)
+    g = datagen.rng(751)
+    for M, ax in ((c.A, 0), (c.B, 1)):
+        sgn = np.where(g.random(M[0].shape) < 0.02, -1.0, 1.0)
+        pick = np.arange(M[0].shape[ax]) % 2 == 0
+        sel = np.broadcast_to(pick[:, None] if ax == 0 else pick[None, :], M[0].shape)
+        M[0][sel] = 0.5 * sgn[sel]
+        M[1][sel] = 2.0 ** -104 * sgn[sel]
+    got, ws = run_crt(mp, c)
+    rep = mp.mp_dd_split_report(ws)
+    assert rep["width_bits"] == 112
+    L = mp.mp_dd_crt_layout(m, n, k)
+    mods = L["moduli"][:rep["count"]]
+    RA, _ = oz.residue_planes(*oz.op_rows(c.A, False, m, k), mods, 14)
+    RB, _ = oz.residue_planes(*oz.op_cols(c.B, False, k, n), mods, 14)
+    assert (RA[0][::2] == -128).all() and (RB[0][::2] == -128).all()
+    N, mp_, np_ = len(mods), L["m_pad"], L["n_pad"]
+    prods = view(ws, L["products"], N * np_ * mp_, np.uint8).reshape(N, np_, mp_)
+    want = oz.crt_products(RA, RB, mods)
+    assert np.array_equal(prods[:, :n, :m].transpose(0, 2, 1).astype(np.int64), want)
+    assert check_against_exact(c, got) <= 1.0
+
+
+@pytest.mark.parametrize("sub", [(401, 303), (64, 1203), (1, 1), (1801, 2)])
+def test_crt_entry_and_pair_threads_agree(cuda_lib, sub):
+    """A product whose reconstruction runs two entries per thread equals, on
+    its leading block, the product of that block alone, which runs one entry
+    per thread (both exact integer products, rounded once)."""
+    m, n, k = 1801, 1203, 70
+    c = datagen.gemm_case(760, "T", "N", m, n, k)
+    whole, ws = run_crt(cuda_lib, c)
+    assert cuda_lib.mp_dd_split_report(ws)["width_bits"] == 112
+    sm, sn = sub
+    part = datagen.GemmCase("T", "N", sm, sn, k, c.alpha, tuple(x[:, :sm] for x in c.A),
+                            tuple(x[:, :sn] for x in c.B), c.beta, tuple(x[:, :sn] for x in c.C))
+    part = datagen.GemmCase("T", "N", sm, sn, k, c.alpha, *(
+        (tuple(np.asfortranarray(x) for x in part.A), tuple(np.asfortranarray(x) for x in part.B),
+         c.beta, tuple(np.asfortranarray(x) for x in part.C))))
+    got, ws = run_crt(cuda_lib, part)
+    assert cuda_lib.mp_dd_split_report(ws)["width_bits"] == 112
+    for t in range(2):
+        assert np.array_equal(got[t], whole[t][:sm, :sn])
