@@ -290,6 +290,7 @@ __device__ __forceinline__ unsigned __int128 biased_integer(double hi, double lo
 __global__ void __launch_bounds__(kResThreads, kResBlocks) residue_kernel(
     const ResOperand a, const ResOperand b, int64_t k, int64_t k_pad, const SplitPlan plan) {
     __shared__ ResShared sh;
+    chain_begin();
     const PlanPick pk = plan_choice(plan);
     if (pk.c < 0) return;
     const int N = pk.count, DG = pk.width / 8;
@@ -637,6 +638,7 @@ __device__ __forceinline__ void crt_loop(const CrtArgs &p, const CrtTables &T, i
 // tests and branches.
 template <int NW0, int G0>
 __global__ void __launch_bounds__(256, 4) crt_kernel(const __grid_constant__ CrtArgs p) {
+    chain_begin();
     if (p.info != nullptr && *p.info != 0) return;   // an earlier step failed
     const PlanPick pk = plan_choice(p.plan);
     if (pk.c < 0) return;                            // the plain kernel computes C
@@ -744,7 +746,7 @@ int crt_candidates(int64_t k, int *widths, int *counts) {
 struct CrtLayout {
     int N;                                 // moduli the workspace holds (the widest candidate)
     int64_t m_pad, n_pad, k_pad;
-    size_t off_rowmax, off_colmax, off_ra, off_rb, off_res, off_ma, off_mb, off_tri, total;
+    size_t off_rowmax, off_colmax, off_ra, off_rb, off_res, off_ma, off_mb, total;
 };
 
 size_t align1k(size_t x) { return (x + 1023) / 1024 * 1024; }
@@ -782,8 +784,6 @@ CrtLayout crt_layout(int64_t m, int64_t n, int64_t k, bool sym = false) {
     L.off_ma = o; o = align1k(o + 2 * (size_t)L.m_pad * L.k_pad);
     L.off_mb = sym ? L.off_ma : o;
     if (!sym) o = align1k(o + 2 * (size_t)L.n_pad * L.k_pad);
-    L.off_tri = o;   // the band launches' triangle table (Rsyrk form)
-    if (sym) o = align1k(o + 4 * (size_t)kTriMax);
     L.total = o;
     return L;
 }
@@ -810,8 +810,9 @@ int launch_residues(const SplitOperand &a, __half *ra, const SplitOperand *b, __
     }
     x.blocks = (unsigned)na;
     y.blocks = (unsigned)nb;
-    residue_kernel<<<(unsigned)(na + nb), kResThreads, 0, st>>>(x, y, k, k_pad, plan);
-    return check_launch("residue_kernel");
+    return chained_ok(launch_chained_if(ia + ib <= 4 * slots, residue_kernel, (unsigned)(na + nb),
+                                        kResThreads, 0, st, x, y, k, k_pad, plan),
+                      "residue_kernel");
 }
 
 // Reconstruction constants for the first N moduli.
@@ -923,9 +924,8 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     // (the Rsyrk form has one operand: its maxima and planes serve as both)
     if ((rc = launch_absmax(oa, sym ? nullptr : &ob, p.k, st))) return rc;
     if ((rc = launch_magnitude(oa, sym ? nullptr : &ob, p.k, L.k_pad, hdr, init, st))) return rc;
-    int *tri_table = (p.tri && sym) ? reinterpret_cast<int *>(w + L.off_tri) : nullptr;
     if ((rc = launch_certificate(p, w + L.off_ma, w + L.off_mb, L.m_pad, L.n_pad, L.k_pad, TN,
-                                 rmax, cmax, hdr, st, tri_table)))
+                                 rmax, cmax, hdr, st)))
         return rc;
     if ((rc = launch_residues(oa, RA, sym ? nullptr : &ob, RB, p.k, L.k_pad, plan, st))) return rc;
 
@@ -947,7 +947,6 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     ba.status = &hdr->status;
     ba.diag = 1;
     ba.tri = p.tri;
-    ba.tri_cum = tri_table;
     ba.plan = plan;
     for (int i = 0; i < L.N; ++i) ba.moduli[i] = modulus(i);
     if ((rc = launch_band(tmA, tmB, ba, TN, st, &tmB_half))) return rc;
@@ -995,9 +994,9 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     else if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     const unsigned nb = (unsigned)blocks;
-    if (which == 0) crt_kernel<8, 8><<<nb, 256, 0, st>>>(ca);
-    else crt_kernel<9, 9><<<nb, 256, 0, st>>>(ca);
-    if ((rc = check_launch("crt_kernel"))) return rc;
+    const cudaError_t le = which == 0 ? launch_chained(crt_kernel<8, 8>, nb, 256, 0, st, ca)
+                                      : launch_chained(crt_kernel<9, 9>, nb, 256, 0, st, ca);
+    if ((rc = chained_ok(le, "crt_kernel"))) return rc;
     rc = launch_plain_fallback(p, plan, st);
     sliced_timing_mark(3, st);
     return rc;

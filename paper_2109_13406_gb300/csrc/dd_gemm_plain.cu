@@ -80,6 +80,7 @@ __device__ __forceinline__ void tile_coords(const GemmArgs &p, int64_t &bi, int6
 template <int TA, int TB, int R>
 __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
     constexpr int BM = 16 * R, BN = 16 * R;
+    chain_begin();
     if (p.info != nullptr && *p.info != 0) return;  // an earlier step failed
     // behind a split-precision call: compute only when its certificate failed
     if (p.gate != nullptr &&
@@ -232,9 +233,9 @@ int64_t tile_count(const GemmArgs &p, int b) {
 template <int TA, int TB, int R>
 void launch_one(dim3 grid, const GemmArgs &p, cudaStream_t stream) {
     if constexpr (R == 4)
-        dd_gemm_plain_kernel<TA, TB><<<grid, NT, 0, stream>>>(p);
+        launch_chained(dd_gemm_plain_kernel<TA, TB>, grid, NT, 0, stream, p);
     else
-        dd_gemm_plain_small_kernel<TA, TB, R><<<grid, NT, 0, stream>>>(p);
+        launch_chained(dd_gemm_plain_small_kernel<TA, TB, R>, grid, NT, 0, stream, p);
 }
 
 template <int R>

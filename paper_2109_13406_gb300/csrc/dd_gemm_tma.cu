@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                        const __grid_constant__ CUtensorMap tAl,
                        const __grid_constant__ CUtensorMap tBh,
                        const __grid_constant__ CUtensorMap tBl, const TmaGemmArgs a) {
+    chain_begin();
     const GemmArgs &p = a.p;
     if (p.info != nullptr && *p.info != 0) return;   // an earlier step failed
     if (p.gate != nullptr &&
@@ -303,8 +304,9 @@ int launch_t(const CUtensorMap (&m)[4], const TmaGemmArgs &a, int grid, cudaStre
         cudaFuncSetAttribute(dd_gemm_tma_kernel<TA, TB>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     });
-    dd_gemm_tma_kernel<TA, TB><<<grid, kThreads, kSmem, st>>>(m[0], m[1], m[2], m[3], a);
-    return check_launch("dd_gemm_tma_kernel");
+    return chained_ok(launch_chained(dd_gemm_tma_kernel<TA, TB>, grid, kThreads, kSmem, st, m[0],
+                                     m[1], m[2], m[3], a),
+                      "dd_gemm_tma_kernel");
 }
 
 std::atomic<int> g_staging{0};   // 0 automatic, 1 registers only, 2 TMA where it applies

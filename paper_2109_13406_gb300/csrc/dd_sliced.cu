@@ -190,6 +190,7 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
 __global__ void __launch_bounds__(256) absmax_kernel(const SplitOperand a, const SplitOperand b,
                                                      int64_t k, unsigned lchunk) {
     __shared__ unsigned long long part[8][32];
+    chain_begin();
     const bool first = blockIdx.x < a.blocks;
     const double *X = first ? a.hi : b.hi;
     const int64_t ld = first ? a.ld : b.ld, rows = first ? a.rows : b.rows;
@@ -295,6 +296,7 @@ __global__ void __launch_bounds__(128) slice_kernel(const double *__restrict__ X
                                                     int64_t rows_pad, int64_t k_pad,
                                                     const unsigned long long *__restrict__ rmax,
                                                     __half *__restrict__ D, const SplitPlan plan) {
+    chain_begin();
     const PlanPick pk = plan_choice(plan);
     if (pk.c < 0) return;
     const int64_t r = (int64_t)blockIdx.x * (blockDim.x / 2) + threadIdx.x / 2;
@@ -339,6 +341,7 @@ __device__ __forceinline__ uint16_t bf16_floor_scaled(double v, int e) {
 __global__ void __launch_bounds__(128) magnitude_kernel(const SplitOperand a, const SplitOperand b,
                                                         int64_t k, int64_t k_pad, SplitHeader *hdr,
                                                         const SplitHeader init) {
+    chain_begin();
     if (blockIdx.x == 0 && threadIdx.x == 0) *hdr = init;
     const bool first = blockIdx.x < a.blocks;
     const double *X = first ? a.hi : b.hi;
@@ -565,12 +568,13 @@ __device__ __forceinline__ void store_residues(const uint32_t (&r)[16], float pm
 // own tensor memory and releases a buffer with one arrival per warp on the
 // leader's "accumulator empty" barrier.  Every tcgen05 operation of this
 // instantiation is of the pair form.
-// TRI: the work items are the tiles inside the triangle (p.tri_cum); the
+// TRI: the work items are the tiles inside the triangle (tri_prepare); the
 // other instantiations carry no code for it.
 template <int TN, bool MAG, bool PAIR = false, bool TRI = false>
 __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
     band_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                      const __grid_constant__ CUtensorMap tmB, const BandArgs p) {
+    chain_begin();
     int S = p.S;
     if (!MAG && p.plan.dmin != nullptr) {
         // the same decision in every thread of every CTA: a word written by
@@ -596,8 +600,39 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(fin + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
     int *tri_s = TRI ? reinterpret_cast<int *>(smem + STAGES * kStageBytes + 256) : nullptr;
-    if (TRI)   // the triangle table, read by every role per item
-        for (int x = threadIdx.x; x <= p.tri_rows; x += blockDim.x) tri_s[x] = p.tri_cum[x];
+    if (TRI) {
+        // the triangle table, read by every role per item: tiles inside the
+        // triangle before (group, row unit) x in raster order.  Each CTA forms
+        // it (a launch of its own cost ~3 us): a run of rows per thread, then
+        // the runs' sums before it.
+        const TriGeom g{p.tri, PAIR ? 2 * TM : TM, TN, p.tiles_n, kGroupTri};
+        const int per = (p.tri_rows + Cfg::THREADS - 1) / Cfg::THREADS;
+        const int x0 = threadIdx.x * per, x1 = x0 + per < p.tri_rows ? x0 + per : p.tri_rows;
+        int sum = 0;
+        for (int x = x0; x < x1; ++x) {
+            int lo, hi;
+            tri_range(g, x / p.tri_units, x % p.tri_units, lo, hi);
+            sum += hi >= lo ? hi - lo + 1 : 0;
+        }
+        int incl = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d *= 2) {
+            const int o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+            if ((int)(threadIdx.x % 32) >= d) incl += o;
+        }
+        __shared__ int wsum[Cfg::THREADS / 32];
+        if (threadIdx.x % 32 == 31) wsum[threadIdx.x / 32] = incl;
+        __syncthreads();
+        int run = incl - sum;
+        for (int w = 0; w < (int)(threadIdx.x / 32); ++w) run += wsum[w];
+        for (int x = x0; x < x1; ++x) {
+            tri_s[x] = run;
+            int lo, hi;
+            tri_range(g, x / p.tri_units, x % p.tri_units, lo, hi);
+            run += hi >= lo ? hi - lo + 1 : 0;
+        }
+        if (threadIdx.x == 0) tri_s[p.tri_rows] = p.tri_tiles;
+    }
 
     static_assert(!PAIR || (TN == 256 && !MAG), "CTA pairs: residue / digit products, 256 wide");
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -949,6 +984,7 @@ __device__ __forceinline__ double i128_to_double(__int128 v) {
 }
 
 __global__ void __launch_bounds__(256) recombine_kernel(const RecArgs p) {
+    chain_begin();
     const PlanPick pk = plan_choice(p.plan);
     if (pk.c < 0) return;
     const int S = pk.count;
@@ -1070,8 +1106,9 @@ int launch_absmax(const SplitOperand &a, const SplitOperand *b, int64_t k, cudaS
     if (na + nb > 0x7fffffffLL) return fail(MP_DD_ERR_TOO_LARGE, "operands too large for the scaling pass");
     x.blocks = (unsigned)na;
     y.blocks = (unsigned)nb;
-    absmax_kernel<<<(unsigned)(na + nb), 256, 0, st>>>(x, y, k, (unsigned)lchunk);
-    return check_launch("absmax_kernel");
+    return chained_ok(launch_chained(absmax_kernel, (unsigned)(na + nb), 256, 0, st, x, y, k,
+                                     (unsigned)lchunk),
+                      "absmax_kernel");
 }
 
 namespace {
@@ -1082,8 +1119,8 @@ void launch_slice_s(const double *Xh, const double *Xl, int64_t ld, int row_cont
                     const unsigned long long *rmax, __half *D, const SplitPlan &plan,
                     cudaStream_t st) {
     dim3 grid((unsigned)ceil_div(rows_pad, 64), (unsigned)(k_pad / 16));
-    slice_kernel<SA, SB><<<grid, 128, 0, st>>>(Xh, Xl, ld, row_contig, rows, k, rows_pad, k_pad,
-                                               rmax, D, plan);
+    launch_chained(slice_kernel<SA, SB>, grid, 128, 0, st, Xh, Xl, ld, row_contig, rows, k, rows_pad,
+                   k_pad, rmax, D, plan);
 }
 
 // Slice with the certified count among the plan's candidates (one fixed S,
@@ -1249,8 +1286,9 @@ int launch_magnitude(const SplitOperand &a, const SplitOperand *b, int64_t k, in
         return fail(MP_DD_ERR_TOO_LARGE, "operands too large for the certificate");
     x.blocks = (unsigned)na;
     y.blocks = (unsigned)nb;
-    magnitude_kernel<<<(unsigned)(na + nb), 128, 0, st>>>(x, y, k, k_pad, hdr, init);
-    return check_launch("magnitude_kernel");
+    return chained_ok(launch_chained(magnitude_kernel, (unsigned)(na + nb), 128, 0, st, x, y, k,
+                                     k_pad, hdr, init),
+                      "magnitude_kernel");
 }
 
 namespace {
@@ -1266,8 +1304,7 @@ double ratio_lower(mp_dd beta, mp_dd alpha) {
 
 int launch_certificate(const GemmArgs &p, void *MA, void *MB, int64_t m_pad, int64_t n_pad,
                        int64_t k_pad, int TN, const unsigned long long *rmax,
-                       const unsigned long long *cmax, SplitHeader *hdr, cudaStream_t st,
-                       int *tri_table) {
+                       const unsigned long long *cmax, SplitHeader *hdr, cudaStream_t st) {
     // the product's own tile width (n_pad is a multiple of it) when that
     // leaves at least 1024 tiles (~7 per SM): at 8192 the 128 x 256 tiles
     // take the magnitude product from 1.23 to 1.09 ms, at 4096 their 512
@@ -1310,7 +1347,6 @@ int launch_certificate(const GemmArgs &p, void *MA, void *MB, int64_t m_pad, int
     // (|A||B|)_ij 2^-(e_i+f_j) with an eightfold margin on the additions.
     ba.c1 = (float)(1.0 - (double)(p.k + 1) * 0x1p-20);
     ba.dmin_out = &hdr->dmin;
-    ba.tri_cum = p.tri ? tri_table : nullptr;
     return launch_band(tmA, tmB, ba, TN, st);
 }
 
@@ -1403,8 +1439,9 @@ int run_sliced(const GemmArgs &p, int slices, void *ws, size_t ws_bytes, cudaStr
     const int64_t total = p.m * p.n;
     int64_t blocks = ceil_div(total, 256);
     if (blocks > (int64_t)sm_count() * 32) blocks = (int64_t)sm_count() * 32;
-    recombine_kernel<<<(unsigned)blocks, 256, 0, st>>>(ra);
-    if ((rc = check_launch("recombine_kernel"))) return rc;
+    if ((rc = chained_ok(launch_chained(recombine_kernel, (unsigned)blocks, 256, 0, st, ra),
+                         "recombine_kernel")))
+        return rc;
     rc = launch_plain_fallback(p, plan, st);
     timer().mark(3, st);
     return rc;
@@ -1416,54 +1453,16 @@ namespace {
 
 namespace {
 
-// The triangle table of launch_band: cum[x] = tiles inside the triangle
-// before (group, row unit) x in raster order, x = 0 .. rows (one block).
-__global__ void __launch_bounds__(256) tri_table_kernel(TriGeom g, int units, int rows,
-                                                        int *cum) {
-    __shared__ int part[256];
-    const int per = (rows + 255) / 256, x0 = threadIdx.x * per;
-    int s = 0;
-    for (int x = x0; x < x0 + per && x < rows; ++x) {
-        int lo, hi;
-        tri_range(g, x / units, x % units, lo, hi);
-        s += hi >= lo ? hi - lo + 1 : 0;
-    }
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int t = 0; t < 256; ++t) {
-            const int v = part[t];
-            part[t] = run;
-            run += v;
-        }
-    }
-    __syncthreads();
-    int run = part[threadIdx.x];
-    for (int x = x0; x < x0 + per && x < rows; ++x) {
-        cum[x] = run;
-        int lo, hi;
-        tri_range(g, x / units, x % units, lo, hi);
-        run += hi >= lo ? hi - lo + 1 : 0;
-    }
-    if (threadIdx.x == 255) cum[rows] = run;
-}
-
-// Geometry of the triangle table for a launch; 0 when the table does not
-// apply (no triangle, no table memory, or too many rows for shared memory).
-int tri_prepare(BandArgs &ba, int TN, bool pair, cudaStream_t st) {
-    if (!ba.tri || ba.tri_cum == nullptr) {
-        ba.tri_cum = nullptr;
-        return 0;
-    }
+// Geometry of the triangle table for a launch (ba.tri_on stays 0 when the
+// table does not apply: no triangle, or too many rows for shared memory).
+void tri_prepare(BandArgs &ba, int TN, bool pair) {
+    ba.tri_on = 0;
+    if (!ba.tri) return;
     const TriGeom g{ba.tri, pair ? 2 * TM : TM, TN, ba.tiles_n, kGroupTri};
     const int units = pair ? ba.tiles_m / 2 : ba.tiles_m;
     const int groups = (ba.tiles_n + kGroupTri - 1) / kGroupTri;
     const int rows = groups * units;
-    if (rows + 1 > kTriMax) {
-        ba.tri_cum = nullptr;
-        return 0;
-    }
+    if (rows + 1 > kTriMax) return;
     int tiles = 0;
     for (int x = 0; x < rows; ++x) {
         int lo, hi;
@@ -1473,8 +1472,7 @@ int tri_prepare(BandArgs &ba, int TN, bool pair, cudaStream_t st) {
     ba.tri_rows = rows;
     ba.tri_units = units;
     ba.tri_tiles = tiles;
-    tri_table_kernel<<<1, 256, 0, st>>>(g, units, rows, ba.tri_cum);
-    return check_launch("tri_table_kernel");
+    ba.tri_on = 1;
 }
 
 // 0: CTA pairs (the 2-SM MMA) for the Rsyrk triangle, single CTAs for full
@@ -1537,13 +1535,12 @@ int launch_band(const CUtensorMap &tmA, const CUtensorMap &tmB, const BandArgs &
                       (g_band_pairs.load() == 1 || (g_band_pairs.load() == 0 && ba.tri != 0)) &&
                       pair_clusters() > 0;
     BandArgs b = ba;
-    int rc;
-    if ((rc = tri_prepare(b, TN, pair, st))) return rc;
+    tri_prepare(b, TN, pair);
     // work items (see item_coords; S: the most bands the plan may choose)
     const int units = pair ? b.tiles_m / 2 : b.tiles_m;
-    const int tiles = b.tri_cum != nullptr ? b.tri_tiles : units * b.tiles_n;
+    const int tiles = b.tri_on ? b.tri_tiles : units * b.tiles_n;
     const int items = b.diag || b.split ? tiles * b.S : tiles;
-    const bool tt = b.tri_cum != nullptr;
+    const bool tt = b.tri_on != 0;
     if (pair) {
         const int clusters = items < pair_clusters() ? items : pair_clusters();
         cudaLaunchConfig_t cfg{};
@@ -1551,13 +1548,15 @@ int launch_band(const CUtensorMap &tmA, const CUtensorMap &tmB, const BandArgs &
         cfg.blockDim = dim3(BandCfg<256, true>::THREADS);
         cfg.dynamicSmemBytes = tt ? BandCfg<256, true>::SMEM_TRI : BandCfg<256, true>::SMEM;
         cfg.stream = st;
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = 2;
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // (launch_chained)
+        at[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         const cudaError_t e =
             tt ? cudaLaunchKernelEx(&cfg, band_gemm_kernel<256, false, true, true>, tmA,
                                     *tmB_half, b)
@@ -1566,10 +1565,11 @@ int launch_band(const CUtensorMap &tmA, const CUtensorMap &tmB, const BandArgs &
         return check_launch("band_gemm_kernel");
     }
     const int grid = items < sm_count() ? (items > 0 ? items : 1) : sm_count();
-#define MPDD_BAND(TN_, MAG_, TRI_)                                                          \
-    band_gemm_kernel<TN_, MAG_, false, TRI_>                                                \
-        <<<grid, BandCfg<TN_>::THREADS, TRI_ ? BandCfg<TN_>::SMEM_TRI : BandCfg<TN_>::SMEM, \
-           st>>>(tmA, tmB, b)
+    cudaError_t e = cudaSuccess;
+#define MPDD_BAND(TN_, MAG_, TRI_)                                                           \
+    e = launch_chained(band_gemm_kernel<TN_, MAG_, false, TRI_>, (unsigned)grid,             \
+                       BandCfg<TN_>::THREADS,                                                \
+                       TRI_ ? BandCfg<TN_>::SMEM_TRI : BandCfg<TN_>::SMEM, st, tmA, tmB, b)
     if (b.mag && TN == 256) {
         if (tt) MPDD_BAND(256, true, true);
         else MPDD_BAND(256, true, false);
@@ -1584,7 +1584,7 @@ int launch_band(const CUtensorMap &tmA, const CUtensorMap &tmB, const BandArgs &
         else MPDD_BAND(128, false, false);
     }
 #undef MPDD_BAND
-    return check_launch("band_gemm_kernel");
+    return chained_ok(e, "band_gemm_kernel");
 }
 
 int read_status(const void *ws, int *status) {

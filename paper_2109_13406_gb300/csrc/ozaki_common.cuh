@@ -106,11 +106,11 @@ struct BandArgs {
     float c1;                  // 1 - (k + 1) 2^-20 (exact in fp32): the sums' safety factor
     float ba_ratio32;          // ba_ratio rounded toward zero to fp32
     unsigned int *dmin_out;
-    // triangle mode: the work items are the tiles inside the triangle only,
-    // in raster order, through a table of cumulative tile counts per
-    // (raster group, row unit) (tri_rows + 1 entries in device memory,
-    // filled by launch_band); NULL: all tiles, the outside ones skipped
-    int *tri_cum;
+    // tri_on: the work items are the tiles inside the triangle only, in
+    // raster order, through a table of cumulative tile counts per (raster
+    // group, row unit) (tri_rows + 1 entries) that the kernel forms; else all
+    // tiles, the outside ones skipped
+    int tri_on;
     int tri_rows, tri_units, tri_tiles;
 };
 
@@ -176,8 +176,7 @@ int launch_magnitude(const SplitOperand &a, const SplitOperand *b, int64_t k, in
 struct GemmArgs;
 int launch_certificate(const GemmArgs &p, void *MA, void *MB, int64_t m_pad, int64_t n_pad,
                        int64_t k_pad, int TN, const unsigned long long *rmax,
-                       const unsigned long long *cmax, SplitHeader *hdr, cudaStream_t st,
-                       int *tri_table = nullptr);
+                       const unsigned long long *cmax, SplitHeader *hdr, cudaStream_t st);
 // The plain kernel behind the split-precision call: runs only when the
 // certificate fails (plan_choice < 0).
 int launch_plain_fallback(const GemmArgs &p, const SplitPlan &plan, cudaStream_t st);

@@ -320,3 +320,38 @@ def test_crt_entry_and_pair_threads_agree(cuda_lib, sub):
     assert cuda_lib.mp_dd_split_report(ws)["width_bits"] == 112
     for t in range(2):
         assert np.array_equal(got[t], whole[t][:sm, :sn])
+
+
+@pytest.mark.parametrize("m,n,k", [(140, 270, 90), (1400, 1300, 200)])
+def test_chained_launches_replay_from_a_graph(cuda_lib, m, n, k):
+    """The call's kernels, launched chained, captured in a CUDA graph: replays
+    on new operand values give the bits of an eager call."""
+    mp = cuda_lib
+    cases = [datagen.gemm_case(770 + t, "N", "N", m, n, k) for t in range(2)]
+    A, B, C = dev(cases[0].A), dev(cases[0].B), dev(cases[0].C)
+    ws = mp.workspace(mp.mp_dd_Rgemm_crt_workspace(m, n, k))
+
+    def call():
+        mp.mp_dd_Rgemm_crt("N", "N", m, n, k, (1.5, 0.0), A, m, B, k, (0.0, 0.0), C, m, ws,
+                           ws.numel())
+
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        call()
+    torch.cuda.current_stream().wait_stream(s)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    for c in (*cases, cases[0]):
+        for dst, src in zip((*A, *B), (*dev(c.A), *dev(c.B))):
+            dst.copy_(src)
+        call()
+        want = host(C, m, n)
+        for x in C:
+            x.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert mp.mp_dd_workspace_status(ws) == 0
+        got = host(C, m, n)
+        assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
