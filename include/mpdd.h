@@ -21,8 +21,8 @@
  * pointer is DEVICE memory owned by the caller, and every call is
  * asynchronous on the calling thread's current stream (mp_dd_set_stream).
  * The library keeps nothing allocated beyond a call except what a call
- * documents (the host forms' memory pool, the no-allocation form's fixed
- * array).
+ * documents (the host forms' memory pool, the triangular solves' pool, the
+ * no-allocation form's fixed array).
  *
  * Return codes (all int-returning calls):
  *    0            success
@@ -236,7 +236,12 @@ int mp_dd_Rsyrk_host(const char *uplo, const char *trans, int64_t n, int64_t k, 
  * or n = 0 returns at once.  Arithmetic: substitution on 64 x 64 diagonal
  * blocks (dd division by the diagonal) and dd Rgemm updates of the
  * off-diagonal blocks, split recursively in halves so that the updates are
- * large products.  Accuracy: the componentwise backward error of
+ * large products; the large ones (all three dimensions at least 96) run in
+ * residue form on the tensor cores at an operand width that rounds within 2
+ * u^2 (u = 2^-53) of |A||X| + |B| entry by entry, or on the FP64 pipe when no
+ * width does, while the stream is being captured, or when their workspace (at
+ * most 4 GiB, stream-ordered, from a pool of the library that keeps at most 2
+ * GiB between calls) cannot be had.  Accuracy: the componentwise backward error of
  * substitution, |op(A) X - alpha B| <= 4 (n_A + 2) 2^-104 (|op(A)||X| +
  * |alpha B|), n_A the order of A; a zero diagonal entry gives Inf/NaN as
  * DTRSM does (no check).  Asynchronous on the current stream.
@@ -258,7 +263,8 @@ int mp_dd_Rtrsm(const char *side, const char *uplo, const char *transa, const ch
  * of largest dd magnitude.  *info (DEVICE int64, required) receives 0 or
  * j > 0 when U(j, j) is exactly zero (the factorisation completes, as in
  * LAPACK).  Recursive column splitting (LAPACK's dgetrf2): the updates are
- * dd Rtrsm and dd Rgemm products, the leaves panels of at most 32 columns,
+ * dd Rtrsm and dd Rgemm products (the large ones on the tensor cores, as in
+ * mp_dd_Rtrsm), the leaves panels of at most 32 columns,
  * each one cooperative launch with its rows spread over the SMs.  A
  * panel's grid-barrier waits are bounded (~2 s, which co-resident CTAs
  * never reach); a wait that gives up stops the panel and sets *info = -1.

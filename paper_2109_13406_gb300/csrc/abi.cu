@@ -58,13 +58,15 @@ int require_device() {
 }
 
 // The library's own stream-ordered memory pool on each device, for the
-// scratch buffers of the host-buffer forms and the LU panels.  Its release
-// threshold keeps freed memory mapped for the next call (the device's
-// default pool would hand it back to the driver at every synchronisation,
-// and mapping a gigabyte again costs tens of milliseconds).
-cudaError_t pool_alloc(void **ptr, size_t bytes, cudaStream_t st) {
+// scratch buffers of the host-buffer forms and the LU panels, and another for
+// the workspaces of tensor-core updates.  The first one's release threshold
+// keeps freed memory mapped for the next call (the device's default pool
+// would hand it back to the driver at every synchronisation, and mapping a
+// gigabyte again costs tens of milliseconds); the second keeps kScratchKeep.
+cudaError_t pool_alloc(void **ptr, size_t bytes, cudaStream_t st, PoolKind kind) {
     static std::mutex mu;
-    static cudaMemPool_t pools[kMaxDevices] = {};
+    static cudaMemPool_t all_pools[kPoolKinds][kMaxDevices] = {};
+    cudaMemPool_t *pools = all_pools[kind];
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= kMaxDevices) return cudaMallocAsync(ptr, bytes, st);
@@ -81,7 +83,7 @@ cudaError_t pool_alloc(void **ptr, size_t bytes, cudaStream_t st) {
                 pools[dev] = nullptr;
                 return e;
             }
-            uint64_t keep = UINT64_MAX;
+            uint64_t keep = kind == kPoolScratch ? kScratchKeep : UINT64_MAX;
             cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
         }
         pool = pools[dev];

@@ -122,8 +122,13 @@ int require_device();
 
 // Number of SMs of the current device (cached).
 int sm_count();
-// Stream-ordered allocation from the library's own pool (freed memory stays
-// mapped for later calls); free with cudaFreeAsync.
-cudaError_t pool_alloc(void **ptr, size_t bytes, cudaStream_t st);
+// Stream-ordered allocation from the library's own pools; free with
+// cudaFreeAsync.  kPoolHost (the host forms' buffers, small exchange buffers):
+// freed memory stays mapped for later calls.  kPoolScratch (workspaces of the
+// factorisations' and solves' tensor-core updates): at most kScratchKeep bytes
+// of freed memory stay mapped past a synchronisation.
+enum PoolKind { kPoolHost = 0, kPoolScratch = 1, kPoolKinds = 2 };
+constexpr uint64_t kScratchKeep = 2ull << 30;
+cudaError_t pool_alloc(void **ptr, size_t bytes, cudaStream_t st, PoolKind kind = kPoolHost);
 
 }  // namespace mpdd

@@ -289,6 +289,66 @@ int launch_plain_fallback(const GemmArgs &p, const SplitPlan &plan, cudaStream_t
     return launch_gemm_plain(q, stream);
 }
 
+// Where the residue form takes an update of a factorisation or solve over
+// from the plain kernel.  The plain kernel's time is its busiest SM's: 0.72 us
+// per step of k and 16 x 16 tile (9.75 FP64 instructions per multiply-add at
+// 526 G/s over 152 SMs); the residue form must be estimated at four fifths of
+// it.  LU and solve of order 1536 with 500 right-hand sides: 71.0 ms with every
+// update on the FP64 pipe, 31.9 so.
+// The inner dimension and both outer ones have to reach kUpdateMin: below it
+// the time is latency either way, and a solve's or a factorisation's result
+// then does not depend on how many columns go with it.
+// With `tight` = 2 the residue form's operand rounding stays within 2 u^2
+// (|A||B| + |C|) entry by entry, and its other roundings within 4 u^2, against
+// the plain kernel's sum of k roundings of up to ~8 u^2; a call whose operands
+// do not allow that at 128 bits, or hold an infinity or NaN, is computed by
+// the plain kernel behind it.
+constexpr int64_t kUpdateMin = 96;
+constexpr double kTightUpdate = 2.0;
+constexpr size_t kUpdateScratch = size_t(4) << 30;   // larger updates go in blocks
+
+int launch_gemm_update(const GemmArgs &p, cudaStream_t stream) {
+    if (p.m < kUpdateMin || p.n < kUpdateMin || p.k < kUpdateMin || p.k > ((int64_t)1 << 17) - 1 ||
+        p.tri != 0 || p.alpha_zero || p.a2h != nullptr || p.sym_a || p.sym_b)
+        return launch_gemm_plain(p, stream);
+    const double plain_us = 0.72 * (double)p.k * (double)plain_tile_cost(p, plain_tile_r(p));
+    if (crt_estimate_us(p.m, p.n, p.k) > 0.8 * plain_us) return launch_gemm_plain(p, stream);
+    // allocations inside a stream capture would belong to the graph
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return launch_gemm_plain(p, stream);
+    }
+    int64_t bm = p.m, bn = p.n;
+    while (crt_workspace_bytes(bm, bn, p.k) > kUpdateScratch) {
+        int64_t &big = bm > bn ? bm : bn;
+        if (big <= 1024) return launch_gemm_plain(p, stream);
+        big = ceil_div(big / 2, (int64_t)256) * 256;
+    }
+    const size_t bytes = crt_workspace_bytes(bm, bn, p.k);
+    void *ws = nullptr;
+    if (pool_alloc(&ws, bytes, stream, kPoolScratch) != cudaSuccess) {
+        cudaGetLastError();
+        return launch_gemm_plain(p, stream);
+    }
+    int rc = 0;
+    for (int64_t j = 0; j < p.n && rc == 0; j += bn)
+        for (int64_t i = 0; i < p.m && rc == 0; i += bm) {
+            GemmArgs q = p;
+            q.m = p.m - i < bm ? p.m - i : bm;
+            q.n = p.n - j < bn ? p.n - j : bn;
+            const int64_t oa = p.ta ? i * p.lda : i, ob = p.tb ? j : j * p.ldb;
+            q.ah += oa; q.al += oa;
+            q.bh += ob; q.bl += ob;
+            q.ch += i + j * p.ldc; q.cl += i + j * p.ldc;
+            q.tight = kTightUpdate;
+            rc = run_crt(q, ws, bytes, stream);
+        }
+    const cudaError_t e = cudaFreeAsync(ws, stream);
+    if (rc == 0 && e != cudaSuccess) return cuda_fail(e, "update workspace");
+    return rc;
+}
+
 int launch_gemm_plain(const GemmArgs &p, cudaStream_t stream) {
     int rc = 0;
     if (try_launch_gemm_tma(p, stream, &rc)) return rc;

@@ -749,8 +749,9 @@ int run_potrs(int lower, int64_t n, int64_t nrhs, const double *ah, const double
 // T recursively into halves (at multiples of 64): solve the first half,
 // update the second half's right-hand sides with one dd Rgemm of the whole
 // off-diagonal block, solve the second half.  The leaves are 64 x 64
-// diagonal blocks in shared memory.  alpha is applied where each row block
-// of B' is first touched: by the leaf kernel (the first block) or as the
+// diagonal blocks in shared memory.  Large updates run in residue form on the
+// tensor cores at dd accuracy (launch_gemm_update).  alpha is applied where
+// each row block of B' is first touched: by the leaf kernel (the first block) or as the
 // beta of its first Rgemm update.
 
 namespace {
@@ -807,7 +808,7 @@ int trsm_update(const TrsmPlan &P, int64_t r0, int64_t mr, int64_t c0, int64_t k
         p.bh = P.ah + ot; p.bl = P.al + ot; p.ldb = P.lda; p.tb = !tl;
         p.ch = P.bh + r0 * P.ldb; p.cl = P.bl + r0 * P.ldb; p.ldc = P.ldb;
     }
-    return launch_gemm_plain(p, P.st);
+    return launch_gemm_update(p, P.st);
 }
 
 int trsm_rec(const TrsmPlan &P, int64_t j0, int64_t nt, bool first) {
@@ -850,8 +851,9 @@ int run_trsm(int right, int lower, int trans, int unit, int64_t m, int64_t n, mp
 // LU factorisation with partial pivoting, P A = L U (DGETRF semantics), by
 // the recursive column splitting of LAPACK's dgetrf2: factor the left half
 // of the columns (recursively), solve L11 U12 = A12 (the Rtrsm above, unit
-// lower), update A22 -= L21 U12 (the plain dd Rgemm kernel, or a
-// one-thread-per-entry kernel when k or n is small), factor A22
+// lower), update A22 -= L21 U12 (in residue form on the tensor cores or by the
+// plain dd Rgemm kernel, see launch_gemm_update, or by a one-thread-per-entry
+// kernel when k or n is small), factor A22
 // (recursively).  The leaves are panels of at most 32 columns, each one
 // cooperative launch (getrf_panel_kernel below) followed by one launch that
 // applies its interchanges to the other columns; where that kernel cannot
@@ -1375,7 +1377,7 @@ int getrf_rec(const LuPlan &P, int64_t j0, int64_t n) {
         g.ch = P.ah + o22; g.cl = P.al + o22; g.ldc = P.lda;
         g.ta = 0; g.tb = 0; g.tri = 0;
         g.alpha_zero = 0; g.alpha_one = 0; g.beta_zero = 0;
-        if ((rc = launch_gemm_plain(g, P.st))) return rc;
+        if ((rc = launch_gemm_update(g, P.st))) return rc;
         if ((rc = getrf_rec(P, j0 + n1, n2))) return rc;
     }
     return 0;

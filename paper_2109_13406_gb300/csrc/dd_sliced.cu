@@ -440,6 +440,7 @@ __device__ __forceinline__ void item_coords(const BandArgs &p, int S, int item, 
 }
 
 constexpr unsigned int kInfBits32 = 0x7F800000u;   // +inf as fp32 bits
+constexpr unsigned long long kInfBits64 = 0x7FF0000000000000ull;   // +inf as binary64 bits
 
 // A lower bound of |c| 2^-s (c a finite binary64, s an integer) as an fp32:
 // the significand truncated to 24 bits and the exponent shifted; 0 below
@@ -464,7 +465,8 @@ __device__ __forceinline__ float scaled_floor_f32(double c, int s) {
 // margin of a lower bound of (|A||B|)_ij.  Rows or columns that are all zero
 // (exact in every form), entries outside C or the requested triangle, and
 // entries whose C is infinite or NaN (then so is the result) do not
-// constrain.  Used by all 32 lanes of an epilogue warp (rows i of the lanes,
+// constrain.  An infinite or NaN row or column maximum leaves no margin: the
+// plain kernel computes such a product.  Used by all 32 lanes of an epilogue warp (rows i of the lanes,
 // the same EC columns): each lane loads EC / 32 column maxima and the warp
 // shares them by shuffles.  C is read 16 columns at a time, the first 16
 // before the tile's accumulator is complete (under the tile's MMAs).  The
@@ -474,6 +476,7 @@ struct Margin {
     static_assert(EC == 64 || EC == 128, "64 or 128 columns");
     static constexpr int NC = EC / 32;   // column maxima per lane
     unsigned mask;
+    bool bad;   // a row or column with an infinity or NaN
     int fcol[NC];
     bool zcol[NC];
     bool row_ok, use_c;
@@ -485,15 +488,18 @@ struct Margin {
         : i(i_), j0(j0_) {
         mask = __activemask();
         const int lane = threadIdx.x & 31;
+        bad = false;
 #pragma unroll
         for (int h = 0; h < NC; ++h) {
             const int64_t j = j0 + 32 * h + lane;
             const unsigned long long cm = j < p.n ? p.cmax[j] : 0ull;
+            bad |= cm >= kInfBits64;
             zcol[h] = cm == 0;
             fcol[h] = scale_exponent(cm);
         }
         const unsigned long long rm = i < p.m ? p.rmax[i] : 0ull;
         row_ok = rm != 0;
+        bad |= rm >= kInfBits64;
         ei = scale_exponent(rm);
         use_c = p.ba_ratio32 > 0.0f;
         dm = kInfBits32;
@@ -524,6 +530,7 @@ struct Margin {
         }
     }
     __device__ __forceinline__ void finish(const BandArgs &p) {
+        if (bad) dm = 0;
         dm = __reduce_min_sync(mask, dm);
         if ((threadIdx.x & 31) == 0 && dm != kInfBits32) atomicMin(p.dmin_out, dm);
     }

@@ -37,10 +37,19 @@ struct GemmArgs {
     // below gate_below, i.e. when no operand width certified the bound.
     const unsigned int *gate = nullptr;
     unsigned int gate_below = 0;
+    // Split-precision calls: 0 = the width certifies the accuracy bound
+    // (operand rounding within 12 k u^2 of |alpha||A||B| + |beta||C|, u =
+    // 2^-53); otherwise within `tight` u^2 of it, so that the result is at
+    // least as accurate as the dd arithmetic of the plain kernel.
+    double tight = 0.0;
 };
 
 // Plain FP64 dd kernel (64 x 64 output tiles, 4 x 4 dd accumulators per thread).
 int launch_gemm_plain(const GemmArgs &p, cudaStream_t stream);
+// An update of a factorisation or solve: the residue form at dd accuracy
+// (tight) where it is faster and its workspace can be had, else the plain
+// kernel.
+int launch_gemm_update(const GemmArgs &p, cudaStream_t stream);
 // The TMA-staged form of the plain kernel (dd_gemm_tma.cu): 1 when it took the
 // problem (*rc its launch status), 0 when the register-staged kernels must.
 int try_launch_gemm_tma(const GemmArgs &p, cudaStream_t stream, int *rc);
@@ -111,6 +120,8 @@ int launch_trsm_batch(int64_t count, const mp_dd_trsm_desc *ds, int64_t max_rhs,
 
 // Residue (CRT) form of the split-precision Rgemm.
 size_t crt_workspace_bytes(int64_t m, int64_t n, int64_t k, bool sym = false);
+// Estimated time of the residue form of an m x n x k product (us).
+double crt_estimate_us(int64_t m, int64_t n, int64_t k);
 int crt_layout_query(int64_t m, int64_t n, int64_t k, size_t *offsets, int *count);
 // p.tri != 0: the Rsyrk form (op(B) = op(A)^T, one triangle of C).
 int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t stream);

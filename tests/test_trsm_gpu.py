@@ -168,3 +168,47 @@ def test_result_independent_of_columns_per_cta(cuda_lib, transa):
         outs.append(gpu_trsm(cuda_lib, sub))
     for h, l in outs[1:]:
         assert np.array_equal(h[:, :6], outs[0][0]) and np.array_equal(l[:, :6], outs[0][1])
+
+
+@pytest.mark.parametrize("side,uplo,transa,diag",
+                         [("L", "U", "N", "N"), ("L", "L", "N", "U"), ("R", "U", "T", "N"),
+                          ("R", "L", "T", "U")])
+@pytest.mark.parametrize("form", ["plain", "scaled", "nonfinite"])
+def test_tensor_core_updates(cuda_lib, side, uplo, transa, diag, form):
+    """Orders whose updates run in residue form (700 with 900 right-hand
+    sides): the backward error stays within a tenth of the bound of
+    substitution (per entry at most five updates of 6u^2 and 64 steps of 8u^2
+    against 16 * 702 u^2: 0.05).  "scaled": rows of the triangle and of B over
+    120 binades, so that updates need wider operands or the FP64 pipe.
+    "nonfinite": an infinity in one column (row) of B spoils that one only."""
+    m, n = (700, 900) if side == "L" else (900, 700)
+    c = datagen.trsm_case(860, side, uplo, transa, diag, m, n)
+    g = datagen.rng(861)
+    order = 700
+    if form == "scaled":
+        # D A D^-1 keeps the triangle's diagonal; B scaled along the other side
+        e = g.integers(-30, 31, order)
+        f = np.ldexp(1.0, e)
+        for P in c.A:
+            P[:order] *= f[:, None] / f[None, :]
+        h = np.ldexp(1.0, g.integers(-60, 61, 900))
+        for P in c.B:
+            P[:m] *= h[None, :] if side == "L" else h[:, None]
+    if form == "nonfinite":
+        c.B[0][(5, 7) if side == "L" else (7, 5)] = np.inf
+    X = gpu_trsm(cuda_lib, c)
+    keep = np.arange(900) != 7
+    if form == "nonfinite":
+        bad = X[0][:, 7] if side == "L" else X[0][7]
+        assert not np.isfinite(bad).all()
+        rest = X[0][:, keep] if side == "L" else X[0][keep]
+        assert np.isfinite(rest).all()
+    rows, cols = g.integers(0, m, 1200), g.integers(0, n, 1200)
+    rows[:40], cols[40:80] = m - 1, n - 1
+    rows[80:120], cols[120:160] = 0, 0
+    if form == "nonfinite":
+        ok = (cols if side == "L" else rows) != 7
+        rows, cols = rows[ok], cols[ok]
+        for P in (*c.B, *X):
+            P[~np.isfinite(P)] = 0.0
+    assert trsm_residual_over_bound(c, X, rows, cols) <= 0.1
