@@ -718,15 +718,21 @@ uint32_t inv_mod(uint32_t a, uint32_t p) {   // a^-1 mod p (gcd(a, p) = 1)
 // Smallest even moduli count with P >= k 2^(2W) > 4 max |A' B'| (|A'|,
 // |B'| < 2^(W-1)); -1 when the 40 moduli do not reach it.
 int moduli_count(int64_t k, int W) {
+    static int bits[kMaxMod + 1];   // of the products of the first N moduli
+    static std::once_flag once;
+    std::call_once(once, [] {
+        Big P{1};
+        for (int N = 1; N <= kMaxMod; ++N) {
+            P = big_mul_small(P, modulus(N - 1));
+            bits[N] = big_bits(P);
+        }
+    });
     const int need = 2 * W + (int)std::ceil(std::log2((double)(k > 1 ? k : 1)));
-    Big P{1};
-    for (int N = 1; N <= kMaxMod; ++N) {
-        P = big_mul_small(P, modulus(N - 1));
-        if (big_bits(P) > need) {                        // P >= 2^need
+    for (int N = 1; N <= kMaxMod; ++N)
+        if (bits[N] > need) {                            // P >= 2^need
             const int even = N % 2 ? N + 1 : N;          // residues come in pairs
             return even <= kMaxMod ? even : -1;
         }
-    }
     return -1;
 }
 
@@ -815,8 +821,9 @@ int launch_residues(const SplitOperand &a, __half *ra, const SplitOperand *b, __
                       "residue_kernel");
 }
 
-// Reconstruction constants for the first N moduli.
-int crt_tables(int N, CrtTables &T, int *nwords) {
+// Reconstruction constants for the first N moduli, formed with multiword
+// integers on the host.
+int make_crt_tables(int N, CrtTables &T, int *nwords) {
     memset(&T, 0, sizeof T);
     Big P{1};
     for (int i = 0; i < N; ++i) P = big_mul_small(P, modulus(i));
@@ -849,6 +856,24 @@ int crt_tables(int N, CrtTables &T, int *nwords) {
     int need = big_bits(P) + 1;
     for (int64_t x = 255LL * N - 1; x > 0; x >>= 1) ++need;
     *nwords = (need + 31) / 32;
+    return 0;
+}
+
+// The same, formed once per N and process (forming them took ~8 us per
+// candidate width and call: 56 us of host time per call, 32 since).
+int crt_tables(int N, CrtTables &T, int *nwords) {
+    struct Entry {
+        std::once_flag once;
+        CrtTables T;
+        int words = 0, rc = 0;
+    };
+    static Entry cache[kMaxMod + 1];
+    if (N < 1 || N > kMaxMod) return fail(MP_DD_ERR_TOO_LARGE, "%d moduli", N);
+    Entry &e = cache[N];
+    std::call_once(e.once, [&] { e.rc = make_crt_tables(N, e.T, &e.words); });
+    if (e.rc) return fail(e.rc, "moduli product too wide");
+    T = e.T;
+    *nwords = e.words;
     return 0;
 }
 
