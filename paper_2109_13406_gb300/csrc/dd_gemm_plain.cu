@@ -13,8 +13,11 @@
 // On GB300 the FP64 pipe is the bottleneck by a wide margin (9.75 FP64
 // instructions per dd multiply-add), so the kernel is organised to keep that
 // pipe busy and nothing else (large plain products go to the TMA-staged form
-// of this kernel, dd_gemm_tma.cu, whose per-entry arithmetic is identical): each CTA owns a 16R x 16R tile of C (R = 4, 2
-// or 1), each thread an R x R block of dd accumulators, and the hi/lo planes
+// of this kernel, dd_gemm_tma.cu, whose per-entry arithmetic is identical):
+// each CTA owns a 16R x 16R tile of C (R = 4, 2 or 1), each thread an R x R
+// block of dd accumulators (or a 16 x 8 or 32 x 4 tile of one entry per
+// thread, for products that leave SMs without a 16 x 16 tile: four warps, one
+// per partition of the SM, so a step of k takes half as long), and the hi/lo planes
 // of the op(A) and op(B) panels are staged through shared memory 16 columns
 // of k at a time with a register prefetch of the next panel.  One SM's FP64
 // pipe issues only 2 lanes per clock, so a few warps keep it busy whatever R
@@ -33,13 +36,24 @@
 namespace mpdd {
 namespace {
 
-constexpr int BK = 16, NT = 256;
+constexpr int BK = 16;
 
+// Tile shapes: TX x TY threads, each an R x R block of entries TX (TY) apart.
+template <int R_, int TX_, int TY_>
+struct PlainShape {
+    static constexpr int R = R_, TX = TX_, TY = TY_, NT = TX_ * TY_;
+    static constexpr int BM = TX_ * R_, BN = TY_ * R_;
+    static constexpr int QA = (BM * BK + NT - 1) / NT, QB = (BN * BK + NT - 1) / NT;
+};
 template <int R>
+using Square = PlainShape<R, 16, 16>;
+using Half = PlainShape<1, 16, 8>;    // 16 x 8
+using Tall = PlainShape<1, 32, 4>;    // 32 x 4
+
+template <class S>
 struct PlainSmem {
-    static constexpr int B = 16 * R;
-    double ah[BK][B + 1], al[BK][B + 1];  // op(A) panel, [l][i]
-    double bh[BK][B + 1], bl[BK][B + 1];  // op(B) panel, [l][j]
+    double ah[BK][S::BM + 1], al[BK][S::BM + 1];  // op(A) panel, [l][i]
+    double bh[BK][S::BN + 1], bl[BK][S::BN + 1];  // op(B) panel, [l][j]
 };
 
 constexpr int GROUP_N = 8;  // tile columns per rasterisation group
@@ -48,8 +62,8 @@ constexpr int GROUP_N = 8;  // tile columns per rasterisation group
 // tile columns with the tile row fastest inside a group, so the CTAs
 // resident at one time share a few A row panels and B column panels in L2
 // (a plain column-by-column order re-reads all of A for every tile column).
-// Rsyrk: a 1-D grid over the tiles of one triangle, t -> (row, col) with
-// row <= col (upper) or row >= col (lower).
+// Rsyrk: a 1-D grid over the square tiles of one triangle, t -> (row, col)
+// with row <= col (upper) or row >= col (lower); a 16 x 8 tile is half of one.
 template <int BM, int BN>
 __device__ __forceinline__ void tile_coords(const GemmArgs &p, int64_t &bi, int64_t &bj) {
     if (p.tri == 0) {
@@ -63,7 +77,8 @@ __device__ __forceinline__ void tile_coords(const GemmArgs &p, int64_t &bi, int6
         bi = local / gn;
         return;
     }
-    int64_t t = blockIdx.x;
+    constexpr int64_t kParts = BM / BN;
+    int64_t t = blockIdx.x / kParts;
     int64_t r = (int64_t)((__dsqrt_rn(8.0 * (double)t + 1.0) - 1.0) * 0.5);
     while (r * (r + 1) / 2 > t) --r;
     while ((r + 1) * (r + 2) / 2 <= t) ++r;
@@ -75,11 +90,13 @@ __device__ __forceinline__ void tile_coords(const GemmArgs &p, int64_t &bi, int6
         bi = r;
         bj = c;
     }
+    bj = bj * kParts + blockIdx.x % kParts;
 }
 
-template <int TA, int TB, int R>
-__device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
-    constexpr int BM = 16 * R, BN = 16 * R;
+template <int TA, int TB, class S>
+__device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<S> &s) {
+    constexpr int R = S::R, BM = S::BM, BN = S::BN, NT = S::NT, QA = S::QA, QB = S::QB;
+    constexpr int TX = S::TX, TY = S::TY;
     chain_begin();
     if (p.info != nullptr && *p.info != 0) return;  // an earlier step failed
     // behind a split-precision call: compute only when its certificate failed
@@ -88,7 +105,7 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
         return;
     int64_t bi, bj;
     tile_coords<BM, BN>(p, bi, bj);
-    const int t = threadIdx.x, tx = t % 16, ty = t / 16;
+    const int t = threadIdx.x, tx = t % TX, ty = t / TX;
     const int64_t i0 = bi * BM, j0 = bj * BN;
     // the k loop: [0, k) over (A, B), then for Rsyr2k [k1, k1 + k) over
     // (A2, B2), k1 = k rounded up to whole panels (zero products between)
@@ -101,8 +118,8 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
 #pragma unroll
         for (int c = 0; c < R; ++c) acc[r][c] = dd{0.0, 0.0};
 
-    // a panel holds 16R x 16 entries of op(A) and of op(B): R per thread
-    double rah[R], ral[R], rbh[R], rbl[R];
+    // a panel holds BM x 16 entries of op(A) and BN x 16 of op(B)
+    double rah[QA], ral[QA], rbh[QB], rbl[QB];
     // Element q of this thread's share of a panel: (row-in-panel, l).
     auto a_pos = [&](int q, int &ii, int &ll) {
         int idx = t + NT * q;
@@ -121,7 +138,7 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
         const int64_t lda = second ? p.lda2 : p.lda, ldb = second ? p.ldb2 : p.ldb;
         const int64_t lb = second ? l0 - k1 : l0;
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
+        for (int q = 0; q < QA; ++q) {
             int ii, ll;
             a_pos(q, ii, ll);
             int64_t gi = i0 + ii, gl = lb + ll;
@@ -133,12 +150,14 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
             }
             rah[q] = ok ? Ah[off] : 0.0;
             ral[q] = ok ? Al[off] : 0.0;
-            int jj;
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            int jj, ll;
             b_pos(q, jj, ll);
-            int64_t gj = j0 + jj;
-            gl = lb + ll;
-            ok = gj < p.n && gl < p.k;
-            off = TB ? (gj + gl * ldb) : (gl + gj * ldb);
+            int64_t gj = j0 + jj, gl = lb + ll;
+            bool ok = gj < p.n && gl < p.k && (BN * BK >= NT || t < BN * BK);
+            int64_t off = TB ? (gj + gl * ldb) : (gl + gj * ldb);
             if (p.sym_b) {
                 const bool direct = p.sym_b == 1 ? gl <= gj : gl >= gj;
                 off = direct ? gl + gj * ldb : gj + gl * ldb;
@@ -149,14 +168,20 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
     };
     auto stage = [&]() {
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-            int ii, jj, ll;
+        for (int q = 0; q < QA; ++q) {
+            int ii, ll;
             a_pos(q, ii, ll);
             s.ah[ll][ii] = rah[q];
             s.al[ll][ii] = ral[q];
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
+            int jj, ll;
             b_pos(q, jj, ll);
-            s.bh[ll][jj] = rbh[q];
-            s.bl[ll][jj] = rbl[q];
+            if (BN * BK >= NT || t < BN * BK) {
+                s.bh[ll][jj] = rbh[q];
+                s.bl[ll][jj] = rbl[q];
+            }
         }
     };
 
@@ -174,10 +199,10 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
                     dd a[R], b[R];
 #pragma unroll
                     for (int r = 0; r < R; ++r)
-                        a[r] = dd{s.ah[l][tx + 16 * r], s.al[l][tx + 16 * r]};
+                        a[r] = dd{s.ah[l][tx + TX * r], s.al[l][tx + TX * r]};
 #pragma unroll
                     for (int c = 0; c < R; ++c)
-                        b[c] = dd{s.bh[l][ty + 16 * c], s.bl[l][ty + 16 * c]};
+                        b[c] = dd{s.bh[l][ty + TY * c], s.bl[l][ty + TY * c]};
 #pragma unroll
                     for (int r = 0; r < R; ++r)
 #pragma unroll
@@ -196,7 +221,7 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
     for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < R; ++c) {
-            int64_t i = i0 + tx + 16 * r, j = j0 + ty + 16 * c;
+            int64_t i = i0 + tx + TX * r, j = j0 + ty + TY * c;
             if (i >= p.m || j >= p.n) continue;
             if ((p.tri == 1 && i > j) || (p.tri == 2 && i < j)) continue;
             dd v = p.alpha_one ? acc[r][c] : mul(alpha, acc[r][c]);
@@ -210,65 +235,90 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<R> &s) {
 // 64 x 64 tiles (one CTA per SM by registers) and the smaller tiles (two or
 // more CTAs per SM, registers capped accordingly).
 template <int TA, int TB>
-__global__ void __launch_bounds__(NT) dd_gemm_plain_kernel(const GemmArgs p) {
-    __shared__ PlainSmem<4> s;
-    plain_body<TA, TB, 4>(p, s);
+__global__ void __launch_bounds__(256) dd_gemm_plain_kernel(const GemmArgs p) {
+    __shared__ PlainSmem<Square<4>> s;
+    plain_body<TA, TB, Square<4>>(p, s);
 }
 
-template <int TA, int TB, int R>
-__global__ void __launch_bounds__(NT, 2) dd_gemm_plain_small_kernel(const GemmArgs p) {
-    __shared__ PlainSmem<R> s;
-    plain_body<TA, TB, R>(p, s);
+template <int TA, int TB, class S>
+__global__ void __launch_bounds__(S::NT, 2) dd_gemm_plain_small_kernel(const GemmArgs p) {
+    __shared__ PlainSmem<S> s;
+    plain_body<TA, TB, S>(p, s);
 }
 
 }  // namespace
 
 namespace {
 
-int64_t tile_count(const GemmArgs &p, int b) {
-    const int64_t tm = ceil_div(p.m, b), tn = ceil_div(p.n, b);
-    return p.tri == 0 ? tm * tn : tm * (tm + 1) / 2;
+int64_t tile_count(const GemmArgs &p, int bm, int bn) {
+    const int64_t tm = ceil_div(p.m, bm);
+    return p.tri == 0 ? tm * ceil_div(p.n, bn) : tm * (tm + 1) / 2 * (bm / bn);
 }
 
-template <int TA, int TB, int R>
+template <int TA, int TB, class S>
 void launch_one(dim3 grid, const GemmArgs &p, cudaStream_t stream) {
-    if constexpr (R == 4)
-        launch_chained(dd_gemm_plain_kernel<TA, TB>, grid, NT, 0, stream, p);
+    if constexpr (S::R == 4)
+        launch_chained(dd_gemm_plain_kernel<TA, TB>, grid, S::NT, 0, stream, p);
     else
-        launch_chained(dd_gemm_plain_small_kernel<TA, TB, R>, grid, NT, 0, stream, p);
+        launch_chained(dd_gemm_plain_small_kernel<TA, TB, S>, grid, S::NT, 0, stream, p);
 }
 
-template <int R>
-int launch_r(const GemmArgs &p, cudaStream_t stream) {
-    const int64_t tiles = tile_count(p, 16 * R);
+template <class S>
+int launch_shape(const GemmArgs &p, cudaStream_t stream) {
+    const int64_t tiles = tile_count(p, S::BM, S::BN);
     if (tiles > 0x7fffffffLL) return fail(MP_DD_ERR_TOO_LARGE, "m x n too large");
     const dim3 grid((unsigned)tiles);
-    if (p.ta == 0 && p.tb == 0) launch_one<0, 0, R>(grid, p, stream);
-    else if (p.ta == 1 && p.tb == 0) launch_one<1, 0, R>(grid, p, stream);
-    else if (p.ta == 0 && p.tb == 1) launch_one<0, 1, R>(grid, p, stream);
-    else launch_one<1, 1, R>(grid, p, stream);
+    if (p.ta == 0 && p.tb == 0) launch_one<0, 0, S>(grid, p, stream);
+    else if (p.ta == 1 && p.tb == 0) launch_one<1, 0, S>(grid, p, stream);
+    else if (p.ta == 0 && p.tb == 1) launch_one<0, 1, S>(grid, p, stream);
+    else launch_one<1, 1, S>(grid, p, stream);
     return check_launch("dd_gemm_plain_kernel");
 }
 
 }  // namespace
 
 // Tile size: the time of a launch is about (tiles per SM, rounded up) x
-// (work per tile), i.e. ceil(tiles_R / SMs) R^2 in units of a 16 x 16 tile;
-// the largest R with the least such time wins (the per-entry operation
-// sequence, and hence the result, does not depend on R).
+// (work per tile), in units of 128 entries -- one accumulator for each of four
+// warps, one per partition of the SM, 0.36 us per step of k (9.75 FP64
+// instructions per multiply-add at 526 G/s over 152 SMs); the largest tile
+// with the least such time wins (the per-entry operation sequence, and hence
+// the result, does not depend on it).  16 x 8 and 32 x 4 tiles are one unit:
+// they halve the time of products with fewer 16 x 16 tiles than SMs, and of
+// those with few columns, whose 16-column tiles are mostly padding: Rgemm 96 x
+// 80 x 70 58.0 -> 31.9 us; Cholesky and solve of order 3000, whose updates
+// have a depth of 64, 36.5 -> 33.2 ms.
 int64_t plain_tile_cost(const GemmArgs &p, int r) {
     const int64_t sms = sm_count() > 0 ? sm_count() : 152;
-    return ceil_div(tile_count(p, 16 * r), sms) * r * r;
+    return ceil_div(tile_count(p, 16 * r, 16 * r), sms) * 2 * r * r;
 }
 
-int plain_tile_r(const GemmArgs &p) {
-    int best = 4;
-    int64_t best_t = -1;
-    for (int r = 4; r >= 1; r /= 2) {
-        const int64_t t = plain_tile_cost(p, r);
-        if (best_t < 0 || t < best_t) { best_t = t; best = r; }
-    }
+namespace {
+
+enum PlainTile { kTile64, kTile32, kTile16, kTileHalf, kTileTall };
+
+PlainTile plain_tile(const GemmArgs &p, int64_t *cost) {
+    const int64_t sms = sm_count() > 0 ? sm_count() : 152;
+    PlainTile best = kTile64;
+    *cost = plain_tile_cost(p, 4);
+    auto offer = [&](PlainTile t, int64_t c) {
+        if (c < *cost) {
+            *cost = c;
+            best = t;
+        }
+    };
+    offer(kTile32, plain_tile_cost(p, 2));
+    offer(kTile16, plain_tile_cost(p, 1));
+    offer(kTileHalf, ceil_div(tile_count(p, Half::BM, Half::BN), sms));
+    if (p.tri == 0) offer(kTileTall, ceil_div(tile_count(p, Tall::BM, Tall::BN), sms));
     return best;
+}
+
+}  // namespace
+
+int64_t plain_best_cost(const GemmArgs &p) {
+    int64_t cost;
+    plain_tile(p, &cost);
+    return cost;
 }
 
 // The plain kernel behind a split-precision call: the same launch, gated on
@@ -285,15 +335,13 @@ int launch_plain_fallback(const GemmArgs &p, const SplitPlan &plan, cudaStream_t
     int rc = 0;
     if (try_launch_gemm_tma(q, stream, &rc)) return rc;
     const int64_t sms = sm_count() > 0 ? sm_count() : 152;
-    if (tile_count(q, 64) >= 2 * sms) return launch_r<4>(q, stream);
+    if (tile_count(q, 64, 64) >= 2 * sms) return launch_shape<Square<4>>(q, stream);
     return launch_gemm_plain(q, stream);
 }
 
 // Where the residue form takes an update of a factorisation or solve over
-// from the plain kernel.  The plain kernel's time is its busiest SM's: 0.72 us
-// per step of k and 16 x 16 tile (9.75 FP64 instructions per multiply-add at
-// 526 G/s over 152 SMs); the residue form must be estimated at four fifths of
-// it.  LU and solve of order 1536 with 500 right-hand sides: 71.0 ms with every
+// from the plain kernel: where its estimated time is at most four fifths of
+// the plain kernel's busiest SM's (plain_tile_cost).  LU and solve of order 1536 with 500 right-hand sides: 71.0 ms with every
 // update on the FP64 pipe, 31.9 so.
 // The inner dimension and both outer ones have to reach kUpdateMin: below it
 // the time is latency either way, and a solve's or a factorisation's result
@@ -311,7 +359,7 @@ int launch_gemm_update(const GemmArgs &p, cudaStream_t stream) {
     if (p.m < kUpdateMin || p.n < kUpdateMin || p.k < kUpdateMin || p.k > ((int64_t)1 << 17) - 1 ||
         p.tri != 0 || p.alpha_zero || p.a2h != nullptr || p.sym_a || p.sym_b)
         return launch_gemm_plain(p, stream);
-    const double plain_us = 0.72 * (double)p.k * (double)plain_tile_cost(p, plain_tile_r(p));
+    const double plain_us = 0.36 * (double)p.k * (double)plain_best_cost(p);
     if (crt_estimate_us(p.m, p.n, p.k) > 0.8 * plain_us) return launch_gemm_plain(p, stream);
     // allocations inside a stream capture would belong to the graph
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -352,10 +400,13 @@ int launch_gemm_update(const GemmArgs &p, cudaStream_t stream) {
 int launch_gemm_plain(const GemmArgs &p, cudaStream_t stream) {
     int rc = 0;
     if (try_launch_gemm_tma(p, stream, &rc)) return rc;
-    switch (plain_tile_r(p)) {
-        case 1: return launch_r<1>(p, stream);
-        case 2: return launch_r<2>(p, stream);
-        default: return launch_r<4>(p, stream);
+    int64_t cost;
+    switch (plain_tile(p, &cost)) {
+        case kTileTall: return launch_shape<Tall>(p, stream);
+        case kTileHalf: return launch_shape<Half>(p, stream);
+        case kTile16: return launch_shape<Square<1>>(p, stream);
+        case kTile32: return launch_shape<Square<2>>(p, stream);
+        default: return launch_shape<Square<4>>(p, stream);
     }
 }
 

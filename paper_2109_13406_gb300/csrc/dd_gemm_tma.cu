@@ -341,11 +341,7 @@ int try_launch_gemm_tma(const GemmArgs &p, cudaStream_t st, int *rc) {
         // best tile size's busiest-SM time (thinner products and the Rsyrk
         // triangle run faster on the smaller register-staged tiles)
         if (p.tri != 0 || tiles < sms) return 0;
-        int64_t best = plain_tile_cost(p, 4);
-        for (int r = 2; r >= 1; r /= 2) {
-            const int64_t c = plain_tile_cost(p, r);
-            best = c < best ? c : best;
-        }
+        const int64_t best = plain_best_cost(p);
         if (100 * plain_tile_cost(p, 4) > 101 * best) return 0;
     }
     if (p.k > ((int64_t)1 << 31) - 1 || p.m > ((int64_t)1 << 31) - 1 ||

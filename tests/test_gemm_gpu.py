@@ -190,3 +190,38 @@ def test_ddmac_peak_is_positive(cuda_lib):
     FP64 issue rate divided by the 12 FP64 instructions it needs at least."""
     r = cuda_lib.mp_dd_peak_ddmac()
     assert 1e9 < r < cuda_lib.mp_dd_peak_fp64() / 10
+
+
+@pytest.mark.parametrize("ta,tb", [("N", "N"), ("T", "N"), ("N", "T"), ("T", "T")])
+@pytest.mark.parametrize("shape", [(1, 1), (16, 8), (17, 9), (95, 81), (33, 5), (32, 4), (700, 3),
+                                   (3, 700)])
+def test_small_tiles_give_the_same_bits(cuda_lib, ta, tb, shape):
+    """Products on 16 x 8 and 32 x 4 tiles (few tiles, few columns) equal the
+    leading block of a product on large tiles."""
+    M, N, k = 1300, 1100, 37
+    c = datagen.gemm_case(130 + ["NN", "TN", "NT", "TT"].index(ta + tb), ta, tb, M, N, k, pad=1)
+    whole = run_gemm(c)
+    m, n = shape
+    part = datagen.GemmCase(ta, tb, m, n, k, c.alpha, c.A, c.B, c.beta, c.C)
+    got = run_gemm(part)
+    for t in range(2):
+        assert np.array_equal(got[t], whole[t][:m, :n])
+
+
+@pytest.mark.parametrize("uplo", ["U", "L"])
+@pytest.mark.parametrize("n", [1, 16, 17, 90, 150])
+def test_small_triangles_give_the_same_bits(cuda_lib, uplo, n):
+    """The triangle on 16 x 8 tiles equals the full product's, and the other
+    triangle keeps its entries."""
+    k = 29
+    c = datagen.gemm_case(140 + n, "N", "T", n, n, k, alpha=(1.0, 0.0), beta=(1.0, 0.0))
+    c.B = c.A
+    full = run_gemm(c)
+    A, C = dev(c.A), dev(c.C)
+    cuda_lib.mp_dd_Rsyrk(uplo, "N", n, k, (1.0, 0.0), A, n, (1.0, 0.0), C, n)
+    got = host(C, n, n)
+    tri = np.triu if uplo == "U" else np.tril
+    other = (lambda x: np.tril(x, -1)) if uplo == "U" else (lambda x: np.triu(x, 1))
+    for t in range(2):
+        assert np.array_equal(tri(got[t]), tri(full[t]))
+        assert np.array_equal(other(got[t]), other(c.C[t]))
