@@ -179,16 +179,35 @@ __device__ __forceinline__ dd div(dd a, dd b) {
     return q;
 }
 
+// The exponent field of x lies in [128, 1918]: products, quotients and
+// remainders of such numbers with 2^-53-sized factors stay normal.
+__device__ __forceinline__ bool mid_range(double x) {
+    return (((unsigned int)__double2hiint(x) >> 20) & 0x7FFu) - 128u <= 1790u;
+}
+
+// a / b for binary64 numbers from y, an approximation of 1 / b within a few
+// ulps: q0 = RN(a y) is within a few ulps of a / b, and the remainder a - q0 b
+// (one FMA) times y corrects it, so the result is a / b rounded once, but for
+// near-ties, and a / b itself whenever that is a binary64 number (Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990).  Three FP64 instructions on the dependent chain, where
+// the division takes as long as nine (576 cycles of a warp).  Operands near
+// the ends of the exponent range, zeros and non-finite ones are divided.
+__device__ __forceinline__ double quotient(double a, double b, double y) {
+    if (!(mid_range(a) && mid_range(b))) return __ddiv_rn(a, b);
+    const double q = __dmul_rn(a, y);
+    return __fma_rn(__fma_rn(-q, b, a), y, q);
+}
+
 // dd division with a given approximate reciprocal y of b.hi (within a few
-// ulps): div's long division with the second quotient digit taken as
-// remainder * y instead of a second binary64 division, so the dependent
-// chain holds one division.  The second digit's extra relative error (a few
-// u) is scaled by |q2| <= ~3u |a / b|: the result's relative error stays
+// ulps): div's long division with both quotient digits taken by y, so the
+// dependent chain holds no division.  The second digit's extra relative error
+// (a few u) is scaled by |q2| <= ~3u |a / b|: the result's relative error stays
 // at most ~20 u^2, and an exactly representable quotient of binary64
 // operands is still exact (its remainder is 0).  a need not be
 // renormalised: |a.lo| may be a few ulps of a.hi.
 __device__ __forceinline__ dd div_rcp(dd a, dd b, double y) {
-    const double q1 = __ddiv_rn(a.hi, b.hi);
+    const double q1 = quotient(a.hi, b.hi, y);
     double r = __fma_rn(-q1, b.hi, a.hi);
     r = __dadd_rn(r, __fma_rn(-q1, b.lo, a.lo));
     const double q2 = __dmul_rn(r, y);
@@ -209,23 +228,32 @@ __device__ __forceinline__ dd rcp_dd(dd b) {
     return q;
 }
 
-// dd square root: x = RN(sqrt(a.hi)), whose remainder a.hi - x^2 is a
+// dd square root: x = sqrt(a.hi) rounded, whose remainder a.hi - x^2 is a
 // binary64 number (one FMA gives it exactly), plus one Newton correction
 // (a - x^2) / (2x) with a.lo added, the division taken as a product with
 // z = rsqrt(a.hi) (1 ulp); the neglected second-order term is below u^2 / 8
-// relative.  Exact when a.hi is the square of a binary64 number and a.lo =
-// 0.  z, an approximate reciprocal of the result's leading part within a
-// few ulps, is returned for div_rcp.  a need not be renormalised.  Returns
-// 0 (and z = 0) for a <= 0.
+// relative.  x is x0 = RN(a.hi z) corrected once by its own remainder,
+// x0 + (a.hi - x0^2) z / 2: sqrt(a.hi) rounded once but for near-ties, and the
+// root itself when that is a binary64 number (the same method as quotient);
+// near the ends of the exponent range the square root is taken.  Exact when
+// a.hi is the square of a binary64 number and a.lo = 0.  z, an approximate
+// reciprocal of the result's leading part within a few ulps, is returned for
+// div_rcp.  a need not be renormalised.  Returns 0 (and z = 0) for a <= 0.
 __device__ __forceinline__ dd sqrt_dd(dd a, double &z) {
     z = 0.0;
     if (!(a.hi > 0.0)) return dd{0.0, 0.0};
-    const double x = __dsqrt_rn(a.hi);
     z = rsqrt(a.hi);
+    const double hz = __dmul_rn(z, 0.5);
+    double x;
+    if (mid_range(a.hi)) {
+        const double x0 = __dmul_rn(a.hi, z);
+        x = __fma_rn(__fma_rn(-x0, x0, a.hi), hz, x0);
+    } else {
+        x = __dsqrt_rn(a.hi);
+    }
     const double r = __dadd_rn(__fma_rn(-x, x, a.hi), a.lo);
-    const double corr = __dmul_rn(__dmul_rn(r, z), 0.5);
     dd s;
-    fast_two_sum(x, corr, s.hi, s.lo);
+    fast_two_sum(x, __dmul_rn(r, hz), s.hi, s.lo);
     return s;
 }
 

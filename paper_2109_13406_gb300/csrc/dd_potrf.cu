@@ -8,7 +8,7 @@
 //
 //  * diag:  unblocked Cholesky of one nb x nb diagonal block (nb <= 64), in
 //           registers, on a cluster of up to 8 CTAs per block;
-//  * trsm:  triangular solve with one nb x nb factor block for 4 to 32
+//  * trsm:  triangular solve with one nb x nb factor block for 2 to 32
 //           right-hand-side columns per CTA (forward with U^T, backward
 //           with U), optionally scaling the right-hand sides by alpha and
 //           taking the diagonal as unit;
@@ -285,18 +285,18 @@ struct TrsmScale {
 
 __device__ __forceinline__ int col_start(int c) { return (c * (c + 1)) / 2; }
 
-// Shared memory of one solve CTA with RG row groups: U's triangle packed
-// (hi, lo) and the solved rows x_i of its NT / RG columns.
-__host__ __device__ constexpr size_t trsm_smem_bytes(int rg) {
-    return sizeof(double) * (2 * (size_t)kTri + 2 * (size_t)NB * (NT / rg) + NB);
+// Shared memory of one solve CTA of `cols` columns: U's triangle packed
+// (hi, lo) and the solved rows x_i.
+__host__ __device__ constexpr size_t trsm_smem_bytes(int cols) {
+    return sizeof(double) * (2 * (size_t)kTri + 2 * (size_t)NB * cols + NB);
 }
 
 // Solve U^T X = B (trans = 1) or U X = B (trans = 0) for the columns
-// [c0, c0 + NT / RG) of B, in place.  U is the n x n upper factor block;
+// [c0, c0 + THR / RG) of B, in place.  U is the n x n upper factor block;
 // with d.unit_diag its diagonal is taken as one and never read.
 //
-// Thread t owns column t % (NT / RG) and the rows t / (NT / RG) + RG q (q <
-// 64 / RG) as dd accumulators in registers.  Step i: the owner of row i
+// Thread t of THR owns column t % (THR / RG) and the rows t / (THR / RG) + RG q
+// (q < 64 / RG) as dd accumulators in registers.  Step i: the owner of row i
 // finishes x_i (its accumulator, divided by U(i, i)) and publishes it in
 // shared memory; after one barrier every thread subtracts U-entry x_i from
 // its rows still to be solved, with the deferred renormalisation of the GEMM
@@ -304,11 +304,16 @@ __host__ __device__ constexpr size_t trsm_smem_bytes(int rg) {
 // triangle sits in shared memory packed in the order the steps read it: by
 // rows for U^T (step i reads U(i, i+1:)), by columns for U (step i reads
 // U(:i-1, i)).  Every row takes the same operations in the same order
-// whatever RG is, so the result does not depend on it: RG only trades
-// columns per CTA (32, 16, 8, 4) against the number of CTAs.
-template <int TRANS, int RG>
+// whatever RG and THR are, so the result does not depend on them: they only
+// trade columns per CTA (32, 16, 8, 4, 2) against the number of CTAs.
+//
+// What bounds a row: the owner's division (10 dependent FP64 instructions of
+// ~64 cycles), the barrier, and every warp's multiply-add (9.75 more, twice
+// that where two warps share a partition of the SM, as in the first half of a
+// solve with four columns; with two columns each partition has one).
+template <int TRANS, int RG, int THR>
 __device__ void trsm_one(const mp_dd_trsm_desc &d, int64_t c0, double *sm, TrsmScale sc) {
-    constexpr int COLS = NT / RG, RPT = NB / RG;
+    constexpr int COLS = THR / RG, RPT = NB / RG;
     double *uh = sm, *ul = sm + kTri, *xh = sm + 2 * kTri, *xl = xh + NB * COLS;
     double *rcp = xl + NB * COLS;   // 1 / U(i, i).hi
     const int n = d.n < NB ? (int)d.n : NB;   // (n > 64 is taken as 64)
@@ -319,14 +324,30 @@ __device__ void trsm_one(const mp_dd_trsm_desc &d, int64_t c0, double *sm, TrsmS
     const int unit = d.unit_diag != 0;
     const int col = tid % COLS, rg = tid / COLS;
     const bool col_ok = col < ncol;
-    for (int e = tid; e < n * n; e += NT) {
-        const int r = e % n, c = e / n;
-        if (r < c || (r == c && !unit)) {
+    // U's triangle: eight entries of a thread in flight at a time, along the
+    // direction that is contiguous in memory
+    constexpr int kFly = 8;
+    for (int e0 = tid; e0 < NB * NB; e0 += kFly * THR) {
+        double vh[kFly], vl[kFly];
+#pragma unroll
+        for (int f = 0; f < kFly; ++f) {
+            const int e = e0 + f * THR, x = e % NB, y = e / NB;
+            const int r = d.lower_u ? y : x, c = d.lower_u ? x : y;
+            const bool ok = c < n && (r < c || (r == c && !unit));
             const int64_t o = uidx(d.lower_u, r, c, d.ldu);
-            const int k = TRANS ? tri_start(r) + (c - r) : col_start(c) + r;
-            uh[k] = d.u_hi[o];
-            ul[k] = d.u_lo[o];
-            if (r == c) rcp[r] = __drcp_rn(d.u_hi[o]);
+            vh[f] = ok ? __ldg(d.u_hi + o) : 0.0;
+            vl[f] = ok ? __ldg(d.u_lo + o) : 0.0;
+        }
+#pragma unroll
+        for (int f = 0; f < kFly; ++f) {
+            const int e = e0 + f * THR, x = e % NB, y = e / NB;
+            const int r = d.lower_u ? y : x, c = d.lower_u ? x : y;
+            if (c < n && (r < c || (r == c && !unit))) {
+                const int k = TRANS ? tri_start(r) + (c - r) : col_start(c) + r;
+                uh[k] = vh[f];
+                ul[k] = vl[f];
+                if (r == c) rcp[r] = __drcp_rn(vh[f]);
+            }
         }
     }
     dd acc[RPT];
@@ -398,46 +419,50 @@ __device__ void trsm_one(const mp_dd_trsm_desc &d, int64_t c0, double *sm, TrsmS
     }
 }
 
-template <int RG>
+template <int RG, int THR>
 __device__ __forceinline__ void trsm_any(const mp_dd_trsm_desc &d, int64_t c0, double *sm,
                                          TrsmScale sc) {
     if (d.trans)
-        trsm_one<1, RG>(d, c0, sm, sc);
+        trsm_one<1, RG, THR>(d, c0, sm, sc);
     else
-        trsm_one<0, RG>(d, c0, sm, sc);
+        trsm_one<0, RG, THR>(d, c0, sm, sc);
 }
 
-template <int RG>
-__global__ void __launch_bounds__(NT, 2) trsm_batch_kernel(const mp_dd_trsm_desc *ds) {
+template <int RG, int THR>
+__global__ void __launch_bounds__(THR, 2) trsm_batch_kernel(const mp_dd_trsm_desc *ds) {
     extern __shared__ double smem_t[];
-    trsm_any<RG>(ds[blockIdx.x], (int64_t)blockIdx.y * (NT / RG), smem_t,
-                 TrsmScale{dd{1.0, 0.0}, 0});
+    trsm_any<RG, THR>(ds[blockIdx.x], (int64_t)blockIdx.y * (THR / RG), smem_t,
+                      TrsmScale{dd{1.0, 0.0}, 0});
 }
 
-template <int RG>
-__global__ void __launch_bounds__(NT, 2) trsm_single_kernel(const mp_dd_trsm_desc d,
-                                                         TrsmScale sc) {
+template <int RG, int THR>
+__global__ void __launch_bounds__(THR, 2) trsm_single_kernel(const mp_dd_trsm_desc d,
+                                                             TrsmScale sc) {
     extern __shared__ double smem_t[];
-    trsm_any<RG>(d, (int64_t)blockIdx.y * (NT / RG), smem_t, sc);
+    trsm_any<RG, THR>(d, (int64_t)blockIdx.y * (THR / RG), smem_t, sc);
 }
 
 constexpr TrsmScale kNoScale{dd{1.0, 0.0}, 0};
 
-// Row groups for count solves of nrhs columns.  Measured on GB300 (one
+// Columns per CTA for count solves of nrhs columns.  Measured on GB300 (one
 // 64-row solve of many columns; microseconds for an SM holding k resident
 // CTAs of each width): a wide CTA (32 columns) makes the best use of the
 // FP64 pipe once every SM has two of them, narrow ones win while the
 // columns are too few to fill the SMs.  The cost of a choice is the busiest
 // SM's: ceil(CTAs / SMs) CTAs in waves of the kernel's occupancy.  The
-// cheapest is taken, or a wider one within 5 % of it.
-constexpr int kRgCount = 4;                 // rg = 8, 16, 32, 64
+// cheapest is taken, or a wider one within 5 % of it.  (With the division
+// instruction and the triangle loaded one entry at a time, 32, 16, 8 and 4
+// columns took 318, 199, 133 and 109 us alone on an SM.)
+constexpr int kRgCount = 5;
+constexpr int kSolveCols[kRgCount] = {32, 16, 8, 4, 2};
 constexpr float kSolveUs[kRgCount][5] = {
-    {318.f, 552.f, 552.f, 552.f, 552.f},    // 32 columns per CTA (2 resident)
-    {199.f, 311.f, 442.f, 442.f, 442.f},    // 16 (3 resident)
-    {133.f, 186.f, 253.f, 330.f, 330.f},    //  8 (4 resident)
-    {109.f, 147.f, 195.f, 244.f, 300.f},    //  4 (5 resident)
+    {249.f, 431.f, 431.f, 431.f, 431.f},    // 32 columns per CTA (2 resident)
+    {154.f, 245.f, 465.f, 465.f, 465.f},    // 16 (2 resident)
+    {104.f, 144.f, 269.f, 269.f, 269.f},    //  8 (2 resident)
+    {88.f, 120.f, 203.f, 221.f, 304.f},     //  4 (4 resident)
+    {78.f, 90.f, 111.f, 133.f, 164.f},      //  2 (5 resident)
 };
-int g_trsm_occ[kRgCount] = {0, 0, 0, 0};    // resident CTAs per SM (0: not queried)
+int g_trsm_occ[kRgCount] = {0, 0, 0, 0, 0};    // resident CTAs per SM (0: not queried)
 
 float trsm_cost(int idx, int64_t per_sm) {
     int occ = g_trsm_occ[idx];
@@ -447,37 +472,41 @@ float trsm_cost(int idx, int64_t per_sm) {
     return (float)full * kSolveUs[idx][occ - 1] + (rem ? kSolveUs[idx][rem - 1] : 0.f);
 }
 
-int trsm_row_groups(int64_t count, int64_t nrhs) {
+int trsm_config(int64_t count, int64_t nrhs) {
     const int64_t sms = sm_count() > 0 ? sm_count() : 152;
     float cost[kRgCount];
     int cheapest = 0;
     for (int idx = 0; idx < kRgCount; ++idx) {
-        const int64_t cols = NT / (8 << idx);
-        cost[idx] = trsm_cost(idx, ceil_div(count * ceil_div(nrhs, cols), sms));
+        cost[idx] = trsm_cost(idx, ceil_div(count * ceil_div(nrhs, (int64_t)kSolveCols[idx]), sms));
+        if (ceil_div(nrhs, (int64_t)kSolveCols[idx]) > 65535) cost[idx] = 1e30f;   // grid.y
         if (cost[idx] < cost[cheapest]) cheapest = idx;
     }
     for (int idx = 0; idx < cheapest; ++idx)      // wider, nearly as cheap
-        if (cost[idx] <= 1.05f * cost[cheapest]) return 8 << idx;
-    return 8 << cheapest;
+        if (cost[idx] <= 1.05f * cost[cheapest]) return idx;
+    return cheapest;
 }
 
 // One launch of count solves (ds on the device) or of the single solve d.
 int launch_trsm(const mp_dd_trsm_desc *ds, int64_t count, const mp_dd_trsm_desc &d,
                 TrsmScale sc, int64_t nrhs, cudaStream_t st) {
-    const int rg = trsm_row_groups(ds != nullptr ? count : 1, nrhs);
-    const int64_t gy = ceil_div(nrhs, NT / rg);
+    const int idx = trsm_config(ds != nullptr ? count : 1, nrhs);
+    const int64_t gy = ceil_div(nrhs, (int64_t)kSolveCols[idx]);
     if (gy > 65535) return fail(MP_DD_ERR_TOO_LARGE, "too many right-hand sides");
     const dim3 grid(ds != nullptr ? (unsigned)count : 1u, (unsigned)gy);
-    const size_t sm = trsm_smem_bytes(rg);
-    switch (rg) {
-#define MPDD_TRSM_CASE(RG)                                                  \
-    case RG:                                                                \
+    const size_t sm = trsm_smem_bytes(kSolveCols[idx]);
+    switch (idx) {
+#define MPDD_TRSM_CASE(IDX, RG, THR)                                        \
+    case IDX:                                                               \
         if (ds != nullptr)                                                  \
-            trsm_batch_kernel<RG><<<grid, NT, sm, st>>>(ds);                \
+            trsm_batch_kernel<RG, THR><<<grid, THR, sm, st>>>(ds);          \
         else                                                                \
-            trsm_single_kernel<RG><<<grid, NT, sm, st>>>(d, sc);            \
+            trsm_single_kernel<RG, THR><<<grid, THR, sm, st>>>(d, sc);      \
         break;
-        MPDD_TRSM_CASE(8) MPDD_TRSM_CASE(16) MPDD_TRSM_CASE(32) MPDD_TRSM_CASE(64)
+        MPDD_TRSM_CASE(0, 8, 256)
+        MPDD_TRSM_CASE(1, 16, 256)
+        MPDD_TRSM_CASE(2, 32, 256)
+        MPDD_TRSM_CASE(3, 64, 256)
+        MPDD_TRSM_CASE(4, 64, 128)
 #undef MPDD_TRSM_CASE
     }
     return check_launch(ds != nullptr ? "trsm_batch_kernel" : "trsm_single_kernel");
@@ -489,33 +518,28 @@ int launch_trsm_single(const mp_dd_trsm_desc &d, TrsmScale sc, cudaStream_t st) 
 
 bool g_attr_done = false;
 
-template <int RG>
-cudaError_t trsm_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(trsm_batch_kernel<RG>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)trsm_smem_bytes(RG));
+template <int RG, int THR>
+cudaError_t trsm_attrs(int idx) {
+    const int sm = (int)trsm_smem_bytes(THR / RG);
+    cudaError_t e = cudaFuncSetAttribute(trsm_batch_kernel<RG, THR>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(trsm_single_kernel<RG>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)trsm_smem_bytes(RG));
+        e = cudaFuncSetAttribute(trsm_single_kernel<RG, THR>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_trsm_occ[idx],
+                                                          trsm_batch_kernel<RG, THR>, THR, sm);
     return e;
 }
 
 int set_attrs() {
     if (g_attr_done) return 0;
-    cudaError_t e = trsm_attrs<8>();
-    if (e == cudaSuccess) e = trsm_attrs<16>();
-    if (e == cudaSuccess) e = trsm_attrs<32>();
-    if (e == cudaSuccess) e = trsm_attrs<64>();
+    cudaError_t e = trsm_attrs<8, 256>(0);
+    if (e == cudaSuccess) e = trsm_attrs<16, 256>(1);
+    if (e == cudaSuccess) e = trsm_attrs<32, 256>(2);
+    if (e == cudaSuccess) e = trsm_attrs<64, 256>(3);
+    if (e == cudaSuccess) e = trsm_attrs<64, 128>(4);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(potrf kernels)");
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_trsm_occ[0], trsm_batch_kernel<8>, NT,
-                                                  trsm_smem_bytes(8));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_trsm_occ[1], trsm_batch_kernel<16>, NT,
-                                                  trsm_smem_bytes(16));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_trsm_occ[2], trsm_batch_kernel<32>, NT,
-                                                  trsm_smem_bytes(32));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_trsm_occ[3], trsm_batch_kernel<64>, NT,
-                                                  trsm_smem_bytes(64));
     g_attr_done = true;
     return 0;
 }

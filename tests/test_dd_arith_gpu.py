@@ -125,3 +125,34 @@ def test_errors(cuda_lib):
     assert mp.mp_dd_elementwise("sqrt", 4, x, None, (None, None), check=False) == -5
     assert mp.mp_dd_elementwise("sqrt", 4, x, None, z, check=False) == 0
     assert mp.mp_dd_elementwise("add", 0, x, x, z, check=False) == 0
+
+
+@pytest.mark.parametrize("ea,eb", [(0, 0), (-835, -100), (880, 0), (860, 100), (100, 860),
+                                   (-860, -150), (-150, -860), (0, 830)])
+def test_division_and_root_over_the_exponent_range(cuda_lib, ea, eb):
+    """div_rcp takes its first digit by the reciprocal inside the middle of
+    the exponent range and divides outside it (sqrt_dd likewise): the bounds
+    hold on both sides of the limits, and quotients and roots that are
+    binary64 numbers come out exact."""
+    n = 400
+    g = datagen.rng(910)
+    x, y = operands(911, n), operands(912, n)
+    x, y = (tuple(v * 2.0 ** e for v in p) for p, e in ((x, ea), (y, eb)))
+    zh, zl = run(cuda_lib, "divr", x, y)
+    for i in range(n):
+        ex = exact("divr", x[0][i], x[1][i], y[0][i], y[1][i])
+        got = Fraction(float(zh[i])) + Fraction(float(zl[i]))
+        assert abs(got - ex) <= Fraction(BOUND["divr"]) * abs(ex)
+    q = g.integers(1, 2 ** 26, n).astype(np.float64)
+    b = g.integers(1, 2 ** 26, n).astype(np.float64) * 2.0 ** eb
+    z0 = np.zeros(n)
+    zh, zl = run(cuda_lib, "divr", (q * 2.0 ** (ea - 60) * b, z0), (b, z0)) if abs(ea + eb) < 900 \
+        else (q * 2.0 ** (ea - 60), z0)
+    assert np.array_equal(zh, q * 2.0 ** (ea - 60)) and not zl.any()
+    s = (np.abs(x[0]), np.where(x[0] < 0, -x[1], x[1]))
+    zh, zl = run(cuda_lib, "sqrt", s)
+    worst = max(rel_err_sqrt(zh[i], zl[i], s[0][i], s[1][i]) for i in range(n))
+    assert worst / 2 <= BOUND["sqrt"]
+    r = q * 2.0 ** (ea // 2)
+    zh, zl = run(cuda_lib, "sqrt", (r * r, z0))
+    assert np.array_equal(zh, r) and not zl.any()
