@@ -25,6 +25,8 @@
 // untouched.
 #include <cooperative_groups.h>
 
+#include <cstddef>
+
 #include "common.cuh"
 #include "dd_arith.cuh"
 #include "kernels.cuh"
@@ -895,18 +897,22 @@ namespace {
 
 constexpr int LT = 256;   // threads of the pivot-column kernel
 
-// Pivot candidates: |x| of a normalised dd x orders by |hi| first (compared
-// as the integer bit pattern, off the FP64 pipe), then by lo taken with the
-// sign of hi; ties go to the lower row (the first maximum, as idamax).
+// Pivot candidates: |x| of a normalised dd x orders by |hi| first, then by lo
+// taken with the sign of hi; ties go to the lower row (the first maximum, as
+// idamax).  Both parts are kept as integers in the numbers' order: an FP64
+// comparison takes its partition of the SM as long as 38 integer instructions,
+// and a warp's search makes twenty of them.
 struct PivotKey {
     uint64_t mag;   // |hi| bits
-    double lo;      // lo * sign(hi)
+    uint64_t lo;    // lo * sign(hi), as an unsigned integer in its order
     int64_t row;    // -1: none
 };
 
 __device__ __forceinline__ PivotKey pivot_key(double hi, double lo, int64_t row) {
-    const uint64_t b = (uint64_t)__double_as_longlong(hi);
-    return PivotKey{b & 0x7fffffffffffffffull, (b >> 63) ? -lo : lo, row};
+    const uint64_t b = (uint64_t)__double_as_longlong(hi), sign = 1ull << 63;
+    uint64_t l = (uint64_t)__double_as_longlong(lo) ^ (b & sign);
+    if ((l << 1) == 0) l = 0;   // -0 is 0
+    return PivotKey{b & ~sign, (l & sign) ? ~l : l | sign, row};
 }
 
 // b is the better pivot than a
@@ -928,7 +934,7 @@ __global__ void __launch_bounds__(LT) getrf_pivot_kernel(double *ah, double *al,
                                                          int64_t *info) {
     __shared__ PivotKey wk[LT / 32];
     double *ch = ah + j * lda, *cl = al + j * lda;
-    PivotKey best{0, 0.0, -1};
+    PivotKey best{0, 0, -1};
     for (int64_t i = j + threadIdx.x; i < m; i += LT) {
         const PivotKey c = pivot_key(ch[i], cl[i], i);
         if (better(c, best)) best = c;
@@ -1007,36 +1013,44 @@ __global__ void __launch_bounds__(256) laswp_perm_kernel(double *ah, double *al,
                                                          int64_t c_skip, int64_t n_skip,
                                                          int64_t n_all, const int64_t *ipiv,
                                                          int64_t k0, int64_t k1, int reverse) {
+    // position t < 32: row k0 + t; position 32 + e: the e-th other row
     __shared__ int64_t S[64], src[64];
-    __shared__ int ns;
-    if (threadIdx.x == 0) {
-        const int nk = (int)(k1 - k0);
-        int cnt = nk;
-        for (int t = 0; t < nk; ++t) S[t] = src[t] = k0 + t;
+    if (threadIdx.x < 32) {
+        const int lane = (int)threadIdx.x, nk = (int)(k1 - k0);
+        const int64_t piv = lane < nk ? ipiv[k0 + lane] - 1 : -1;
+        int64_t own = k0 + lane, other = -1, from = own, from_other = -1;
+        int cnt = 0;
         for (int t = 0; t < nk; ++t) {
-            const int64_t p = ipiv[k0 + t] - 1;
-            int ip = -1;
+            const int64_t p = __shfl_sync(0xFFFFFFFFu, piv, t);
+            int ip;   // the position of row p
             if (p >= k0 && p < k1) {
                 ip = (int)(p - k0);
             } else {
-                for (int q = nk; q < cnt; ++q)
-                    if (S[q] == p) ip = q;
-                if (ip < 0) {
-                    ip = cnt++;
-                    S[ip] = src[ip] = p;
+                const unsigned hit = __ballot_sync(0xFFFFFFFFu, lane < cnt && other == p);
+                ip = 32 + (hit ? __ffs((int)hit) - 1 : cnt);
+                if (!hit) {
+                    if (lane == cnt) other = from_other = p;
+                    ++cnt;
                 }
             }
-            const int64_t tmp = src[t];
-            src[t] = src[ip];
-            src[ip] = tmp;
+            const int64_t a = __shfl_sync(0xFFFFFFFFu, from, t);
+            const int64_t b0 = __shfl_sync(0xFFFFFFFFu, from, ip & 31),
+                          b1 = __shfl_sync(0xFFFFFFFFu, from_other, ip & 31);
+            const int64_t b = ip < 32 ? b0 : b1;
+            if (ip < 32 && lane == ip) from = a;
+            if (ip >= 32 && lane == ip - 32) from_other = a;
+            if (lane == t) from = b;
         }
-        ns = cnt;
+        S[lane] = own;
+        src[lane] = lane < nk ? from : own;
+        S[32 + lane] = other;
+        src[32 + lane] = from_other;
     }
     __syncthreads();
     const int i = (int)(threadIdx.x % 64);
     const int64_t q = (int64_t)blockIdx.x * 4 + threadIdx.x / 64;
     const int64_t c = q < c_skip ? q : q + n_skip;
-    const bool act = i < ns && c < n_all && src[i] != S[i];
+    const bool act = c < n_all && src[i] != S[i];
     double vh = 0.0, vl = 0.0;
     if (act) {
         const int64_t from = (reverse ? S[i] : src[i]) + c * lda;
@@ -1092,8 +1106,7 @@ constexpr int kPanelMaxG = 256;
 constexpr int kPanelThreads = 256;
 
 struct PanelCand {
-    uint64_t mag;
-    double lo;
+    uint64_t mag, lo;
     int64_t row;                 // -1: no candidate in this CTA
     double rh, rl;               // dd reciprocal of the candidate
     double vh[kPanelW], vl[kPanelW];
@@ -1102,6 +1115,12 @@ struct PanelCand {
 struct PanelWs {
     unsigned int count;          // grid-barrier arrivals (zeroed before the launch)
     unsigned int abort;          // a wait gave up
+    // getrf_panel_smem_kernel: the column a CTA has published, plus one (zeroed
+    // before the launch), and its candidate's key, by the parity of the column
+    unsigned int seq[2][kPanelMaxG];
+    unsigned long long key_mag[2][kPanelMaxG];
+    unsigned long long key_lo[2][kPanelMaxG];
+    long long key_row[2][kPanelMaxG];
     double rjh[2][kPanelW], rjl[2][kPanelW];
     PanelCand cand[2][kPanelMaxG];
 };
@@ -1165,7 +1184,7 @@ __global__ void __launch_bounds__(kPanelThreads) getrf_panel_kernel(
         //    row j, by its owner.  The published buffers are written and
         //    read at L2, past L1: other CTAs write them between our reads.
         if (warp == 0) {
-            PivotKey best{0, 0.0, -1};
+            PivotKey best{0, 0, -1};
             int dummy = 0;
             for (int64_t i = (j > rs ? j : rs) + lane; i < re; i += 32) {
                 const PivotKey k = pivot_key(Ah[i + jj * lda], Al[i + jj * lda], i);
@@ -1191,7 +1210,8 @@ __global__ void __launch_bounds__(kPanelThreads) getrf_panel_kernel(
                 __stcg(&pc.rl, rl);
                 __stcg(reinterpret_cast<unsigned long long *>(&pc.mag),
                        (unsigned long long)best.mag);
-                __stcg(&pc.lo, best.lo);
+                __stcg(reinterpret_cast<unsigned long long *>(&pc.lo),
+                       (unsigned long long)best.lo);
                 __stcg(reinterpret_cast<long long *>(&pc.row), (long long)best.row);
             }
             __threadfence();
@@ -1212,13 +1232,14 @@ __global__ void __launch_bounds__(kPanelThreads) getrf_panel_kernel(
         // 2. warp 0: the pivot, the best published key (the same in every
         //    CTA), and the pivot row into shared memory; warp 1: row j
         if (warp == 0) {
-            PivotKey pk{0, 0.0, -1};
+            PivotKey pk{0, 0, -1};
             int win = 0;
             for (int q = lane; q < G; q += 32) {
                 const PanelCand &o = ws->cand[par][q];
                 const PivotKey k{
                     (uint64_t)__ldcg(reinterpret_cast<const unsigned long long *>(&o.mag)),
-                    __ldcg(&o.lo), (int64_t)__ldcg(reinterpret_cast<const long long *>(&o.row))};
+                    (uint64_t)__ldcg(reinterpret_cast<const unsigned long long *>(&o.lo)),
+                    (int64_t)__ldcg(reinterpret_cast<const long long *>(&o.row))};
                 if (better(k, pk)) {
                     pk = k;
                     win = q;
@@ -1294,6 +1315,249 @@ __global__ void __launch_bounds__(kPanelThreads) getrf_panel_kernel(
     // columns past the last pivot (a panel wider than its rows): nothing left
 }
 
+// getrf_panel_smem_kernel: the same panel factorisation, bit for bit, for CTAs
+// of at most kPanelRows rows, which they keep in shared memory.  A column's
+// critical path is: all CTAs' candidates seen (each polls the others' column
+// numbers; no counter that every CTA adds to), the winning key, its row;
+// multipliers and the update of the next column only, the search in it, the
+// update of the candidate's row and of row j + 1 in registers, publication.
+// The rest of the rank-1 update runs behind the publication, under the
+// other CTAs' latencies.  A CTA overwrites its published data of column j
+// at column j + 2, when every CTA has published column j + 1 and so has read
+// column j's.  Every wait is bounded (~2 s) and ends the factorisation with
+// info = -1.  A panel of 24 columns over 96 CTAs: 190 us with rows in global
+// memory, a grid barrier and the whole update before it, 152 so.
+constexpr int kPanelRows = 64;
+
+__device__ __forceinline__ unsigned int load_acquire(const unsigned int *p) {
+    unsigned int v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_release(unsigned int *p, unsigned int v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// Warps 0 .. 2 and 4 .. 6.
+__device__ __forceinline__ void publishers_sync() { asm volatile("bar.sync 1, 192;" ::: "memory"); }
+
+__global__ void __launch_bounds__(kPanelThreads) getrf_panel_smem_kernel(
+    double *ah, double *al, int64_t lda, int64_t m, int64_t j0, int w, int64_t R,
+    int64_t *ipiv, int64_t *info, PanelWs *ws) {
+    __shared__ double Sh[kPanelRows][kPanelW + 1], Sl[kPanelRows][kPanelW + 1];
+    __shared__ double lh[kPanelRows], ll[kPanelRows];
+    __shared__ double pvh[kPanelW], pvl[kPanelW];   // the pivot row
+    __shared__ double jvh[kPanelW], jvl[kPanelW];   // row j before the interchange
+    __shared__ int64_t s_p;
+    __shared__ double s_rh, s_rl;
+    __shared__ int s_stop, s_best;
+    const int G = (int)gridDim.x, c = (int)blockIdx.x, tid = (int)threadIdx.x;
+    const int lane = tid % 32, warp = tid / 32;
+    const int64_t rs = j0 + (int64_t)c * R;
+    const int nrow = (int)((rs + R < m ? rs + R : m) - rs);
+    const int mn = (int)((m - j0) < w ? (m - j0) : w);   // columns that take a pivot
+    double *Ah = ah + rs + j0 * lda, *Al = al + rs + j0 * lda;
+    for (int e = tid; e < nrow * w; e += kPanelThreads) {
+        const int r = e % nrow, q = e / nrow;
+        Sh[r][q] = Ah[r + q * lda];
+        Sl[r][q] = Al[r + q * lda];
+    }
+    if (tid == 0) s_stop = 0;
+    __syncthreads();
+    // Candidate of column jj and publication; update: the columns after jj of
+    // the published rows still lack step jj - 1 (multipliers lh, pivot row pv).
+    // All threads call it; it contains one block barrier, after which the
+    // caller may change the rows in shared memory.
+    auto publish = [&](int jj, bool update) {
+        const int64_t j = j0 + jj;
+        const int par = jj & 1;
+        const int jl = (int)(j - rs);              // local row of j
+        double vh = 0.0, vl = 0.0, l_h = 0.0, l_l = 0.0;
+        PivotKey best{0, 0, -1};
+        if (warp == 0) {
+            for (int r = lane; r < nrow; r += 32)
+                if (r >= jl) {
+                    const PivotKey k = pivot_key(Sh[r][jj], Sl[r][jj], rs + r);
+                    if (better(k, best)) best = k;
+                }
+            int dummy = 0;
+            warp_best(best, dummy);
+            const int b = best.row >= 0 ? (int)(best.row - rs) : -1;
+            if (lane == 0) s_best = b;
+            if (b >= 0 && lane < w) {
+                vh = Sh[b][lane];
+                vl = Sl[b][lane];
+                l_h = lh[b];
+                l_l = ll[b];
+            }
+        } else if (warp == 1 && jl >= 0 && jl < nrow && lane < w) {
+            vh = Sh[jl][lane];
+            vl = Sl[jl][lane];
+            l_h = lh[jl];
+            l_l = ll[jl];
+        }
+        __syncthreads();
+        if (warp == 3 || warp == 7) return;
+        if (warp < 2 && update && lane > jj && lane < w) {
+            dd v{vh, vl};
+            mac(v, dd{-l_h, -l_l}, dd{pvh[lane], pvl[lane]});
+            vh = v.hi;
+            vl = v.lo;
+        }
+        if (warp == 0) {
+            PanelCand &pc = ws->cand[par][c];
+            if (best.row >= 0 && lane < w) {
+                __stcg(&pc.vh[lane], vh);
+                __stcg(&pc.vl[lane], vl);
+            }
+            if (lane == 0) {
+                __stcg(&ws->key_mag[par][c], (unsigned long long)best.mag);
+                __stcg(&ws->key_lo[par][c], (unsigned long long)best.lo);
+                __stcg(&ws->key_row[par][c], (long long)best.row);
+            }
+        } else if (warp == 1) {
+            if (jl >= 0 && jl < nrow && lane < w) {
+                __stcg(&ws->rjh[par][lane], vh);
+                __stcg(&ws->rjl[par][lane], vl);
+            }
+        } else if (warp == 2) {                                   // the candidate's dd reciprocal
+            if (lane == 0) {
+                dd r{0.0, 0.0};
+                if (s_best >= 0) {
+                    const dd p{Sh[s_best][jj], Sl[s_best][jj]};
+                    if (fabs(p.hi) >= 0x1p-1021) r = rcp_dd(p);
+                }
+                __stcg(&ws->cand[par][c].rh, r.hi);
+                __stcg(&ws->cand[par][c].rl, r.lo);
+            }
+        }
+        // the release below covers what the CTA wrote before this barrier;
+        // warps 4 .. 6 wait at it too, as their work behind it would take the
+        // FP64 partitions of warps 0 .. 2 from the publication
+        publishers_sync();
+        if (tid == 0) store_release(&ws->seq[par][c], (unsigned)jj + 1u);
+    };
+    publish(0, false);
+    for (int jj = 0; jj < mn; ++jj) {
+        const int64_t j = j0 + jj;
+        const int par = jj & 1;
+        const int jl = (int)(j - rs);
+        // every CTA's candidate, the best of them (the same in every CTA), its
+        // row and row j
+        if (warp == 0) {
+            bool ok = true;
+            const long long t0 = clock64();
+            for (int q = lane; q < G && ok; q += 32)
+                while (load_acquire(&ws->seq[par][q]) != (unsigned)jj + 1u) {
+                    if (*reinterpret_cast<volatile unsigned int *>(&ws->abort)) ok = false;
+                    if (clock64() - t0 > 4000000000LL) {
+                        atomicExch(&ws->abort, 1u);
+                        ok = false;
+                    }
+                    if (!ok) break;
+                }
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            __syncwarp();   // (what the others published is read past L1)
+            if (!ok) {
+                if (lane == 0) s_stop = 1;
+            } else {
+                PivotKey pk{0, 0, -1};
+                int win = 0;
+                for (int q = lane; q < G; q += 32) {
+                    const PivotKey k{(uint64_t)__ldcg(&ws->key_mag[par][q]),
+                                     (uint64_t)__ldcg(&ws->key_lo[par][q]),
+                                     (int64_t)__ldcg(&ws->key_row[par][q])};
+                    if (better(k, pk)) {
+                        pk = k;
+                        win = q;
+                    }
+                }
+                warp_best(pk, win);
+                const PanelCand &wc = ws->cand[par][win];
+                if (lane < w) {
+                    pvh[lane] = __ldcg(&wc.vh[lane]);
+                    pvl[lane] = __ldcg(&wc.vl[lane]);
+                    jvh[lane] = __ldcg(&ws->rjh[par][lane]);
+                    jvl[lane] = __ldcg(&ws->rjl[par][lane]);
+                }
+                if (lane == 0) {
+                    s_p = pk.row;
+                    s_rh = __ldcg(&wc.rh);
+                    s_rl = __ldcg(&wc.rl);
+                }
+            }
+        }
+        __syncthreads();
+        if (s_stop) {
+            if (c == 0 && tid == 0) *info = -1;
+            return;
+        }
+        const int64_t p = s_p;               // >= j: every column has rows j .. m-1
+        const double ph = pvh[jj], pl = pvl[jj];
+        const bool zero = ph == 0.0 && pl == 0.0;
+        if (c == 0 && tid == 0) {
+            ipiv[j] = p + 1;
+            if (zero)
+                atomicCAS(reinterpret_cast<unsigned long long *>(info), 0ull,
+                          (unsigned long long)(j + 1));
+        }
+        const int r0 = jl + 1 > 0 ? jl + 1 : 0;   // first local row below j
+        const bool last = jj + 1 >= mn;
+        if (!zero) {
+            // the interchange: row j := the pivot row, row p := row j
+            if (p != j) {
+                const int pr = (int)(p - rs);
+                if (jl >= 0 && jl < nrow && tid < w) {
+                    Sh[jl][tid] = pvh[tid];
+                    Sl[jl][tid] = pvl[tid];
+                }
+                if (pr >= 0 && pr < nrow && tid >= 64 && tid < 64 + w) {
+                    Sh[pr][tid - 64] = jvh[tid - 64];
+                    Sl[pr][tid - 64] = jvl[tid - 64];
+                }
+                __syncthreads();
+            }
+            // multipliers, and the update of the next column
+            const bool recip = fabs(ph) >= 0x1p-1021;
+            const int r = r0 + tid;
+            if (r < nrow) {
+                const dd a{Sh[r][jj], Sl[r][jj]};
+                const dd l = recip ? mul(a, dd{s_rh, s_rl}) : div(a, dd{ph, pl});
+                lh[r] = l.hi;
+                ll[r] = l.lo;
+                Sh[r][jj] = l.hi;
+                Sl[r][jj] = l.lo;
+                if (jj + 1 < w) {
+                    dd v{Sh[r][jj + 1], Sl[r][jj + 1]};
+                    mac(v, dd{-l.hi, -l.lo}, dd{pvh[jj + 1], pvl[jj + 1]});
+                    Sh[r][jj + 1] = v.hi;
+                    Sl[r][jj + 1] = v.lo;
+                }
+            }
+        }
+        __syncthreads();
+        if (!last) publish(jj + 1, !zero);
+        // the rest of the rank-1 update
+        if (!zero) {
+            const int ncol = w - jj - 2;
+            if (ncol > 0 && r0 < nrow) {
+                const int nr = nrow - r0;
+                for (int e = tid; e < nr * ncol; e += kPanelThreads) {
+                    const int r = r0 + e / ncol, cc = jj + 2 + e % ncol;
+                    dd v{Sh[r][cc], Sl[r][cc]};
+                    mac(v, dd{-lh[r], -ll[r]}, dd{pvh[cc], pvl[cc]});
+                    Sh[r][cc] = v.hi;
+                    Sl[r][cc] = v.lo;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < nrow * w; e += kPanelThreads) {
+        const int r = e % nrow, q = e / nrow;
+        Ah[r + q * lda] = Sh[r][q];
+        Al[r + q * lda] = Sl[r][q];
+    }
+}
 
 struct LuPlan {
     double *ah, *al;
@@ -1336,7 +1600,7 @@ int getrf_rec(const LuPlan &P, int64_t j0, int64_t n) {
     G = ceil_div(rows, R);
     if (P.panel_ws != nullptr && n <= kPanelW && R <= 1024) {
         const int w = (int)n;
-        cudaError_t e = cudaMemsetAsync(P.panel_ws, 0, 2 * sizeof(unsigned int), P.st);
+        cudaError_t e = cudaMemsetAsync(P.panel_ws, 0, offsetof(PanelWs, key_mag), P.st);
         if (e != cudaSuccess) return cuda_fail(e, "panel barrier reset");
         double *ah = P.ah, *al = P.al;
         int64_t lda = P.lda, m = P.m, jj0 = j0;
@@ -1344,8 +1608,9 @@ int getrf_rec(const LuPlan &P, int64_t j0, int64_t n) {
         int64_t *ipiv = P.ipiv, *info = P.info;
         PanelWs *ws = P.panel_ws;
         void *args[] = {&ah, &al, &lda, &m, &jj0, &ww, &R, &ipiv, &info, &ws};
-        e = cudaLaunchCooperativeKernel((const void *)getrf_panel_kernel, dim3((unsigned)G),
-                                        dim3(kPanelThreads), args, 0, P.st);
+        const void *f = R <= kPanelRows ? (const void *)getrf_panel_smem_kernel
+                                        : (const void *)getrf_panel_kernel;
+        e = cudaLaunchCooperativeKernel(f, dim3((unsigned)G), dim3(kPanelThreads), args, 0, P.st);
         if (e != cudaSuccess) return cuda_fail(e, "getrf_panel_kernel launch");
         if ((rc = check_launch("getrf_panel_kernel"))) return rc;
         // the panel's interchanges on the columns left and right of it
@@ -1414,6 +1679,10 @@ int run_getrf(int64_t m, int64_t n, double *ah, double *al, int64_t lda, int64_t
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, getrf_panel_kernel, kPanelThreads, 0);
+    int per_sm2 = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, getrf_panel_smem_kernel, kPanelThreads,
+                                                  0);
+    if (per_sm2 < per_sm) per_sm = per_sm2;
     const int64_t ctas = (int64_t)per_sm * (sm_count() > 0 ? sm_count() : 0);
     if (coop && ctas > 0) {
         e = pool_alloc(reinterpret_cast<void **>(&P.panel_ws), sizeof(PanelWs), st);
