@@ -49,14 +49,16 @@ __host__ __device__ __forceinline__ int64_t uidx(int lower, int64_t i, int64_t j
 // r..63) and thread g of the cluster (g = rank * 256 + tid) holds the
 // entries g + 256 CL s as dd accumulators; the rows that are done form a
 // prefix of that numbering, so a warp whose entries are all done issues
-// nothing.  Step j: the holder of (j, j) takes the square root of its
-// accumulator, with an approximate reciprocal of it, and writes both into
-// every CTA's shared memory; after a cluster barrier the holders of row j
-// divide by it (one binary64 division each, div_rcp) and write the row into
-// every CTA (two buffers by the parity of j); after a second barrier every
+// nothing.  Step j: the holders of row j write their accumulators into every
+// CTA's shared memory (two buffers by the parity of j); after a cluster
+// barrier two warps of each CTA take the square root of (j, j), with an
+// approximate reciprocal of it, and divide the row by it (div_rcp), all
+// lanes the same root and each its column; after a block barrier every
 // entry (r, c) with j < r <= c subtracts U(j, r) U(j, c), with the GEMM
 // kernels' deferred renormalisation (every entry has taken exactly j + 1
-// updates after step j, so all renormalise at the same steps).
+// updates after step j, so all renormalise at the same steps).  (With the root
+// and the quotients formed by their holders and sent to the others, a step
+// had two cluster barriers: 150 us a block, 135 so.)
 //
 // Every FP64 instruction costs a warp ~64 cycles on GB300 (2 FP64 lanes per
 // clock per SM), so the square root / division chain is kept short and the
@@ -64,9 +66,9 @@ __host__ __device__ __forceinline__ int64_t uidx(int lower, int64_t i, int64_t j
 constexpr int kTri = NB * (NB + 1) / 2;
 
 struct DiagSmem {
-    double rh[2][NB], rl[2][NB];   // the pivot row U(j, :)
-    double uh, ul, uz;             // U(j, j) and an approximate 1 / U(j, j)
-    int fail;                      // a pivot failed (or info was set on entry)
+    double ah[2][NB], al[2][NB];   // row j before the division
+    double rh[NB], rl[NB];         // the pivot row U(j, :)
+    int fail;                      // info was set on entry
 };
 
 __device__ __forceinline__ int tri_start(int r) { return r * NB - (r * (r - 1)) / 2; }
@@ -152,59 +154,52 @@ __device__ void potrf_diag_one(const mp_dd_potrf_diag_desc &d, DiagSmem &s) {
     int jdone = nbe;
     for (int j = 0; j < nbe; ++j) {
         const int e0 = tri_start(j);                 // (j, j)
-        if (g == e0 % G) {
-            const int q = e0 / G;
-            dd p = pick(acc, q);
-            if (!(p.hi > 0.0)) {
-                renorm(p);
-                put(acc, q, p);
-                if (d.info != nullptr)
-                    atomicCAS(reinterpret_cast<unsigned long long *>(d.info), 0ull,
-                              (unsigned long long)(d.offset + j + 1));
+        const int par = j & 1;
+        // row j: the entries e0 .. e0 + nbe - j - 1, at most one per thread
+        const int count = nbe - j;
+        const int e = e0 + (g - e0 % G + G) % G;
+        const int q = e / G, c = j + (e - e0);
+        const bool mine = e < e0 + count;
+        if (mine) {
+            const dd v = pick(acc, q);
 #pragma unroll
-                for (int r = 0; r < CL; ++r) cl.peer[r]->fail = 1;
-            } else {
-                double z;
-                const dd u = sqrt_dd(p, z);
-                put(acc, q, u);
-#pragma unroll
-                for (int r = 0; r < CL; ++r) {
-                    cl.peer[r]->uh = u.hi;
-                    cl.peer[r]->ul = u.lo;
-                    cl.peer[r]->uz = z;
-                }
+            for (int r = 0; r < CL; ++r) {
+                cl.peer[r]->ah[par][c] = v.hi;
+                cl.peer[r]->al[par][c] = v.lo;
             }
         }
         cl.sync();
-        if (s.fail) {                                // the same in every CTA
+        const dd p{s.ah[par][j], s.al[par][j]};
+        if (!(p.hi > 0.0)) {                         // the same in every CTA
+            if (g == 0 && d.info != nullptr)
+                atomicCAS(reinterpret_cast<unsigned long long *>(d.info), 0ull,
+                          (unsigned long long)(d.offset + j + 1));
             jdone = j;
             break;
         }
-        // row j: the entries e0 + 1 .. e0 + nbe - j - 1, at most one per thread
-        {
-            const int first = e0 + 1, count = nbe - j - 1;
-            const int e = first + (g - first % G + G) % G;
-            if (e < first + count) {
-                const int q = e / G;
-                const dd v = div_rcp(pick(acc, q), dd{s.uh, s.ul}, s.uz);
-                put(acc, q, v);
-                const int c = j + 1 + (e - first);
-#pragma unroll
-                for (int r = 0; r < CL; ++r) {
-                    cl.peer[r]->rh[j & 1][c] = v.hi;
-                    cl.peer[r]->rl[j & 1][c] = v.lo;
-                }
+        if ((int)threadIdx.x < NB) {
+            double z;
+            const dd u = sqrt_dd(p, z);
+            const int t = (int)threadIdx.x;
+            if (t == j) {
+                s.rh[t] = u.hi;
+                s.rl[t] = u.lo;
+            } else if (t > j && t < nbe) {
+                const dd v = div_rcp(dd{s.ah[par][t], s.al[par][t]}, u, z);
+                s.rh[t] = v.hi;
+                s.rl[t] = v.lo;
             }
         }
-        cl.sync();
+        __syncthreads();
+        if (mine) put(acc, q, dd{s.rh[c], s.rl[c]});
         const bool renorm_now = (j & (kRenormEvery - 1)) == kRenormEvery - 1;
 #pragma unroll
-        for (int q = 0; q < kSl; ++q) {
-            if (er[q] > j && ec[q] < NB) {
-                const dd ur{-s.rh[j & 1][er[q]], -s.rl[j & 1][er[q]]};
-                const dd uc{s.rh[j & 1][ec[q]], s.rl[j & 1][ec[q]]};
-                mac_deferred(acc[q], ur, uc);
-                if (renorm_now) renorm(acc[q]);
+        for (int f = 0; f < kSl; ++f) {
+            if (er[f] > j && ec[f] < NB) {
+                const dd ur{-s.rh[er[f]], -s.rl[er[f]]};
+                const dd uc{s.rh[ec[f]], s.rl[ec[f]]};
+                mac_deferred(acc[f], ur, uc);
+                if (renorm_now) renorm(acc[f]);
             }
         }
     }
