@@ -19,7 +19,7 @@
 //     are summed in int32 registers (|P_b| < 2^31 for k (b+1) 2^14 < 2^31).
 //     Pairs with t + u >= S are dropped (triangular truncation).
 //  4. Recombination.  V = sum_b P_b 256^(S-1-b) is formed exactly in 192-bit
-//     integer arithmetic, rounded once to the nearest dd and scaled by
+//     integer arithmetic, rounded once to dd and scaled by
 //     2^(e_i + f_j - 8S - 8); the alpha/beta epilogue is dd arithmetic.
 //
 // Error: per product |a b - sum_{t+u<S} d_t d'_u 256^-(t+u+2) 2^(e_i+f_j)|
@@ -46,6 +46,7 @@
 #include <mutex>
 #include <vector>
 
+#include "bigfloat.cuh"
 #include "common.cuh"
 #include "dd_arith.cuh"
 #include "kernels.cuh"
@@ -955,104 +956,57 @@ struct RecArgs {
     int64_t ldc;
 };
 
-// x * 2^e, exact for results in the normal range.
-__device__ __forceinline__ double mul_pow2(double x, int e) {
-    while (e > 1000) {
-        x = __dmul_rn(x, __longlong_as_double((long long)(1000 + 1023) << 52));
-        e -= 1000;
-    }
-    while (e < -1000) {
-        x = __dmul_rn(x, __longlong_as_double((long long)(-1000 + 1023) << 52));
-        e += 1000;
-    }
-    return __dmul_rn(x, __longlong_as_double((long long)(e + 1023) << 52));
-}
-
-__device__ __forceinline__ int msb64(unsigned long long x) { return 63 - __clzll(x); }
-
-// Signed 128-bit integer to the nearest binary64.
-__device__ __forceinline__ double i128_to_double(__int128 v) {
-    bool neg = v < 0;
-    unsigned __int128 a = neg ? (unsigned __int128)(-v) : (unsigned __int128)v;
-    unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
-    double r;
-    if (hi == 0) {
-        r = __ull2double_rn(lo);
-    } else {
-        int p = 64 + msb64(hi);               // >= 64
-        int sh = p - 63;                      // keep the top 64 bits
-        unsigned __int128 top = a >> sh;
-        unsigned long long w = (unsigned long long)top;
-        unsigned __int128 dropped = a & (((unsigned __int128)1 << sh) - 1);
-        if (dropped != 0) w |= 1ull;          // sticky bit below the rounding point
-        r = mul_pow2(__ull2double_rn(w), sh);
-    }
-    return neg ? -r : r;
-}
-
+// V = sum_b P_b 256^(S-1-b) as a two's complement integer of six words: four
+// bands at a time make a signed 64-bit digit of base 2^32 (|P_b| < 2^31), the
+// carries run up the digits; S is padded to 16 bands, so the value is V
+// 256^(16 - S).  Rounded to the nearest dd by integer operations (as the
+// residue form's), then the alpha / beta epilogue.  Bound by HBM: 4 S bytes of
+// band sums, C and the result per entry.  192-bit shifts per band and a
+// rounding through the FP64 pipe's conversions took 150 us at 2048 x 2048
+// (S = 14), this 103 (161 and 115 with alpha).
 __global__ void __launch_bounds__(256) recombine_kernel(const RecArgs p) {
     chain_begin();
     const PlanPick pk = plan_choice(p.plan);
     if (pk.c < 0) return;
     const int S = pk.count;
-    const int64_t total = p.m * p.n;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = idx % p.m, j = idx / p.m;
-        // V = sum_b P_b 256^(S-1-b) in 192-bit two's complement (hi:lo)
-        unsigned __int128 lo = 0;
-        long long hi = 0;
-        for (int b = 0; b < S; ++b) {
-            const int32_t v = p.P[((int64_t)b * p.n_pad + j) * p.m_pad + i];
-            hi = (long long)(((unsigned long long)hi << 8) | (unsigned long long)(lo >> 120));
-            lo <<= 8;
-            const unsigned __int128 ext = (unsigned __int128)(__int128)(long long)v;
-            const unsigned __int128 sum = lo + ext;
-            hi += (sum < lo ? 1 : 0) + (v < 0 ? -1 : 0);
-            lo = sum;
-        }
-        const bool neg = hi < 0;
-        if (neg) {
-            lo = ~lo + 1;
-            hi = (long long)(~(unsigned long long)hi + (lo == 0 ? 1ull : 0ull));
-        }
-        double vh = 0.0, vl = 0.0;
-        const unsigned long long w2 = (unsigned long long)hi;
-        const unsigned long long w1 = (unsigned long long)(lo >> 64), w0 = (unsigned long long)lo;
-        int pbit = -1;
-        if (w2) pbit = 128 + msb64(w2);
-        else if (w1) pbit = 64 + msb64(w1);
-        else if (w0) pbit = msb64(w0);
-        const int sc = scale_exponent(p.rmax[i]) + scale_exponent(p.cmax[j]) - 8 * S - 8;
-        if (pbit >= 0 && pbit <= 52) {
-            vh = mul_pow2(__ull2double_rn(w0), sc);
-        } else if (pbit > 52) {
-            const int q = pbit - 52;          // <= 88 for |V| < 2^141
-            const unsigned __int128 shifted =
-                (lo >> q) | (q < 128 ? ((unsigned __int128)w2 << (128 - q)) : 0);
-            unsigned long long H = (unsigned long long)shifted;
-            const unsigned __int128 mask = ((unsigned __int128)1 << q) - 1;
-            const unsigned __int128 R = lo & mask;
-            const unsigned __int128 half = (unsigned __int128)1 << (q - 1);
-            __int128 Rs = (__int128)R;
-            if (R > half || (R == half && (H & 1))) {
-                ++H;
-                Rs = (__int128)R - ((__int128)1 << q);
-            }
-            vh = mul_pow2(__ull2double_rn(H), q + sc);
-            vl = mul_pow2(i128_to_double(Rs), sc);
-        }
-        if (neg) {
-            vh = -vh;
-            vl = -vl;
-        }
-        dd v{vh, vl};
-        if (!p.alpha_one) v = mul(dd{p.alpha.hi, p.alpha.lo}, v);
+    const int64_t plane = p.n_pad * p.m_pad;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int64_t j = idx / p.m, i = idx - j * p.m;
+    const int64_t sj = stride / p.m, si = stride - sj * p.m;
+    while (j < p.n) {
+        const int32_t *src = p.P + j * p.m_pad + i;
+        int32_t v[16];
+#pragma unroll
+        for (int b = 0; b < 16; ++b) v[b] = b < S ? __ldg(src + b * plane) : 0;
         const int64_t off = i + j * p.ldc;
-        if (!p.beta_zero)
-            v = add_sloppy(v, mul(dd{p.beta.hi, p.beta.lo}, dd{p.ch[off], p.cl[off]}));
-        p.ch[off] = v.hi;
-        p.cl[off] = v.lo;
+        dd c{0.0, 0.0};
+        if (!p.beta_zero) c = dd{p.ch[off], p.cl[off]};
+        uint32_t Z[6];
+        long long carry = 0;
+#pragma unroll
+        for (int g = 3; g >= 0; --g) {
+            // |digit| < 2^31 (2^24 + 2^16 + 2^8 + 1), the carry below 2^25
+            const long long t = (long long)v[4 * g] * (1 << 24) + (long long)v[4 * g + 1] * (1 << 16) +
+                                (long long)v[4 * g + 2] * (1 << 8) + v[4 * g + 3] + carry;
+            Z[3 - g] = (uint32_t)t;
+            carry = t >> 32;
+        }
+        Z[4] = (uint32_t)carry;
+        Z[5] = (uint32_t)(carry >> 32);
+        const int sc = scale_exponent(__ldg(p.rmax + i)) + scale_exponent(__ldg(p.cmax + j)) - 136;
+        dd r;
+        bigf::signed_words_to_dd<6>(Z, sc, r.hi, r.lo);
+        if (!p.alpha_one) r = mul(dd{p.alpha.hi, p.alpha.lo}, r);
+        if (!p.beta_zero) r = add_sloppy(r, mul(dd{p.beta.hi, p.beta.lo}, c));
+        p.ch[off] = r.hi;
+        p.cl[off] = r.lo;
+        i += si;
+        j += sj;
+        if (i >= p.m) {
+            i -= p.m;
+            ++j;
+        }
     }
 }
 
