@@ -757,14 +757,16 @@ struct CrtLayout {
 
 size_t align1k(size_t x) { return (x + 1023) / 1024 * 1024; }
 
-// Tile width of the residue products: 256 (a quarter fewer operand bytes per
-// flop than 128) once the (modulus, tile) work items fill the SMs twice over
-// and the wider padding of n adds at most n / 8.
+// Tile width of the residue products: 256 (twice the flops of a 128-wide tile in
+// about its time, see band_tn) once there are 128 (modulus, tile) work items
+// and the wider padding of n adds at most n / 8.  Band phase on 128 / 256
+// columns: 64 x 1024 x 128 (128 items) 12.0 / 10.5 us, 512^3 (256) 22.7 / 17.5,
+// 768^3 49 / 33; 256^3 (64) 10.2 either way, 128 x 256 x 128 (32) 8.2 / 10.2.
 int crt_band_tn(int64_t m, int64_t n, int N) {
     const int64_t items = ceil_div(imax(m, 1), kBandTM) * ceil_div(imax(n, 1), 256) * N;
     const int64_t pad256 = ceil_div(imax(n, 1), 256) * 256;
     const int64_t pad128 = ceil_div(imax(n, 1), 128) * 128;
-    return (items >= 2 * 152 && (pad256 - pad128) * 8 <= imax(n, 1)) ? 256 : 128;
+    return (items >= 128 && (pad256 - pad128) * 8 <= imax(n, 1)) ? 256 : 128;
 }
 
 // sym: the Rsyrk form, op(B) = op(A)^T (m = n): one set of maxima and
@@ -805,14 +807,28 @@ int launch_residues(const SplitOperand &a, __half *ra, const SplitOperand *b, __
         return o.row_contig ? o.rows_pad / 16 * (k_pad / 64)
                             : ceil_div(o.rows_pad * (k_pad / 64), kResWarps);
     };
-    const int64_t ia = items(x), ib = items(y), rows = x.rows_pad + y.rows_pad;
+    // a block item takes its warps two rows (row-contiguous) or one
+    const int64_t ia = items(x), ib = items(y), ca = x.row_contig ? 2 : 1, cb = y.row_contig ? 2 : 1;
     int64_t na = ia, nb = ib;
     if (ia + ib > slots) {
-        na = slots * x.rows_pad / rows;
-        if (na < 1) na = 1;
-        if (na > ia) na = ia;
+        na = slots * (ia * ca) / (ia * ca + ib * cb);
+        na = na < 1 ? 1 : na > ia ? ia : na;
         nb = slots - na < ib ? slots - na : ib;
         if (b && nb < 1) nb = 1;
+        // few rounds: the split with the shortest longest one
+        if (b && ia * ca + ib * cb <= 16 * slots) {
+            int64_t best = -1;
+            for (int64_t r = 1; r <= 16; ++r) {
+                const int64_t ta = ceil_div(ia, r), tb = slots - ta;
+                if (tb < 1) continue;
+                const int64_t rb = ceil_div(ib, tb), t = r * ca > rb * cb ? r * ca : rb * cb;
+                if (best < 0 || t < best) {
+                    best = t;
+                    na = ta;
+                    nb = ceil_div(ib, rb);
+                }
+            }
+        }
     }
     x.blocks = (unsigned)na;
     y.blocks = (unsigned)nb;

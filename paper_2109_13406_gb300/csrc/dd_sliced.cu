@@ -466,10 +466,13 @@ __device__ __forceinline__ float scaled_floor_f32(double c, int s) {
 // margin of a lower bound of (|A||B|)_ij.  Rows or columns that are all zero
 // (exact in every form), entries outside C or the requested triangle, and
 // entries whose C is infinite or NaN (then so is the result) do not
-// constrain.  An infinite or NaN row or column maximum leaves no margin: the
-// plain kernel computes such a product.  Used by all 32 lanes of an epilogue warp (rows i of the lanes,
+// constrain; each lane keeps its row's constraining columns as a bit mask.  An
+// infinite or NaN row or column maximum leaves no margin: the plain kernel
+// computes such a product.  Used by all 32 lanes of an epilogue warp (rows i of the lanes,
 // the same EC columns): each lane loads EC / 32 column maxima and the warp
-// shares them by shuffles.  C is read 16 columns at a time, the first 16
+// shares their scales by shuffles where C counts.  (Testing every column's
+// range, triangle and zero flag in its turn took 8.7 us a 128 x 128 tile,
+// under 2 with the masks.)  C is read 16 columns at a time, the first 16
 // before the tile's accumulator is complete (under the tile's MMAs).  The
 // minimum over the warp goes to *dmin_out with one atomic.
 template <int EC>
@@ -477,9 +480,9 @@ struct Margin {
     static_assert(EC == 64 || EC == 128, "64 or 128 columns");
     static constexpr int NC = EC / 32;   // column maxima per lane
     unsigned mask;
-    bool bad;   // a row or column with an infinity or NaN
+    bool bad;                // a row or column with an infinity or NaN
     int fcol[NC];
-    bool zcol[NC];
+    unsigned ok[NC];         // columns that constrain this lane's row
     bool row_ok, use_c;
     int ei;
     unsigned int dm;
@@ -490,18 +493,25 @@ struct Margin {
         mask = __activemask();
         const int lane = threadIdx.x & 31;
         bad = false;
+        const unsigned long long rm = i < p.m ? p.rmax[i] : 0ull;
+        row_ok = rm != 0;
+        bad |= rm >= kInfBits64;
+        ei = scale_exponent(rm);
 #pragma unroll
         for (int h = 0; h < NC; ++h) {
             const int64_t j = j0 + 32 * h + lane;
             const unsigned long long cm = j < p.n ? p.cmax[j] : 0ull;
             bad |= cm >= kInfBits64;
-            zcol[h] = cm == 0;
             fcol[h] = scale_exponent(cm);
+            unsigned in = __ballot_sync(mask, cm != 0);
+            if (p.tri) {   // upper: columns from i on, lower: up to i
+                const int64_t d = i - (j0 + 32 * h);
+                const unsigned from = d <= 0 ? 0xFFFFFFFFu : d >= 32 ? 0u : 0xFFFFFFFFu << d;
+                const unsigned upto = d < 0 ? 0u : d >= 31 ? 0xFFFFFFFFu : (2u << d) - 1u;
+                in &= p.tri == 1 ? from : upto;
+            }
+            ok[h] = row_ok ? in : 0u;
         }
-        const unsigned long long rm = i < p.m ? p.rmax[i] : 0ull;
-        row_ok = rm != 0;
-        bad |= rm >= kInfBits64;
-        ei = scale_exponent(rm);
         use_c = p.ba_ratio32 > 0.0f;
         dm = kInfBits32;
     }
@@ -519,15 +529,13 @@ struct Margin {
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
             const int jj = 16 * g + u;
-            const int64_t j = j0 + jj;
-            const int fj = __shfl_sync(mask, fcol[jj / 32], jj % 32);
-            const bool zj = __shfl_sync(mask, (int)zcol[jj / 32], jj % 32) != 0;
             float d = __fmul_rz(__uint_as_float(r[u]), p.c1);
-            if (use_c) d = __fadd_rz(d, __fmul_rz(scaled_floor_f32(cv[u], ei + fj), p.ba_ratio32));
-            const bool inside = row_ok && !zj && j < p.n && !(p.tri == 1 && i > j) &&
-                                !(p.tri == 2 && i < j);
-            const unsigned int db = __float_as_uint(d);
-            dm = (inside && db < dm) ? db : dm;
+            if (use_c) {
+                const int fj = __shfl_sync(mask, fcol[jj / 32], jj % 32);
+                d = __fadd_rz(d, __fmul_rz(scaled_floor_f32(cv[u], ei + fj), p.ba_ratio32));
+            }
+            const unsigned int db = (ok[jj / 32] >> (jj % 32)) & 1u ? __float_as_uint(d) : kInfBits32;
+            dm = db < dm ? db : dm;
         }
     }
     __device__ __forceinline__ void finish(const BandArgs &p) {
@@ -582,15 +590,6 @@ template <int TN, bool MAG, bool PAIR = false, bool TRI = false>
 __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
     band_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                      const __grid_constant__ CUtensorMap tmB, const BandArgs p) {
-    chain_begin();
-    int S = p.S;
-    if (!MAG && p.plan.dmin != nullptr) {
-        // the same decision in every thread of every CTA: a word written by
-        // an earlier launch of this call
-        const PlanPick pk = plan_choice(p.plan);
-        if (pk.c < 0) return;
-        S = pk.count;
-    }
     using Cfg = BandCfg<TN, PAIR>;
     constexpr int STAGES = Cfg::STAGES;
     constexpr uint32_t kStageBytes = Cfg::STAGE_BYTES;
@@ -648,6 +647,8 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
     const int item0 = PAIR ? (int)cluster_id_x() : (int)blockIdx.x;
     const int item_step = PAIR ? (int)cluster_count_x() : (int)gridDim.x;
     if (threadIdx.x == 0) {
+        prefetch_tmap(&tmA);
+        prefetch_tmap(&tmB);
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
@@ -676,6 +677,17 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
     if (PAIR) cluster_sync();   // the peer's barriers exist before anything lands there
     const uint32_t tmem = *tmem_holder;
 
+    // (what precedes this touches no global memory: it runs while the kernel
+    // before finishes)
+    chain_begin();
+    int S = p.S;
+    if (!MAG && p.plan.dmin != nullptr) {
+        // the same decision in every thread of every CTA: a word written by
+        // an earlier launch of this call
+        const PlanPick pk = plan_choice(p.plan);
+        S = pk.c < 0 ? 0 : pk.count;   // no width: no items
+    }
+
     const int num_tiles = TRI ? p.tri_tiles : (PAIR ? p.tiles_m / 2 : p.tiles_m) * p.tiles_n;
     const int KB = p.kb_count;
     const int num_items = p.diag || p.split ? num_tiles * S : num_tiles;
@@ -683,8 +695,6 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
     if (warp == 0) {
         // ---------------- TMA producer
         if (lane == 0) {
-            prefetch_tmap(&tmA);
-            prefetch_tmap(&tmB);
             uint32_t it = 0;
             bool ok = true;
             for (int item = item0; item < num_items && ok; item += item_step) {
@@ -800,12 +810,14 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
                 }
             }
             // every issued MMA has completed before the tensor memory is freed
-            if (PAIR)
-                mma_commit_pair(fin, (uint16_t)1);
-            else
-                mma_commit(fin);
-            long long t0 = clock64();
-            while (!mbar_try_wait(fin, 0) && clock64() - t0 < kWaitCycles) {
+            if (it > 0) {
+                if (PAIR)
+                    mma_commit_pair(fin, (uint16_t)1);
+                else
+                    mma_commit(fin);
+                long long t0 = clock64();
+                while (!mbar_try_wait(fin, 0) && clock64() - t0 < kWaitCycles) {
+                }
             }
         }
         __syncwarp();
