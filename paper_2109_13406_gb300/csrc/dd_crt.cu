@@ -998,7 +998,11 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     ba.diag = 1;
     ba.tri = p.tri;
     ba.plan = plan;
-    for (int i = 0; i < L.N; ++i) ba.moduli[i] = modulus(i);
+    for (int i = 0; i < L.N; ++i) {
+        const int p_i = modulus(i), r = p_i / 2;   // residues: |r| <= 128 mod 256, (p - 1) / 2
+        ba.moduli[i] = p_i;
+        ba.run_kb[i] = (1 << 24) / (r * r) / kBandTK;   // r^2 64 run_kb <= 2^24
+    }
     if ((rc = launch_band(tmA, tmB, ba, TN, st, &tmB_half))) return rc;
     sliced_timing_mark(2, st);
 

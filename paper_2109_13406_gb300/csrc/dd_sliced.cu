@@ -60,10 +60,22 @@ using namespace sm100;
 
 constexpr int TM = 128, TK = 64;            // tile rows and k-block
 constexpr int CHUNK_KB = 16;                // k-blocks per exact fp32 run (1024 products)
-// The magnitude product needs no exact runs (its fp32 sums only have to stay
-// within the certificate's safety factor): one run over the whole k.
+// Exact runs of a band: products of digits run for 1024 (|d| <= 128), those of
+// residues mod p for as many as keep the sum of squares of (p - 1) / 2 within
+// 2^24 (BandArgs::run_kb: 1024 for the largest moduli, 6400 for 103), the
+// magnitude product (whose fp32 sums only have to stay within the
+// certificate's safety factor) in one run over the whole k.  A band's runs
+// are made about equally long.  Fewer drains leave the tensor memory to the
+// MMAs: 158 runs instead of 256 for the 32 moduli at k = 8192, and 2 % of the band
+// phase at 1501 x 2777 x 1999 (377 -> 369 us), 2048^3 (364 -> 356) and for the 4096
+// Rsyrk (1407 -> 1374); at 8192, where the clock follows the power, nothing.
 template <bool MAG>
-__host__ __device__ constexpr int chunk_kb() { return MAG ? (1 << 30) : CHUNK_KB; }
+__device__ __forceinline__ int run_length(const BandArgs &p, int b, int steps) {
+    if (MAG) return steps;
+    const int most = p.diag ? p.run_kb[b] : CHUNK_KB;
+    const int runs = (steps + most - 1) / most;
+    return (steps + runs - 1) / runs;
+}
 // Tile columns per rasterisation group: 8 for full products; 4 for the
 // Rsyrk triangle, where the balance of the skipped tiles over the CTAs
 // matters more than operand reuse (13 % faster at 8192; 4 and 16 are 1.4 %
@@ -758,14 +770,15 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
                 item_coords<TN, PAIR>(p, S, item, num_tiles, rank, tri_s, tm, tn, b0, b1);
                 for (int b = b0; b < b1 && ok; ++b) {
                     const int steps = (p.diag ? 1 : b + 1) * KB;
-                    int sidx = 0;
+                    const int run = run_length<MAG>(p, b, steps);
+                    int sidx = 0, in_run = 0;
                     for (int t = p.diag ? b : 0; t <= b && ok; ++t)
                         for (int kb = 0; kb < KB; ++kb, ++it, ++sidx) {
                             const int s = it % STAGES;
                             const uint32_t f = it / STAGES;
-                            const bool first = (sidx % chunk_kb<MAG>()) == 0;
-                            const bool last =
-                                ((sidx + 1) % chunk_kb<MAG>()) == 0 || sidx + 1 == steps;
+                            const bool first = in_run == 0;
+                            const bool last = in_run + 1 == run || sidx + 1 == steps;
+                            in_run = last ? 0 : in_run + 1;
                             const uint32_t buf = chunk & 1, use = chunk >> 1;
                             if (first) {
                                 if (!mbar_wait(&acce[buf], (use & 1) ^ 1, abort_flag)) {
@@ -869,9 +882,10 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
                     continue;
                 }
                 const int steps = (p.diag ? 1 : b + 1) * KB;
-                const int nchunks = (steps + chunk_kb<MAG>() - 1) / chunk_kb<MAG>();
+                const int run = run_length<MAG>(p, b, steps);
+                const int nchunks = (steps + run - 1) / run;
                 if (p.diag && nchunks == 1) {
-                    // one exact run (k <= 1024): reduced mod p as it is read
+                    // one exact run: reduced mod p as it is read
                     const uint32_t buf = chunk & 1, use = chunk >> 1;
                     ++chunk;
                     const float pm = (float)p.moduli[b];

@@ -96,6 +96,7 @@ struct BandArgs {
     int split;    // triangle mode: work items of one band each (else all bands of a tile)
     int tri;      // diagonal / magnitude mode: 1 / 2 = only the upper / lower triangle
     int moduli[kMaxBands];
+    int run_kb[kMaxBands];     // diagonal mode: k-blocks of an exact fp32 run mod moduli[b]
     SplitPlan plan;
     // magnitude mode
     int mag;
