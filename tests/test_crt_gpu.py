@@ -355,3 +355,42 @@ def test_chained_launches_replay_from_a_graph(cuda_lib, m, n, k):
         assert mp.mp_dd_workspace_status(ws) == 0
         got = host(C, m, n)
         assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("k", [2240, 5312, 6400])
+def test_crt_long_runs_at_their_bound(cuda_lib, k):
+    """Entries whose residues are (p - 1) / 2 for the 14 smallest of the 32
+    moduli at once, all of one sign, over the longest exact run of p = 173
+    (2240 steps), 113 (5312) and 103 (6400): the run ends just below 2^24.
+    Product planes bit-exact against the oracle."""
+    mp = cuda_lib
+    m = n = 3
+    mods = oz.crt_moduli(32)
+    Q = 1
+    for p in mods[18:]:
+        Q *= p
+    # X = (Q - 1) / 2 + t Q in [2^110, 2^111), a multiple of 256 (so a dd holds it)
+    t = (-((Q - 1) // 2) * pow(Q, -1, 256)) % 256
+    X = (Q - 1) // 2 + t * Q
+    X += -((X - 2 ** 110) // (256 * Q)) * 256 * Q
+    assert 2 ** 110 <= X < 2 ** 111 and X % 256 == 0
+    assert all(X % p == (p - 1) // 2 for p in mods[18:])
+    hi = float(X)
+    lo = float(X - int(hi))
+    assert int(hi) + int(lo) == X
+    A = tuple(np.full((m, k), v * 2.0 ** -111, order="F") for v in (hi, lo))
+    B = tuple(np.full((k, n), v * 2.0 ** -111, order="F") for v in (hi, lo))
+    c = datagen.GemmCase("N", "N", m, n, k, (1.0, 0.0), A, B, (0.0, 0.0),
+                         datagen.dd_matrix(datagen.rng(780), m, n, m))
+    got, ws = run_crt(mp, c)
+    rep = mp.mp_dd_split_report(ws)
+    assert rep["width_bits"] == 112
+    L = mp.mp_dd_crt_layout(m, n, k)
+    used = L["moduli"][:rep["count"]]
+    RA, _ = oz.residue_planes(*oz.op_rows(c.A, False, m, k), used, 14)
+    RB, _ = oz.residue_planes(*oz.op_cols(c.B, False, k, n), used, 14)
+    assert all(abs(RA[b, 0, 0]) == used[b] // 2 for b in range(18, 32))
+    N, mp_, np_ = len(used), L["m_pad"], L["n_pad"]
+    prods = view(ws, L["products"], N * np_ * mp_, np.uint8).reshape(N, np_, mp_)
+    want = oz.crt_products(RA, RB, used)
+    assert np.array_equal(prods[:, :n, :m].transpose(0, 2, 1).astype(np.int64), want)
