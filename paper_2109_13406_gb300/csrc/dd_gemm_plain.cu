@@ -10,7 +10,7 @@
 // products, TwoSum into the accumulator, and a FastTwoSum renormalisation
 // every 4 steps of k (dd_arith.cuh).
 //
-// On GB300 the FP64 pipe is the bottleneck by a wide margin (9.75 FP64
+// On GB300 the FP64 pipe is the bottleneck by a wide margin (7.75 FP64
 // instructions per dd multiply-add), so the kernel is organised to keep that
 // pipe busy and nothing else (large plain products go to the TMA-staged form
 // of this kernel, dd_gemm_tma.cu, whose per-entry arithmetic is identical):
@@ -39,8 +39,12 @@ namespace {
 constexpr int BK = 16;
 
 // Tile shapes: TX x TY threads, each an R x R block of entries TX (TY) apart.
-template <int R_, int TX_, int TY_>
+// ALONE: for launches of at most one tile per SM, whose time is the latency of
+// a warp's chain, where the integer form of the sums' errors does not help
+// (96 x 80 x 70: 31.9 us against 32.7).
+template <int R_, int TX_, int TY_, bool ALONE_ = false>
 struct PlainShape {
+    static constexpr bool ALONE = ALONE_;
     static constexpr int R = R_, TX = TX_, TY = TY_, NT = TX_ * TY_;
     static constexpr int BM = TX_ * R_, BN = TY_ * R_;
     static constexpr int QA = (BM * BK + NT - 1) / NT, QB = (BN * BK + NT - 1) / NT;
@@ -49,6 +53,8 @@ template <int R>
 using Square = PlainShape<R, 16, 16>;
 using Half = PlainShape<1, 16, 8>;    // 16 x 8
 using Tall = PlainShape<1, 32, 4>;    // 32 x 4
+using HalfAlone = PlainShape<1, 16, 8, true>;
+using TallAlone = PlainShape<1, 32, 4, true>;
 
 template <class S>
 struct PlainSmem {
@@ -194,7 +200,7 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<S> &s) {
             if (l0 + BK < kk) load(l0 + BK);
 #pragma unroll 1
             for (int l4 = 0; l4 < BK; l4 += kRenormEvery) {
-#pragma unroll
+#pragma unroll (R * R >= 8 ? 1 : kRenormEvery)
                 for (int l = l4; l < l4 + kRenormEvery; ++l) {
                     dd a[R], b[R];
 #pragma unroll
@@ -206,7 +212,10 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<S> &s) {
 #pragma unroll
                     for (int r = 0; r < R; ++r)
 #pragma unroll
-                        for (int c = 0; c < R; ++c) mac_deferred(acc[r][c], a[r], b[c]);
+                        for (int c = 0; c < R; ++c) {
+                            if constexpr (S::ALONE) mac_deferred(acc[r][c], a[r], b[c]);
+                            else mac_mixed(acc[r][c], a[r], b[c]);
+                        }
                 }
 #pragma unroll
                 for (int r = 0; r < R; ++r)
@@ -279,7 +288,7 @@ int launch_shape(const GemmArgs &p, cudaStream_t stream) {
 
 // Tile size: the time of a launch is about (tiles per SM, rounded up) x
 // (work per tile), in units of 128 entries -- one accumulator for each of four
-// warps, one per partition of the SM, 0.36 us per step of k (9.75 FP64
+// warps, one per partition of the SM, 0.29 us per step of k (7.75 FP64
 // instructions per multiply-add at 526 G/s over 152 SMs); the largest tile
 // with the least such time wins (the per-entry operation sequence, and hence
 // the result, does not depend on it).  16 x 8 and 32 x 4 tiles are one unit:
@@ -359,7 +368,7 @@ int launch_gemm_update(const GemmArgs &p, cudaStream_t stream) {
     if (p.m < kUpdateMin || p.n < kUpdateMin || p.k < kUpdateMin || p.k > ((int64_t)1 << 17) - 1 ||
         p.tri != 0 || p.alpha_zero || p.a2h != nullptr || p.sym_a || p.sym_b)
         return launch_gemm_plain(p, stream);
-    const double plain_us = 0.36 * (double)p.k * (double)plain_best_cost(p);
+    const double plain_us = 0.29 * (double)p.k * (double)plain_best_cost(p);
     if (crt_estimate_us(p.m, p.n, p.k) > 0.8 * plain_us) return launch_gemm_plain(p, stream);
     // allocations inside a stream capture would belong to the graph
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -401,9 +410,12 @@ int launch_gemm_plain(const GemmArgs &p, cudaStream_t stream) {
     int rc = 0;
     if (try_launch_gemm_tma(p, stream, &rc)) return rc;
     int64_t cost;
-    switch (plain_tile(p, &cost)) {
-        case kTileTall: return launch_shape<Tall>(p, stream);
-        case kTileHalf: return launch_shape<Half>(p, stream);
+    const PlainTile t = plain_tile(p, &cost);
+    switch (t) {   // cost 1: one small tile per SM at most
+        case kTileTall:
+            return cost <= 1 ? launch_shape<TallAlone>(p, stream) : launch_shape<Tall>(p, stream);
+        case kTileHalf:
+            return cost <= 1 ? launch_shape<HalfAlone>(p, stream) : launch_shape<Half>(p, stream);
         case kTile16: return launch_shape<Square<1>>(p, stream);
         case kTile32: return launch_shape<Square<2>>(p, stream);
         default: return launch_shape<Square<4>>(p, stream);

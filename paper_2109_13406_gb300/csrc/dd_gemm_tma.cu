@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint8_t *sbh = st + 2 * kPanelBytes, *sbl = st + 3 * kPanelBytes;
 #pragma unroll 1
             for (int l4 = 0; l4 < kBK; l4 += kRenormEvery) {
-#pragma unroll
+#pragma unroll 1
                 for (int l = l4; l < l4 + kRenormEvery; ++l) {
                     dd av[4], bv[4];
 #pragma unroll
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                     for (int r = 0; r < 4; ++r)
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) mac_deferred(acc[r][c], av[r], bv[c]);
+                        for (int c = 0; c < 4; ++c) mac_mixed(acc[r][c], av[r], bv[c]);
                 }
 #pragma unroll
                 for (int r = 0; r < 4; ++r)

@@ -18,7 +18,7 @@
 // Tile shapes: 16*RM x 16*RN with (RM, RN) in {(2,2), (4,2), (2,4), (1,1)};
 // the 256 threads form a 16 x 16 grid and each holds an RM x RN block of dd
 // accumulators.  Small shapes waste fewer zero-padded multiply-adds on
-// ragged problems (each costs the full 9.75 FP64 instructions); larger ones
+// ragged problems (each costs the full 7.75 FP64 instructions); larger ones
 // give each thread more independent chains.  All shapes fit 128 registers,
 // so two CTAs share an SM.
 #include <algorithm>
@@ -145,7 +145,7 @@ __device__ __forceinline__ void dd_tile(const mp_dd_gemm_desc &d, int64_t bi, in
                                               kRenormEvery;
 #pragma unroll 1
             for (int l4 = 0; l4 < lend; l4 += kRenormEvery) {
-#pragma unroll
+#pragma unroll (RM * RN >= 8 ? 1 : kRenormEvery)
                 for (int l = l4; l < l4 + kRenormEvery; ++l) {
                     dd a[RM], b[RN];
 #pragma unroll
@@ -157,7 +157,7 @@ __device__ __forceinline__ void dd_tile(const mp_dd_gemm_desc &d, int64_t bi, in
 #pragma unroll
                     for (int r = 0; r < RM; ++r)
 #pragma unroll
-                        for (int c = 0; c < RN; ++c) mac_deferred(acc[r][c], a[r], b[c]);
+                        for (int c = 0; c < RN; ++c) mac_mixed(acc[r][c], a[r], b[c]);
                 }
 #pragma unroll
                 for (int r = 0; r < RM; ++r)

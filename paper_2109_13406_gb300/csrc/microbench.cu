@@ -5,12 +5,14 @@
 // with a grid of 8 CTAs x 256 threads per SM.  The chain values stay
 // bounded (x <- x * b + c with |b| < 1) so no operand becomes denormal.
 //
-// dd multiply-add rate: the plain kernel's own multiply-add (mac_deferred,
-// renorm every kRenormEvery steps) on a 4 x 4 block of accumulators per
+// dd multiply-add rate: the multiply-add with every operation on the FP64 pipe
+// (mac_deferred, renorm every kRenormEvery steps: 9.75 instructions; the GEMM
+// kernels form rounding errors on the integer pipe, to the same bits, and run
+// above this rate) on a 4 x 4 block of accumulators per
 // thread, with operands that change every step through integer operations
 // on their bit patterns (no FP64 instruction and no memory access besides
-// the multiply-adds, and nothing the compiler can hoist): the ceiling of the
-// plain kernel's instruction mix on this GPU's FP64 pipe.
+// the multiply-adds, and nothing the compiler can hoist): the ceiling of that
+// instruction mix on this GPU's FP64 pipe.
 //
 // INT8 tensor rate of the warp-level path: sm_103a has no tcgen05 kind::i8,
 // so the only INT8 x INT8 -> INT32 tensor instruction is the legacy

@@ -1,7 +1,8 @@
 // Host check of two_sum (dd_arith.cuh): on operand pairs over the whole
 // binary64 range (equal and adjacent exponents, ties, powers of two,
-// cancellation, subnormals, zeros) its s and e are those of Knuth's six
-// operations, as numbers, in either operand order.  Prints "pairs N bad M".
+// cancellation, subnormals, zeros) its s and e, and sum_error, are those of
+// Knuth's six operations, as numbers, in either operand order.  Prints
+// "pairs N bad M".
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -46,7 +47,7 @@ int main() {
             mpdd::two_sum(x, y, s2, e2);
             ++pairs;
             if (std::isinf(s)) continue;   // (both error words are non-finite)
-            if (!(s2 == s && e2 == e)) ++bad;
+            if (!(s2 == s && e2 == e && mpdd::sum_error(x, y, s) == e)) ++bad;
         }
     }
     printf("pairs %ld bad %ld\n", pairs, bad);
