@@ -51,9 +51,10 @@ METRIC = "dd-Rgemm/Rsyrk GFlops vs roofline; sliced vs plain at bound; p50/p99 s
 UNIT = "dd-GFlop/s"
 # nominal FP64 rate of GB300 (1.25 TFLOP/s counting an FMA as two flops) ->
 # 625 G FP64 instructions per second; a dd multiply-add in the GEMM kernels
-# costs 9.75 of them (1 DMUL + 3 DFMA + 5 DADD, FastTwoSum every 4 steps)
+# costs 6.75 of them (1 DMUL + 2 DFMA + 3 DADD, FastTwoSum every 4 steps; the
+# rounding errors of the product and of the sum come from the integer pipe)
 NOMINAL_FP64_INSTR = 1.25e12 / 2
-FP64_OPS_PER_MAC = 9.75
+FP64_OPS_PER_MAC = 6.75
 QD_OPS_PER_MAC = 73.25   # qd multiply-add: 71 FP64 operations + 2.25 for the level pass
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from single ncu
 # captures of the current kernels (the summaries under profiles/ give the
@@ -364,9 +365,10 @@ def plain_section(mp, torch, size, problems, r64, rmac=None):
     """The plain FP64 path on the step's three problems, one call each timed
     with CUDA events (after the split-precision runs on the same inputs).
     Fractions: of 2 R64 / 15 (the survey's accounting, R64 the measured FP64
-    FMA rate), of the FP64 pipe at the kernel's 9.75 instructions per
-    multiply-add, and of the measured rate of the kernel's own multiply-add
-    mix with operands in registers (mp_dd_peak_ddmac)."""
+    FMA rate), of the FP64 pipe at the kernel's 6.75 instructions per
+    multiply-add, and of the measured rate of the all-FP64 multiply-add
+    (9.75 instructions) with operands in registers (mp_dd_peak_ddmac), which
+    the kernel exceeds: it forms rounding errors on the integer pipe."""
     nn, tn, syrk, dnn, dtn, dsy = problems
     st = torch.cuda.current_stream()
     flops = plain_flops(size)

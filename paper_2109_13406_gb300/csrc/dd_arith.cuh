@@ -110,17 +110,19 @@ __device__ __forceinline__ void mac(dd &acc, dd a, dd b) {
 // alter the result.
 constexpr int kRenormEvery = 4;
 
-// ---- the error of a sum on the integer pipe
+// ---- the errors of a sum and of a product on the integer pipe
 //
-// The error of a sum that the FP64 pipe has rounded is a binary64 number.  The
-// FP64 pipe forms it with two more instructions (two_sum), each of which
-// holds it for ~76 cycles of a warp; the integer pipe, idle beside it, forms it
-// from the significands with ~60 instructions of 2 cycles: modulo 2^64,
-// because it is a small integer in the unit of the smaller operand's last
-// place.  A dd multiply-add takes 7.75 FP64 instructions instead of 9.75:
-// Rgemm 1101 x 700 x 905 12.52 -> 9.88 ms, 512 grouped problems 29.2 -> 23.0.
-// The result is the same bits; the host compares it with the FP64 form over
-// the whole range in a test.
+// The error of a sum or product that the FP64 pipe has rounded is a binary64
+// number.  The FP64 pipe forms it with two more instructions (two_sum) or one
+// (fma), each of which holds it for ~76 cycles of a warp; the integer pipe,
+// idle beside it, forms it from the significands with ~60 or ~40 instructions
+// of 2 cycles: modulo 2^64, because it is a small integer in the unit of the
+// smaller operand's last place (of the product of the last places).  A dd
+// multiply-add takes 6.75 FP64 instructions instead of 9.75: Rgemm 1101 x 700
+// x 905 12.52 ms with neither, 9.88 with the sum's error on the integer pipe,
+// 8.76 with the product's as well; 512 grouped problems 29.2, 23.0 and 20.4.
+// The result is the same bits; the host compares both with the FP64 forms
+// over the whole range in tests.
 
 __host__ __device__ __forceinline__ unsigned long long bits_of(double x) {
 #if defined(__CUDA_ARCH__)
@@ -199,6 +201,30 @@ __host__ __device__ __forceinline__ double sum_error(double x, double y, double 
     return ms.e == 0x7FF ? from_bits(0x7FF8000000000000ull) : e;
 }
 
+// a b - p for p = RN(a b): fma(a, b, -p) from the integer pipe (the sign of a
+// zero aside; NaN where p is an infinity or NaN).  The significands' product
+// and p's agree above the unit 2^52 or 2^53 of p, so the low 64 bits of the
+// one minus the other are the error as an integer of at most 53 bits.  A p
+// below 2^-1021 has an error of half a subnormal unit at most, which rounds to
+// zero; so has one that subnormal factors leave exact.
+__host__ __device__ __forceinline__ double prod_error(double a, double b, double p) {
+    const unsigned long long ua = bits_of(a), ub = bits_of(b);
+    const Significand ma = significand(ua), mb = significand(ub), mp = significand(bits_of(p));
+    int e0 = ma.e + mb.e - 1075;   // the unit of the product is 2^(e0 - 1075)
+    const int sh = mp.e - e0;
+    long long v = (long long)(ma.m * mb.m - (mp.m << (sh & 63)));
+    if (e0 < 1) {   // the error's last places lie below the subnormals: round to even
+        const int t = 1 - e0 > 54 ? 54 : 1 - e0;
+        const unsigned long long w = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+        const unsigned long long q = (w + ((1ull << (t - 1)) - 1) + ((w >> t) & 1)) >> t;
+        v = v < 0 ? -(long long)q : (long long)q;
+        e0 = 1;
+    }
+    double e = exact_double(v, e0, (unsigned int)((ua ^ ub) >> 32) & 0x80000000u);
+    e = (mp.e <= 1 || sh < 0) ? 0.0 : e;
+    return mp.e == 0x7FF ? from_bits(0x7FF8000000000000ull) : e;
+}
+
 __device__ __forceinline__ void mac_deferred(dd &acc, dd a, dd b) {
     double p, e, s, e1;
     prod_terms(a, b, p, e);
@@ -207,10 +233,10 @@ __device__ __forceinline__ void mac_deferred(dd &acc, dd a, dd b) {
     acc.lo = __dadd_rn(acc.lo, __dadd_rn(e1, e));
 }
 
-// mac_deferred with the sum's error from the integer pipe: the same result.
+// mac_deferred with both errors from the integer pipe: the same result.
 __device__ __forceinline__ void mac_mixed(dd &acc, dd a, dd b) {
-    double p, e;
-    prod_terms(a, b, p, e);
+    const double p = __dmul_rn(a.hi, b.hi);
+    const double e = __fma_rn(a.lo, b.hi, __fma_rn(a.hi, b.lo, prod_error(a.hi, b.hi, p)));
     const double s = __dadd_rn(acc.hi, p);
     const double e1 = sum_error(acc.hi, p, s);
     acc.hi = s;

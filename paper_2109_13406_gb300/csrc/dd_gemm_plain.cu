@@ -10,7 +10,7 @@
 // products, TwoSum into the accumulator, and a FastTwoSum renormalisation
 // every 4 steps of k (dd_arith.cuh).
 //
-// On GB300 the FP64 pipe is the bottleneck by a wide margin (7.75 FP64
+// On GB300 the FP64 pipe is the bottleneck by a wide margin (6.75 FP64
 // instructions per dd multiply-add), so the kernel is organised to keep that
 // pipe busy and nothing else (large plain products go to the TMA-staged form
 // of this kernel, dd_gemm_tma.cu, whose per-entry arithmetic is identical):
@@ -40,8 +40,8 @@ constexpr int BK = 16;
 
 // Tile shapes: TX x TY threads, each an R x R block of entries TX (TY) apart.
 // ALONE: for launches of at most one tile per SM, whose time is the latency of
-// a warp's chain, where the integer form of the sums' errors does not help
-// (96 x 80 x 70: 31.9 us against 32.7).
+// a warp's chain, where the integer forms of the errors do not help (96 x 80 x
+// 70: 31.9 us, 32.7 with the sums' on the integer pipe).
 template <int R_, int TX_, int TY_, bool ALONE_ = false>
 struct PlainShape {
     static constexpr bool ALONE = ALONE_;
@@ -288,7 +288,7 @@ int launch_shape(const GemmArgs &p, cudaStream_t stream) {
 
 // Tile size: the time of a launch is about (tiles per SM, rounded up) x
 // (work per tile), in units of 128 entries -- one accumulator for each of four
-// warps, one per partition of the SM, 0.29 us per step of k (7.75 FP64
+// warps, one per partition of the SM, 0.25 us per step of k (6.75 FP64
 // instructions per multiply-add at 526 G/s over 152 SMs); the largest tile
 // with the least such time wins (the per-entry operation sequence, and hence
 // the result, does not depend on it).  16 x 8 and 32 x 4 tiles are one unit:
@@ -368,7 +368,7 @@ int launch_gemm_update(const GemmArgs &p, cudaStream_t stream) {
     if (p.m < kUpdateMin || p.n < kUpdateMin || p.k < kUpdateMin || p.k > ((int64_t)1 << 17) - 1 ||
         p.tri != 0 || p.alpha_zero || p.a2h != nullptr || p.sym_a || p.sym_b)
         return launch_gemm_plain(p, stream);
-    const double plain_us = 0.29 * (double)p.k * (double)plain_best_cost(p);
+    const double plain_us = 0.25 * (double)p.k * (double)plain_best_cost(p);
     if (crt_estimate_us(p.m, p.n, p.k) > 0.8 * plain_us) return launch_gemm_plain(p, stream);
     // allocations inside a stream capture would belong to the graph
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

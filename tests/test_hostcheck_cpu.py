@@ -63,6 +63,15 @@ def test_two_sum_equals_knuths(tmp_path):
     assert pairs == 8000000 and bad == 0
 
 
+def test_prod_error_equals_the_fma(tmp_path):
+    exe = str(tmp_path / "prod_error")
+    _build(os.path.join(HERE, "hostcheck", "prod_error.cu"), exe, shared=False)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    pairs, bad = (int(x) for x in r.stdout.split()[1::2])
+    assert pairs == 6000000 and bad == 0
+
+
 def test_words_to_dd_rounding(tmp_path):
     so = str(tmp_path / "words_dd.so")
     _build(os.path.join(HERE, "hostcheck", "words_dd.cu"), so, shared=True)
