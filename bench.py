@@ -55,7 +55,7 @@ UNIT = "dd-GFlop/s"
 # rounding errors of the product and of the sum come from the integer pipe)
 NOMINAL_FP64_INSTR = 1.25e12 / 2
 FP64_OPS_PER_MAC = 6.75
-QD_OPS_PER_MAC = 73.25   # qd multiply-add: 71 FP64 operations + 2.25 for the level pass
+QD_OPS_PER_MAC = 39.25   # qd multiply-add: 37 FP64 operations + 2.25 for the level pass
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from single ncu
 # captures of the current kernels (the summaries under profiles/ give the
 # commands): the plain Rgemm NN launch at 4096 and the band kernel of the
@@ -854,7 +854,7 @@ def routines_section(mp, torch, size):
     out[f"Rgetrf_{n}"]["info"] = int(info.item())
     del A, B, C, A0
     out.update(potrf_section(mp, torch, n, info))
-    # quad-double Rgemm (73.25 FP64 instructions per qd multiply-add)
+    # quad-double Rgemm (39.25 FP64 instructions per qd multiply-add)
     nq = min(n, 1024)
     gq = datagen.rng(5)
     Aq, Bq, Cq = (dev(datagen.qd_matrix(gq, nq, nq)) for _ in range(3))

@@ -16,13 +16,21 @@
 // products of order u^4 and below (within 7 u^4 |a b|), so the result
 // stays within the qd bound 4 k 2^-209 (|alpha||A||B| + |beta||C|).  Every
 // 4 steps one bottom-up TwoSum pass (L2+L3, L1+L2, L0+L1) brings level t
-// back to order u^t |acc|; the pass is exact.  71 FP64 operations per
-// step plus 2.25 for the pass (113 and 4.5 with Knuth's six-operation TwoSum).
+// back to order u^t |acc|; the pass is exact.
 //
-// Tiles: 16R x 16R of C per CTA (R = 2 or 1, the larger one when the tiles
-// still fill the SMs), R x R qd accumulators per thread, the four planes of
-// the op(A) and op(B) panels staged through shared memory 16 columns of k
-// at a time.  The per-entry operation sequence does not depend on R.
+// The FP64 pipe bounds it, so the errors of the sums (sum_error) and, where
+// more than two warps share a partition of an SM (PE), of the products
+// (prod_error) are formed on the integer pipe, to the same bits: 37 FP64
+// operations per step plus 2.25 for the pass (71 with the errors on the FP64
+// pipe, 113 and 4.5 with Knuth's TwoSum).  331 x 300 x 257: 4.33 ms with
+// neither, 2.66 with the sums', 2.53 with both.  With two warps or fewer the
+// step's latency counts and the fused multiply-add is the better form of the
+// products' errors (150 x 140 x 300: 1.02 ms against 1.10).
+//
+// Tiles: 32 x 32 (2 x 2 qd accumulators per thread), 16 x 16 or 16 x 8 entries
+// of C per CTA, the four planes of the op(A) and op(B) panels staged through
+// shared memory 16 columns of k at a time.  The per-entry operation sequence
+// does not depend on the tile.
 #include "common.cuh"
 #include "dd_arith.cuh"
 #include "kernels.cuh"
@@ -30,35 +38,49 @@
 namespace mpdd {
 namespace {
 
-constexpr int QBK = 16, QNT = 256, kQdRenormEvery = 4;
+constexpr int QBK = 16, kQdRenormEvery = 4;
 
 struct qd4 {
     double x0, x1, x2, x3;
 };
 
+// two_sum with the error from the integer pipe (the same bits).
+__device__ __forceinline__ void two_sum_mixed(double a, double b, double &s, double &e) {
+    const double t = __dadd_rn(a, b);
+    e = sum_error(a, b, t);
+    s = t;
+}
+
+template <bool PE>
+__device__ __forceinline__ double qd_prod_error(double a, double b, double p) {
+    if constexpr (PE) return prod_error(a, b, p);
+    return __fma_rn(a, b, -p);
+}
+
+template <bool PE>
 __device__ __forceinline__ void qd_mac(double (&L)[4], const qd4 &a, const qd4 &b) {
     double e, f0, f1, f2, f3;
-    const double p0 = __dmul_rn(a.x0, b.x0), q0 = __fma_rn(a.x0, b.x0, -p0);
-    two_sum(L[0], p0, L[0], e);
-    const double p1 = __dmul_rn(a.x0, b.x1), q1 = __fma_rn(a.x0, b.x1, -p1);
-    const double p2 = __dmul_rn(a.x1, b.x0), q2 = __fma_rn(a.x1, b.x0, -p2);
-    two_sum(L[1], e, L[1], f0);
-    two_sum(L[1], q0, L[1], f1);
-    two_sum(L[1], p1, L[1], f2);
-    two_sum(L[1], p2, L[1], f3);
-    const double p3 = __dmul_rn(a.x0, b.x2), q3 = __fma_rn(a.x0, b.x2, -p3);
-    const double p4 = __dmul_rn(a.x1, b.x1), q4 = __fma_rn(a.x1, b.x1, -p4);
-    const double p5 = __dmul_rn(a.x2, b.x0), q5 = __fma_rn(a.x2, b.x0, -p5);
+    const double p0 = __dmul_rn(a.x0, b.x0), q0 = qd_prod_error<PE>(a.x0, b.x0, p0);
+    two_sum_mixed(L[0], p0, L[0], e);
+    const double p1 = __dmul_rn(a.x0, b.x1), q1 = qd_prod_error<PE>(a.x0, b.x1, p1);
+    const double p2 = __dmul_rn(a.x1, b.x0), q2 = qd_prod_error<PE>(a.x1, b.x0, p2);
+    two_sum_mixed(L[1], e, L[1], f0);
+    two_sum_mixed(L[1], q0, L[1], f1);
+    two_sum_mixed(L[1], p1, L[1], f2);
+    two_sum_mixed(L[1], p2, L[1], f3);
+    const double p3 = __dmul_rn(a.x0, b.x2), q3 = qd_prod_error<PE>(a.x0, b.x2, p3);
+    const double p4 = __dmul_rn(a.x1, b.x1), q4 = qd_prod_error<PE>(a.x1, b.x1, p4);
+    const double p5 = __dmul_rn(a.x2, b.x0), q5 = qd_prod_error<PE>(a.x2, b.x0, p5);
     double g0, g1, g2, g3, g4, g5, g6, g7, g8;
-    two_sum(L[2], f0, L[2], g0);
-    two_sum(L[2], f1, L[2], g1);
-    two_sum(L[2], f2, L[2], g2);
-    two_sum(L[2], f3, L[2], g3);
-    two_sum(L[2], q1, L[2], g4);
-    two_sum(L[2], q2, L[2], g5);
-    two_sum(L[2], p3, L[2], g6);
-    two_sum(L[2], p4, L[2], g7);
-    two_sum(L[2], p5, L[2], g8);
+    two_sum_mixed(L[2], f0, L[2], g0);
+    two_sum_mixed(L[2], f1, L[2], g1);
+    two_sum_mixed(L[2], f2, L[2], g2);
+    two_sum_mixed(L[2], f3, L[2], g3);
+    two_sum_mixed(L[2], q1, L[2], g4);
+    two_sum_mixed(L[2], q2, L[2], g5);
+    two_sum_mixed(L[2], p3, L[2], g6);
+    two_sum_mixed(L[2], p4, L[2], g7);
+    two_sum_mixed(L[2], p5, L[2], g8);
     const double t3 =
         __fma_rn(a.x0, b.x3, __fma_rn(a.x1, b.x2, __fma_rn(a.x2, b.x1, __dmul_rn(a.x3, b.x0))));
     const double s = __dadd_rn(__dadd_rn(__dadd_rn(__dadd_rn(g0, g1), __dadd_rn(g2, g3)),
@@ -98,21 +120,21 @@ struct QdArgs {
     int alpha_zero, alpha_one, beta_zero;
 };
 
-template <int R>
+template <int R, int TY>
 struct QdSmem {
-    static constexpr int B = 16 * R;
-    double a[4][QBK][B + 1];   // op(A) panel planes, [l][i]
-    double b[4][QBK][B + 1];   // op(B) panel planes, [l][j]
+    double a[4][QBK][16 * R + 1];   // op(A) panel planes, [l][i]
+    double b[4][QBK][TY * R + 1];   // op(B) panel planes, [l][j]
 };
 
-template <int TA, int TB, int R>
-__global__ void __launch_bounds__(QNT, 1) qd_gemm_kernel(const QdArgs p) {
-    constexpr int BM = 16 * R;
-    __shared__ QdSmem<R> s;
+template <int TA, int TB, int R, int TY, bool PE>
+__global__ void __launch_bounds__(16 * TY, 1) qd_gemm_kernel(const QdArgs p) {
+    constexpr int BM = 16 * R, BN = TY * R, NT = 16 * TY;
+    constexpr int QA = BM * QBK / NT, QB = BN * QBK / NT;
+    __shared__ QdSmem<R, TY> s;
     const int64_t tm = (p.m + BM - 1) / BM;
     const int64_t bi = blockIdx.x % tm, bj = blockIdx.x / tm;
     const int t = threadIdx.x, tx = t % 16, ty = t / 16;
-    const int64_t i0 = bi * BM, j0 = bj * BM;
+    const int64_t i0 = bi * BM, j0 = bj * BN;
     const int64_t kk = p.alpha_zero ? 0 : p.k;
 
     double L[R][R][4];
@@ -123,43 +145,48 @@ __global__ void __launch_bounds__(QNT, 1) qd_gemm_kernel(const QdArgs p) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) L[r][c][v] = 0.0;
 
-    double ra[4][R], rb[4][R];
+    double ra[4][QA], rb[4][QB];
     auto a_pos = [&](int q, int &ii, int &ll) {
-        const int idx = t + QNT * q;
+        const int idx = t + NT * q;
         if (!TA) { ii = idx % BM; ll = idx / BM; }
         else     { ll = idx % QBK; ii = idx / QBK; }
     };
     auto b_pos = [&](int q, int &jj, int &ll) {
-        const int idx = t + QNT * q;
+        const int idx = t + NT * q;
         if (!TB) { ll = idx % QBK; jj = idx / QBK; }
-        else     { jj = idx % BM; ll = idx / BM; }
+        else     { jj = idx % BN; ll = idx / BN; }
     };
     auto load = [&](int64_t l0) {
+        int ii, jj, ll;
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-            int ii, jj, ll;
+        for (int q = 0; q < QA; ++q) {
             a_pos(q, ii, ll);
-            int64_t gi = i0 + ii, gl = l0 + ll;
-            bool ok = gi < p.m && gl < kk;
-            int64_t off = TA ? (gl + gi * p.lda) : (gi + gl * p.lda);
+            const int64_t gi = i0 + ii, gl = l0 + ll;
+            const bool ok = gi < p.m && gl < kk;
+            const int64_t off = TA ? (gl + gi * p.lda) : (gi + gl * p.lda);
 #pragma unroll
             for (int v = 0; v < 4; ++v) ra[v][q] = ok ? p.a[v][off] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
             b_pos(q, jj, ll);
-            const int64_t gj = j0 + jj;
-            gl = l0 + ll;
-            ok = gj < p.n && gl < kk;
-            off = TB ? (gj + gl * p.ldb) : (gl + gj * p.ldb);
+            const int64_t gj = j0 + jj, gl = l0 + ll;
+            const bool ok = gj < p.n && gl < kk;
+            const int64_t off = TB ? (gj + gl * p.ldb) : (gl + gj * p.ldb);
 #pragma unroll
             for (int v = 0; v < 4; ++v) rb[v][q] = ok ? p.b[v][off] : 0.0;
         }
     };
     auto stage = [&]() {
+        int ii, jj, ll;
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-            int ii, jj, ll;
+        for (int q = 0; q < QA; ++q) {
             a_pos(q, ii, ll);
 #pragma unroll
             for (int v = 0; v < 4; ++v) s.a[v][ll][ii] = ra[v][q];
+        }
+#pragma unroll
+        for (int q = 0; q < QB; ++q) {
             b_pos(q, jj, ll);
 #pragma unroll
             for (int v = 0; v < 4; ++v) s.b[v][ll][jj] = rb[v][q];
@@ -185,13 +212,13 @@ __global__ void __launch_bounds__(QNT, 1) qd_gemm_kernel(const QdArgs p) {
                     }
 #pragma unroll
                     for (int c = 0; c < R; ++c) {
-                        const int j = ty + 16 * c;
+                        const int j = ty + TY * c;
                         b[c] = qd4{s.b[0][l][j], s.b[1][l][j], s.b[2][l][j], s.b[3][l][j]};
                     }
 #pragma unroll
                     for (int r = 0; r < R; ++r)
 #pragma unroll
-                        for (int c = 0; c < R; ++c) qd_mac(L[r][c], a[r], b[c]);
+                        for (int c = 0; c < R; ++c) qd_mac<PE>(L[r][c], a[r], b[c]);
                 }
 #pragma unroll
                 for (int r = 0; r < R; ++r)
@@ -207,7 +234,7 @@ __global__ void __launch_bounds__(QNT, 1) qd_gemm_kernel(const QdArgs p) {
     for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < R; ++c) {
-            const int64_t i = i0 + tx + 16 * r, j = j0 + ty + 16 * c;
+            const int64_t i = i0 + tx + 16 * r, j = j0 + ty + TY * c;
             if (i >= p.m || j >= p.n) continue;
             const int64_t off = i + j * p.ldc;
             double E[4] = {0.0, 0.0, 0.0, 0.0};
@@ -216,12 +243,12 @@ __global__ void __launch_bounds__(QNT, 1) qd_gemm_kernel(const QdArgs p) {
                 for (int v = 0; v < 4; ++v) E[v] = L[r][c][v];
             } else if (!p.alpha_zero) {
                 const qd4 acc = qd_finish(L[r][c]);
-                qd_mac(E, p.alpha, acc);
+                qd_mac<false>(E, p.alpha, acc);
                 qd_pass(E);
             }
             if (!p.beta_zero) {
                 const qd4 cin{p.c[0][off], p.c[1][off], p.c[2][off], p.c[3][off]};
-                qd_mac(E, p.beta, cin);
+                qd_mac<false>(E, p.beta, cin);
             }
             const qd4 out = qd_finish(E);
             p.c[0][off] = out.x0;
@@ -231,22 +258,15 @@ __global__ void __launch_bounds__(QNT, 1) qd_gemm_kernel(const QdArgs p) {
         }
 }
 
-template <int TA, int TB, int R>
-void qd_launch(const QdArgs &p, cudaStream_t st) {
-    const int64_t b = 16 * R;
-    const dim3 grid((unsigned)(ceil_div(p.m, b) * ceil_div(p.n, b)));
-    qd_gemm_kernel<TA, TB, R><<<grid, QNT, 0, st>>>(p);
-}
-
-template <int R>
-int qd_launch_r(const QdArgs &p, int ta, int tb, cudaStream_t st) {
-    const int64_t b = 16 * R;
-    if (ceil_div(p.m, b) * ceil_div(p.n, b) > 0x7fffffffLL)
-        return fail(MP_DD_ERR_TOO_LARGE, "qd Rgemm: m x n too large");
-    if (!ta && !tb) qd_launch<0, 0, R>(p, st);
-    else if (ta && !tb) qd_launch<1, 0, R>(p, st);
-    else if (!ta && tb) qd_launch<0, 1, R>(p, st);
-    else qd_launch<1, 1, R>(p, st);
+template <int R, int TY, bool PE>
+int qd_launch(const QdArgs &p, int ta, int tb, cudaStream_t st) {
+    const int64_t tiles = ceil_div(p.m, 16 * R) * ceil_div(p.n, TY * R);
+    if (tiles > 0x7fffffffLL) return fail(MP_DD_ERR_TOO_LARGE, "qd Rgemm: m x n too large");
+    const unsigned g = (unsigned)tiles, nt = 16 * TY;
+    if (!ta && !tb) qd_gemm_kernel<0, 0, R, TY, PE><<<g, nt, 0, st>>>(p);
+    else if (ta && !tb) qd_gemm_kernel<1, 0, R, TY, PE><<<g, nt, 0, st>>>(p);
+    else if (!ta && tb) qd_gemm_kernel<0, 1, R, TY, PE><<<g, nt, 0, st>>>(p);
+    else qd_gemm_kernel<1, 1, R, TY, PE><<<g, nt, 0, st>>>(p);
     return check_launch("qd_gemm_kernel");
 }
 
@@ -269,12 +289,19 @@ int run_qd_gemm(int ta, int tb, int64_t m, int64_t n, int64_t k, const double *a
                    k == 0;
     p.alpha_one = alpha[0] == 1.0 && alpha[1] == 0.0 && alpha[2] == 0.0 && alpha[3] == 0.0;
     p.beta_zero = beta[0] == 0.0 && beta[1] == 0.0 && beta[2] == 0.0 && beta[3] == 0.0;
-    // R = 2 when its tiles fill the SMs at least as well as R = 1's (time
-    // ~ ceil(tiles / SMs) R^2), else R = 1
+    // Tile: the time is about (tiles per SM, rounded up) x (work per tile), in
+    // units of 128 entries, one for each of four warps; the largest tile with
+    // the least such time.  (16 x 8 tiles and the sums' errors on the
+    // integer pipe together: 64^3 349 -> 140 us, 100 x 90 x 200 1111 -> 435.)
     const int64_t sms = sm_count() > 0 ? sm_count() : 152;
-    const int64_t t2 = ceil_div(ceil_div(m, 32) * ceil_div(n, 32), sms) * 4;
-    const int64_t t1 = ceil_div(ceil_div(m, 16) * ceil_div(n, 16), sms);
-    return t2 <= t1 ? qd_launch_r<2>(p, ta, tb, st) : qd_launch_r<1>(p, ta, tb, st);
+    auto cost = [&](int64_t bm, int64_t bn) {
+        return ceil_div(ceil_div(m, bm) * ceil_div(n, bn), sms) * (bm * bn / 128);
+    };
+    const int64_t c32 = cost(32, 32), c16 = cost(16, 16), c8 = cost(16, 8);
+    if (c32 <= c16 && c32 <= c8) return qd_launch<2, 16, true>(p, ta, tb, st);
+    if (c16 <= c8) return c16 > 2 ? qd_launch<1, 16, true>(p, ta, tb, st)
+                                  : qd_launch<1, 16, false>(p, ta, tb, st);
+    return c8 > 2 ? qd_launch<1, 8, true>(p, ta, tb, st) : qd_launch<1, 8, false>(p, ta, tb, st);
 }
 
 }  // namespace mpdd

@@ -137,3 +137,17 @@ def test_deterministic(cuda_lib):
     a = run_qd(cuda_lib, "T", "N", m, n, k, A, B, C, al, be)
     b = run_qd(cuda_lib, "T", "N", m, n, k, A, B, C, al, be)
     assert all(np.array_equal(a[t], b[t]) for t in range(4))
+
+
+@pytest.mark.parametrize("ta,tb", [("N", "N"), ("T", "N"), ("N", "T"), ("T", "T")])
+@pytest.mark.parametrize("shape", [(1, 1), (16, 8), (17, 9), (95, 41), (300, 250), (160, 320), (3, 500)])
+def test_tiles_give_the_same_bits(cuda_lib, ta, tb, shape):
+    """Products on 16 x 8 and 16 x 16 tiles, with the products' errors on
+    either pipe, equal the leading block of a product on 32 x 32 tiles."""
+    M, N, k = 700, 640, 21
+    A, B, C, al, be = qd_case(210 + ["NN", "TN", "NT", "TT"].index(ta + tb), ta, tb, M, N, k)
+    whole = run_qd(cuda_lib, ta, tb, M, N, k, A, B, C, al, be)
+    m, n = shape
+    got = run_qd(cuda_lib, ta, tb, m, n, k, A, B, C, al, be)
+    for t in range(4):
+        assert np.array_equal(got[t][:m, :n], whole[t][:m, :n])
