@@ -51,11 +51,11 @@ METRIC = "dd-Rgemm/Rsyrk GFlops vs roofline; sliced vs plain at bound; p50/p99 s
 UNIT = "dd-GFlop/s"
 # nominal FP64 rate of GB300 (1.25 TFLOP/s counting an FMA as two flops) ->
 # 625 G FP64 instructions per second; a dd multiply-add in the GEMM kernels
-# costs 6.75 of them (1 DMUL + 2 DFMA + 3 DADD, FastTwoSum every 4 steps; the
-# rounding errors of the product and of the sum come from the integer pipe)
+# costs 6.25 of them (1 DMUL + 2 DFMA + 3 DADD, one more every 4 steps; the
+# rounding errors of the product and of the sums come from the integer pipe)
 NOMINAL_FP64_INSTR = 1.25e12 / 2
-FP64_OPS_PER_MAC = 6.75
-QD_OPS_PER_MAC = 39.25   # qd multiply-add: 37 FP64 operations + 2.25 for the level pass
+FP64_OPS_PER_MAC = 6.25
+QD_OPS_PER_MAC = 37.75   # qd multiply-add: 37 FP64 operations + 0.75 for the level pass
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from single ncu
 # captures of the current kernels (the summaries under profiles/ give the
 # commands): the plain Rgemm NN launch at 4096 and the band kernel of the
@@ -365,7 +365,7 @@ def plain_section(mp, torch, size, problems, r64, rmac=None):
     """The plain FP64 path on the step's three problems, one call each timed
     with CUDA events (after the split-precision runs on the same inputs).
     Fractions: of 2 R64 / 15 (the survey's accounting, R64 the measured FP64
-    FMA rate), of the FP64 pipe at the kernel's 6.75 instructions per
+    FMA rate), of the FP64 pipe at the kernel's 6.25 instructions per
     multiply-add, and of the measured rate of the all-FP64 multiply-add
     (9.75 instructions) with operands in registers (mp_dd_peak_ddmac), which
     the kernel exceeds: it forms rounding errors on the integer pipe."""
@@ -636,11 +636,10 @@ def run_default(args):
             "sections": sections,
             "cpu_baseline": cpu,
             "e2e": e2e,
-            # per step 10 + 10 + 9 launches: each Rgemm runs maxima x2, magnitude
-            # planes x2, the magnitude product, residues x2, the products, the
-            # reconstruction and the gated plain kernel; the Rsyrk one operand's
-            # worth of those plus two triangle tables
-            "gpu_launches": 29 * args.steps,
+            # per step three calls of 7 launches: maxima, magnitude planes, the
+            # magnitude product, residues, the products, the reconstruction and
+            # the gated plain kernel
+            "gpu_launches": 21 * args.steps,
             "clocks": clocks,
             "roofline": roofline,
             "summary": summary,
@@ -854,7 +853,7 @@ def routines_section(mp, torch, size):
     out[f"Rgetrf_{n}"]["info"] = int(info.item())
     del A, B, C, A0
     out.update(potrf_section(mp, torch, n, info))
-    # quad-double Rgemm (39.25 FP64 instructions per qd multiply-add)
+    # quad-double Rgemm (37.75 FP64 instructions per qd multiply-add)
     nq = min(n, 1024)
     gq = datagen.rng(5)
     Aq, Bq, Cq = (dev(datagen.qd_matrix(gq, nq, nq)) for _ in range(3))
@@ -1243,7 +1242,8 @@ def run_sliced_workload(args):
                 "h2d_bytes_per_step": 3 * mat, "d2h_bytes_per_step": mat,
                 "api": "Python binding mp_dd_Rgemm_" + ("crt" if crt else "sliced") +
                        ", pinned host buffers"},
-        "gpu_launches": 6 * args.steps, "clocks": clocks,  # maxima x2, split x2, products, recombination
+        # maxima, magnitudes, certificate, split (x2 sliced), products, epilogue, gated plain
+        "gpu_launches": (7 if crt else 8) * args.steps, "clocks": clocks,
     }
     if ranks.rank == 0:
         print(json.dumps(line), flush=True)

@@ -103,7 +103,7 @@ __device__ __forceinline__ void mac(dd &acc, dd a, dd b) {
 // the GEMM kernels call after every kRenormEvery steps of k (at l = 3, 7, 11,
 // ... counted from the start of k, so every kernel renormalises at the same
 // places).  4 + 3 + 2 = 9 FP64 operations per step, 9.75 with the
-// renormalisation.  Between renormalisations |acc.lo| stays within a few
+// renormalisation (3 + 1 + 2 and 0.25 with the errors on the integer pipe).  Between renormalisations |acc.lo| stays within a few
 // ulps of acc.hi, so each step's rounding error is at most ~(G+4) u^2
 // (|acc| + |a b|) with G = 4: within the Rgemm bound 4 k 2^-104 (...).  A
 // zero product leaves the state unchanged, so zero padding of k does not
@@ -118,9 +118,10 @@ constexpr int kRenormEvery = 4;
 // idle beside it, forms it from the significands with ~60 or ~40 instructions
 // of 2 cycles: modulo 2^64, because it is a small integer in the unit of the
 // smaller operand's last place (of the product of the last places).  A dd
-// multiply-add takes 6.75 FP64 instructions instead of 9.75: Rgemm 1101 x 700
-// x 905 12.52 ms with neither, 9.88 with the sum's error on the integer pipe,
-// 8.76 with the product's as well; 512 grouped problems 29.2, 23.0 and 20.4.
+// multiply-add takes 6.25 FP64 instructions instead of 9.75: Rgemm 1101 x 700
+// x 905 12.52 ms with none, 9.88 with the sum's error on the integer pipe,
+// 8.73 with the product's as well, 8.08 with the renormalisation's; 512
+// grouped problems 29.2, 23.0, 20.3 and 19.3 ms.
 // The result is the same bits; the host compares both with the FP64 forms
 // over the whole range in tests.
 
@@ -242,6 +243,16 @@ __device__ __forceinline__ void mac_mixed(dd &acc, dd a, dd b) {
     acc.hi = s;
     acc.lo = __dadd_rn(acc.lo, __dadd_rn(e1, e));
 }
+
+// The GEMM kernels' renormalisation: TwoSum, exact whatever cancellation has
+// left in hi, with the error from the integer pipe (one FP64 instruction
+// instead of FastTwoSum's three) or, the same bits, from the FP64 pipe.
+__device__ __forceinline__ void renorm_mixed(dd &acc) {
+    const double s = __dadd_rn(acc.hi, acc.lo);
+    acc.lo = sum_error(acc.hi, acc.lo, s);
+    acc.hi = s;
+}
+__device__ __forceinline__ void renorm_exact(dd &acc) { two_sum(acc.hi, acc.lo, acc.hi, acc.lo); }
 
 __device__ __forceinline__ void renorm(dd &acc) { fast_two_sum(acc.hi, acc.lo, acc.hi, acc.lo); }
 

@@ -7,10 +7,10 @@
 // operand is read through the stored triangle); MPBLAS semantics (manual
 // Sec. 7.3 and the routine table of Sec. 6).  Every multiply-add is dd
 // arithmetic: the exact product of the hi parts by FMA, the two cross
-// products, TwoSum into the accumulator, and a FastTwoSum renormalisation
+// products, TwoSum into the accumulator, and a TwoSum renormalisation
 // every 4 steps of k (dd_arith.cuh).
 //
-// On GB300 the FP64 pipe is the bottleneck by a wide margin (6.75 FP64
+// On GB300 the FP64 pipe is the bottleneck by a wide margin (6.25 FP64
 // instructions per dd multiply-add), so the kernel is organised to keep that
 // pipe busy and nothing else (large plain products go to the TMA-staged form
 // of this kernel, dd_gemm_tma.cu, whose per-entry arithmetic is identical):
@@ -220,7 +220,10 @@ __device__ __forceinline__ void plain_body(const GemmArgs &p, PlainSmem<S> &s) {
 #pragma unroll
                 for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int c = 0; c < R; ++c) renorm(acc[r][c]);
+                    for (int c = 0; c < R; ++c) {
+                        if constexpr (S::ALONE) renorm_exact(acc[r][c]);
+                        else renorm_mixed(acc[r][c]);
+                    }
             }
         }
     }
@@ -288,7 +291,7 @@ int launch_shape(const GemmArgs &p, cudaStream_t stream) {
 
 // Tile size: the time of a launch is about (tiles per SM, rounded up) x
 // (work per tile), in units of 128 entries -- one accumulator for each of four
-// warps, one per partition of the SM, 0.25 us per step of k (6.75 FP64
+// warps, one per partition of the SM, 0.23 us per step of k (6.25 FP64
 // instructions per multiply-add at 526 G/s over 152 SMs); the largest tile
 // with the least such time wins (the per-entry operation sequence, and hence
 // the result, does not depend on it).  16 x 8 and 32 x 4 tiles are one unit:
@@ -368,7 +371,7 @@ int launch_gemm_update(const GemmArgs &p, cudaStream_t stream) {
     if (p.m < kUpdateMin || p.n < kUpdateMin || p.k < kUpdateMin || p.k > ((int64_t)1 << 17) - 1 ||
         p.tri != 0 || p.alpha_zero || p.a2h != nullptr || p.sym_a || p.sym_b)
         return launch_gemm_plain(p, stream);
-    const double plain_us = 0.25 * (double)p.k * (double)plain_best_cost(p);
+    const double plain_us = 0.23 * (double)p.k * (double)plain_best_cost(p);
     if (crt_estimate_us(p.m, p.n, p.k) > 0.8 * plain_us) return launch_gemm_plain(p, stream);
     // allocations inside a stream capture would belong to the graph
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int r = 0; r < 4; ++r)
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) renorm(acc[r][c]);
+                    for (int c = 0; c < 4; ++c) renorm_mixed(acc[r][c]);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[s]);

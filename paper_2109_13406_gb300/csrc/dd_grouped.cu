@@ -18,7 +18,7 @@
 // Tile shapes: 16*RM x 16*RN with (RM, RN) in {(2,2), (4,2), (2,4), (1,1)};
 // the 256 threads form a 16 x 16 grid and each holds an RM x RN block of dd
 // accumulators.  Small shapes waste fewer zero-padded multiply-adds on
-// ragged problems (each costs the full 6.75 FP64 instructions); larger ones
+// ragged problems (each costs the full 6.25 FP64 instructions); larger ones
 // give each thread more independent chains.  All shapes fit 128 registers,
 // so two CTAs share an SM.
 #include <algorithm>
@@ -162,7 +162,7 @@ __device__ __forceinline__ void dd_tile(const mp_dd_gemm_desc &d, int64_t bi, in
 #pragma unroll
                 for (int r = 0; r < RM; ++r)
 #pragma unroll
-                    for (int c = 0; c < RN; ++c) renorm(acc[r][c]);
+                    for (int c = 0; c < RN; ++c) renorm_mixed(acc[r][c]);
             }
         }
     }

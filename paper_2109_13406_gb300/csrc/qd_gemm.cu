@@ -20,12 +20,13 @@
 //
 // The FP64 pipe bounds it, so the errors of the sums (sum_error) and, where
 // more than two warps share a partition of an SM (PE), of the products
-// (prod_error) are formed on the integer pipe, to the same bits: 37 FP64
-// operations per step plus 2.25 for the pass (71 with the errors on the FP64
-// pipe, 113 and 4.5 with Knuth's TwoSum).  331 x 300 x 257: 4.33 ms with
-// neither, 2.66 with the sums', 2.53 with both.  With two warps or fewer the
-// step's latency counts and the fused multiply-add is the better form of the
-// products' errors (150 x 140 x 300: 1.02 ms against 1.10).
+// (prod_error) and of the pass are formed on the integer pipe, to the same
+// bits: 37 FP64 operations per step plus 0.75 for the pass (71 and 2.25 with
+// the errors on the FP64 pipe, 113 and 4.5 with Knuth's TwoSum).  331 x 300 x
+// 257: 4.33 ms with none, 2.66 with the sums', 2.53 with the products' too,
+// 2.49 with the pass's.  With two warps or fewer the step's latency counts and
+// the FP64 forms are the better ones there (150 x 140 x 300: 1.02 ms against
+// 1.10 for the products; 64^3: 140 us against 145 for the pass).
 //
 // Tiles: 32 x 32 (2 x 2 qd accumulators per thread), 16 x 16 or 16 x 8 entries
 // of C per CTA, the four planes of the op(A) and op(B) panels staged through
@@ -89,19 +90,22 @@ __device__ __forceinline__ void qd_mac(double (&L)[4], const qd4 &a, const qd4 &
     L[3] = __dadd_rn(L[3], s);
 }
 
+template <bool PE>
 __device__ __forceinline__ void qd_pass(double (&L)[4]) {
-    two_sum(L[2], L[3], L[2], L[3]);
-    two_sum(L[1], L[2], L[1], L[2]);
-    two_sum(L[0], L[1], L[0], L[1]);
+#pragma unroll
+    for (int v = 2; v >= 0; --v) {
+        if constexpr (PE) two_sum_mixed(L[v], L[v + 1], L[v], L[v + 1]);
+        else two_sum(L[v], L[v + 1], L[v], L[v + 1]);
+    }
 }
 
 // Four non-overlapping components (|x_{t+1}| <= ulp(x_t) / 2) of the value of
 // the levels: three exact bottom-up passes concentrate the value in the
 // leading terms, then a top-down FastTwoSum pass separates them.
 __device__ __forceinline__ qd4 qd_finish(double (&L)[4]) {
-    qd_pass(L);
-    qd_pass(L);
-    qd_pass(L);
+    qd_pass<false>(L);
+    qd_pass<false>(L);
+    qd_pass<false>(L);
     fast_two_sum(L[0], L[1], L[0], L[1]);
     fast_two_sum(L[1], L[2], L[1], L[2]);
     fast_two_sum(L[2], L[3], L[2], L[3]);
@@ -223,7 +227,7 @@ __global__ void __launch_bounds__(16 * TY, 1) qd_gemm_kernel(const QdArgs p) {
 #pragma unroll
                 for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int c = 0; c < R; ++c) qd_pass(L[r][c]);
+                    for (int c = 0; c < R; ++c) qd_pass<PE>(L[r][c]);
             }
         }
     }
@@ -244,7 +248,7 @@ __global__ void __launch_bounds__(16 * TY, 1) qd_gemm_kernel(const QdArgs p) {
             } else if (!p.alpha_zero) {
                 const qd4 acc = qd_finish(L[r][c]);
                 qd_mac<false>(E, p.alpha, acc);
-                qd_pass(E);
+                qd_pass<false>(E);
             }
             if (!p.beta_zero) {
                 const qd4 cin{p.c[0][off], p.c[1][off], p.c[2][off], p.c[3][off]};
