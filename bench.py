@@ -56,12 +56,10 @@ UNIT = "dd-GFlop/s"
 NOMINAL_FP64_INSTR = 1.25e12 / 2
 FP64_OPS_PER_MAC = 6.25
 QD_OPS_PER_MAC = 37.75   # qd multiply-add: 37 FP64 operations + 0.75 for the level pass
-# dram__bytes_read.sum + dram__bytes_write.sum per launch, from single ncu
-# captures of the current kernels (the summaries under profiles/ give the
-# commands): the plain Rgemm NN launch at 4096 and the band kernel of the
-# CRT form at 8192 (one-pass metrics, 30.20 GB read and 2.14 GB written,
+# dram__bytes_read.sum + dram__bytes_write.sum per launch, from a single ncu
+# capture (the summaries under profiles/ give the command): the band kernel of
+# the CRT form at 8192 (one-pass metrics, 30.20 GB read and 2.14 GB written,
 # against 8.59 and 2.15 GB algorithmic)
-PLAIN_NN_4096_DRAM_BYTES = 3626772736 + 278080000
 BAND_CRT_8192_DRAM_BYTES = 30.20e9 + 2.14e9
 
 
@@ -291,9 +289,7 @@ def run_plain_workload(args):
         "peak_source": "nominal GB300 FP64 1.25 TFLOP/s = 625 G FP64 instr/s (derived)",
         "peak_measured_fp64_microbench": (peak_fp64 / 1e9) if peak_fp64 else None,
         "frac_of_measured": (achieved / (peak_fp64 / 1e9)) if peak_fp64 else None,
-        # DRAM bytes of one Rgemm NN launch at 4096 from one ncu capture of
-        # this kernel (profiles/dd_gemm_plain_4096.md); None at other sizes
-        "traffic": PLAIN_NN_4096_DRAM_BYTES if size == 4096 else None,
+        "traffic": None,   # no capture of the current tiles
         "fp64_instr_per_dd_mac": FP64_OPS_PER_MAC,
     }
     e2e = None

@@ -12,18 +12,17 @@
 //
 // On GB300 the FP64 pipe is the bottleneck by a wide margin (6.25 FP64
 // instructions per dd multiply-add), so the kernel is organised to keep that
-// pipe busy and nothing else (large plain products go to the TMA-staged form
-// of this kernel, dd_gemm_tma.cu, whose per-entry arithmetic is identical):
-// each CTA owns a 16R x 16R tile of C (R = 4, 2 or 1), each thread an R x R
-// block of dd accumulators (or a 16 x 8 or 32 x 4 tile of one entry per
-// thread, for products that leave SMs without a 16 x 16 tile: four warps, one
-// per partition of the SM, so a step of k takes half as long), and the hi/lo planes
+// pipe busy and nothing else: each CTA owns a 16 x 16 tile of C, one dd
+// accumulator per thread (a 16 x 8 or 32 x 4 tile for products that leave SMs
+// without a 16 x 16 tile: four warps, one per partition of the SM, so a step of
+// k takes half as long; 64 x 64 tiles of 4 x 4 accumulators a thread for
+// launches behind a certificate, which mostly return at once and cost their
+// CTA count, where the TMA-staged form of this kernel, dd_gemm_tma.cu, whose
+// per-entry arithmetic is identical, does not apply), and the hi/lo planes
 // of the op(A) and op(B) panels are staged through shared memory 16 columns
 // of k at a time with a register prefetch of the next panel.  One SM's FP64
-// pipe issues only 2 lanes per clock, so a few warps keep it busy whatever R
-// is; the launch picks R so that the tiles fill all SMs (large products:
-// 64 x 64, the fewest operand loads per multiply-add; thin ones: smaller
-// tiles, more CTAs).  Loads are zero-filled outside the matrices; a zero product leaves
+// pipe issues only 2 lanes per clock, so one chain a warp keeps it busy.
+// Loads are zero-filled outside the matrices; a zero product leaves
 // a normalised accumulator bitwise unchanged, so the per-entry operation
 // sequence (l = 0, 1, ..., k-1) and hence the result are independent of the
 // tiling.  Rsyrk uses the same instantiation as Rgemm(N, T) / (T, N) over
@@ -292,13 +291,17 @@ int launch_shape(const GemmArgs &p, cudaStream_t stream) {
 // Tile size: the time of a launch is about (tiles per SM, rounded up) x
 // (work per tile), in units of 128 entries -- one accumulator for each of four
 // warps, one per partition of the SM, 0.23 us per step of k (6.25 FP64
-// instructions per multiply-add at 526 G/s over 152 SMs); the largest tile
-// with the least such time wins (the per-entry operation sequence, and hence
-// the result, does not depend on it).  16 x 8 and 32 x 4 tiles are one unit:
-// they halve the time of products with fewer 16 x 16 tiles than SMs, and of
-// those with few columns, whose 16-column tiles are mostly padding: Rgemm 96 x
-// 80 x 70 58.0 -> 31.9 us; Cholesky and solve of order 3000, whose updates
-// have a depth of 64, 36.5 -> 33.2 ms.
+// instructions per multiply-add at 526 G/s over 152 SMs); the per-entry
+// operation sequence, and hence the result, does not depend on the tile.
+// 16 x 16 tiles never take longer by that count than larger ones, and their
+// six or more warps a partition hide the multiply-add's long integer part best: 8192
+// x 8192 x 256 takes 197.2 ms on them, 198.1 on 32 x 32 tiles, 212 on 64 x 64
+// and 222 on the TMA-staged 64 x 64 (two warps a partition); 1216 x 1024 x 512
+// 7.28, 7.33, 7.86 and 8.27 ms.  16 x 8 and 32 x 4 tiles are one unit: they
+// halve the time of products with fewer 16 x 16 tiles than SMs, and of those
+// with few columns, whose 16-column tiles are mostly padding: Rgemm 96 x 80 x
+// 70 58.0 -> 31.9 us; Cholesky and solve of order 3000, whose updates have a
+// depth of 64, 36.5 -> 33.2 ms.
 int64_t plain_tile_cost(const GemmArgs &p, int r) {
     const int64_t sms = sm_count() > 0 ? sm_count() : 152;
     return ceil_div(tile_count(p, 16 * r, 16 * r), sms) * 2 * r * r;
@@ -306,20 +309,18 @@ int64_t plain_tile_cost(const GemmArgs &p, int r) {
 
 namespace {
 
-enum PlainTile { kTile64, kTile32, kTile16, kTileHalf, kTileTall };
+enum PlainTile { kTile16, kTileHalf, kTileTall };
 
 PlainTile plain_tile(const GemmArgs &p, int64_t *cost) {
     const int64_t sms = sm_count() > 0 ? sm_count() : 152;
-    PlainTile best = kTile64;
-    *cost = plain_tile_cost(p, 4);
+    PlainTile best = kTile16;
+    *cost = plain_tile_cost(p, 1);
     auto offer = [&](PlainTile t, int64_t c) {
         if (c < *cost) {
             *cost = c;
             best = t;
         }
     };
-    offer(kTile32, plain_tile_cost(p, 2));
-    offer(kTile16, plain_tile_cost(p, 1));
     offer(kTileHalf, ceil_div(tile_count(p, Half::BM, Half::BN), sms));
     if (p.tri == 0) offer(kTileTall, ceil_div(tile_count(p, Tall::BM, Tall::BN), sms));
     return best;
@@ -419,9 +420,7 @@ int launch_gemm_plain(const GemmArgs &p, cudaStream_t stream) {
             return cost <= 1 ? launch_shape<TallAlone>(p, stream) : launch_shape<Tall>(p, stream);
         case kTileHalf:
             return cost <= 1 ? launch_shape<HalfAlone>(p, stream) : launch_shape<Half>(p, stream);
-        case kTile16: return launch_shape<Square<1>>(p, stream);
-        case kTile32: return launch_shape<Square<2>>(p, stream);
-        default: return launch_shape<Square<4>>(p, stream);
+        default: return launch_shape<Square<1>>(p, stream);
     }
 }
 

@@ -321,10 +321,12 @@ int plain_staging() { return g_staging.load(); }
 // The TMA-staged kernel applies to plain Rgemm / Rsyrk products (no second
 // product, no symmetric operand, alpha != 0) whose planes start on 16-byte
 // boundaries with even leading dimensions (the copy engine's stride rule).
-// Automatically it takes the Rgemm products large enough for 64 x 64 tiles
-// (measured on GB300: 85.8 dd-GFlop/s at 4096, as the register-staged
-// kernel; at 2048 and for the Rsyrk triangle the smaller register-staged
-// tiles are faster).  Returns 1 when it launched (or failed to: *rc), 0 when
+// Automatically it takes only the gated Rgemm launches behind a certificate
+// that are large enough for 64 x 64 tiles: with the gate closed its one CTA per
+// SM returns at once.  Plain products run faster on the register-staged 16 x
+// 16 tiles, whose six or more warps a partition cover the integer part of the
+// multiply-add that this kernel's two do not (8192 x 8192 x 256: 197 ms against
+// 222).  Returns 1 when it launched (or failed to: *rc), 0 when
 // the caller should use the register-staged kernels.
 int try_launch_gemm_tma(const GemmArgs &p, cudaStream_t st, int *rc) {
     if (g_staging.load() == 1) return 0;
@@ -337,10 +339,9 @@ int try_launch_gemm_tma(const GemmArgs &p, cudaStream_t st, int *rc) {
     const int64_t tiles = p.tri == 0 ? tm * tn : tm * (tm + 1) / 2;
     const int sms = sm_count() > 0 ? sm_count() : 152;
     if (g_staging.load() == 0) {
-        // automatic: Rgemm products whose 64 x 64 tiling is within 1 % of the
-        // best tile size's busiest-SM time (thinner products and the Rsyrk
-        // triangle run faster on the smaller register-staged tiles)
-        if (p.tri != 0 || tiles < sms) return 0;
+        // automatic: gated Rgemm launches whose 64 x 64 tiling is within 1 % of
+        // the best tile size's busiest-SM time
+        if (p.gate == nullptr || p.tri != 0 || tiles < sms) return 0;
         const int64_t best = plain_best_cost(p);
         if (100 * plain_tile_cost(p, 4) > 101 * best) return 0;
     }
