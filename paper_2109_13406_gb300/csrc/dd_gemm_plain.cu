@@ -354,8 +354,9 @@ int launch_plain_fallback(const GemmArgs &p, const SplitPlan &plan, cudaStream_t
 
 // Where the residue form takes an update of a factorisation or solve over
 // from the plain kernel: where its estimated time is at most four fifths of
-// the plain kernel's busiest SM's (plain_tile_cost).  LU and solve of order 1536 with 500 right-hand sides: 71.0 ms with every
-// update on the FP64 pipe, 31.9 so.
+// the plain kernel's busiest SM's (plain_tile_cost).  LU and solve of order 1536
+// with 500 right-hand sides: 71.0 ms with every update on the FP64 pipe
+// (9.75 instructions a multiply-add), 31.9 so.
 // The inner dimension and both outer ones have to reach kUpdateMin: below it
 // the time is latency either way, and a solve's or a factorisation's result
 // then does not depend on how many columns go with it.
