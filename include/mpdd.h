@@ -30,8 +30,8 @@
  *                 LAPACK routine) is illegal -- the xerbla convention the
  *                 manual's MPBLAS tests compare (Sec. 8.1)
  *   1000 + e      CUDA runtime error e while launching or copying
- *   2001          a device-side wait ran out of time (the kernel stopped
- *                 early; the output is undefined)
+ *   2001          a device-side wait ran out of time (see
+ *                 mp_dd_workspace_status)
  *   2002          requested size beyond a documented limit
  *   2003          workspace too small
  *   2004          the CUDA extension cannot run (no device / wrong arch)
@@ -239,9 +239,9 @@ int mp_dd_Rsyrk_host(const char *uplo, const char *trans, int64_t n, int64_t k, 
  * large products; the large ones (all three dimensions at least 96) run in
  * residue form on the tensor cores at an operand width that rounds within 2
  * u^2 (u = 2^-53) of |A||X| + |B| entry by entry, or on the FP64 pipe when no
- * width does, while the stream is being captured, or when their workspace (at
- * most 4 GiB, stream-ordered, from a pool of the library that keeps at most 2
- * GiB between calls) cannot be had.  Accuracy: the componentwise backward error of
+ * width does (or a device wait of the update gave up), while the stream is
+ * being captured, or when their workspace (at most 4 GiB, stream-ordered, from
+ * a pool of the library that keeps at most 2 GiB between calls) cannot be had.  Accuracy: the componentwise backward error of
  * substitution, |op(A) X - alpha B| <= 4 (n_A + 2) 2^-104 (|op(A)||X| +
  * |alpha B|), n_A the order of A; a zero diagonal entry gives Inf/NaN as
  * DTRSM does (no check).  Asynchronous on the current stream.
@@ -441,7 +441,8 @@ int mp_qd_Rgemm(const char *transa, const char *transb, int64_t m, int64_t n, in
 /* What the last split-precision call on a workspace did (no counterpart in
  * the manual): the certificate's outcome and a guaranteed error estimate. */
 typedef struct mp_dd_split_info_s {
-    int status;          /* 0, or 2001 when a device wait timed out (C undefined) */
+    int status;          /* 0, or 2001 when a device wait timed out (the plain
+                            FP64 kernel computed C) */
     int form;            /* 1 digit slices, 2 residues; 0: no product was formed
                             (alpha = 0 or k = 0: C := beta C) */
     int width_bits;      /* bits W each operand entry was rounded to (8 S, or
@@ -524,7 +525,7 @@ int mp_dd_Rgemm_sliced_noalloc(const char *transa, const char *transb, int64_t m
 
 /* mp_dd_split_report for the built-in scratch array of the current device:
  * the status word (0, or 2001 when a device wait of the last
- * mp_dd_Rgemm_sliced_noalloc call timed out) and its certificate.  Waits for
+ * mp_dd_Rgemm_sliced_noalloc call timed out and the plain kernel computed C) and its certificate.  Waits for
  * the calling thread's current stream.  Errors: -1 info NULL, 1000 + e. */
 int mp_dd_noalloc_report(mp_dd_split_info *info);
 
@@ -591,7 +592,9 @@ int mp_dd_crt_layout(int64_t m, int64_t n, int64_t k, size_t offsets[48], int *m
 int mp_dd_sliced_layout(int64_t m, int64_t n, int64_t k, int slices, size_t offsets[8]);
 
 /* Read the device status word of a workspace (waits for the calling
- * thread's current stream, then copies). */
+ * thread's current stream, then copies): 0, or 2001 when a device wait of the
+ * call timed out; the call's certificate is then taken back and the plain
+ * FP64 kernel, launched behind it, computes C. */
 int mp_dd_workspace_status(const void *workspace, int *status);
 
 /* Fill *info from the header of `workspace` after a mp_dd_Rgemm_sliced,

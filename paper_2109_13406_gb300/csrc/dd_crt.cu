@@ -994,7 +994,7 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     ba.n_pad = L.n_pad;
     ba.P = nullptr;
     ba.R = RES;
-    ba.status = &hdr->status;
+    ba.hdr = hdr;
     ba.diag = 1;
     ba.tri = p.tri;
     ba.plan = plan;

@@ -965,7 +965,7 @@ __global__ void __launch_bounds__(BandCfg<TN, PAIR>::THREADS, 1)
     } else if (warp == 1) {
         tmem_dealloc(tmem, kTmemCols);
     }
-    if (threadIdx.x == 0 && *abort_flag) atomicExch(p.status, MP_DD_ERR_TIMEOUT);
+    if (threadIdx.x == 0 && *abort_flag) give_up(p.hdr);
     if (PAIR) cluster_sync();   // no CTA leaves while its peer may still signal it
 }
 
@@ -1308,7 +1308,7 @@ int launch_certificate(const GemmArgs &p, void *MA, void *MB, int64_t m_pad, int
     ba.tiles_n = (int)(n_pad / TN);
     ba.m_pad = m_pad;
     ba.n_pad = n_pad;
-    ba.status = &hdr->status;
+    ba.hdr = hdr;
     ba.diag = 1;
     ba.tri = p.tri;
     ba.mag = 1;
@@ -1411,7 +1411,7 @@ int run_sliced(const GemmArgs &p, int slices, void *ws, size_t ws_bytes, cudaStr
     ba.R = nullptr;
     ba.diag = 0;
     ba.split = (int64_t)ba.tiles_m * ba.tiles_n < kSplitTiles;
-    ba.status = &hdr->status;
+    ba.hdr = hdr;
     ba.plan = plan;
     if ((rc = launch_band(tmA, tmB, ba, TN, st, &tmB_half))) return rc;
     timer().mark(2, st);

@@ -10,6 +10,8 @@
 
 #include <cstdint>
 
+#include "mpdd.h"
+
 namespace mpdd {
 
 // ------------------------------------------------------------------ certificate
@@ -37,7 +39,7 @@ constexpr int kMaxCand = 3;
 
 // Workspace header (the first bytes of every split-precision workspace).
 struct SplitHeader {
-    int status;                        // 0, or 2001 when a device wait timed out
+    int status;                        // 0, or 2001 when a device wait timed out (see give_up)
     int form;                          // 1 digit slices, 2 residues; 0: no product formed
     int ncand;                         // candidate widths, ascending
     int reserved;
@@ -66,7 +68,7 @@ struct PlanPick {
 
 // (Every index below is a constant after unrolling, so the plan stays in the
 // kernel's parameter space instead of being copied to local memory.)
-__device__ __forceinline__ PlanPick plan_choice(const SplitPlan &pl) {
+__host__ __device__ __forceinline__ PlanPick plan_choice(const SplitPlan &pl) {
     if (pl.dmin == nullptr) return PlanPick{0, pl.count[0], pl.width[0]};
     const unsigned int d = *reinterpret_cast<const volatile unsigned int *>(pl.dmin);
     PlanPick r{-1, 0, 0};
@@ -74,6 +76,21 @@ __device__ __forceinline__ PlanPick plan_choice(const SplitPlan &pl) {
     for (int c = kMaxCand - 1; c >= 0; --c)
         if (c < pl.ncand && d >= pl.thr[c]) r = PlanPick{c, pl.count[c], pl.width[c]};
     return r;
+}
+
+// A device wait of one of the call's products gave up: the status, and the
+// certificate taken back (no margin reaches a candidate's threshold), so that
+// the kernels behind it leave C alone and the plain kernel computes it.  Calls
+// whose header nobody reads (updates of a solve or factorisation) are right
+// all the same.
+__host__ __device__ inline void give_up(SplitHeader *hdr) {
+#if defined(__CUDA_ARCH__)
+    atomicExch(&hdr->status, MP_DD_ERR_TIMEOUT);
+    atomicExch(&hdr->dmin, 0u);
+#else
+    hdr->status = MP_DD_ERR_TIMEOUT;
+    hdr->dmin = 0u;
+#endif
 }
 
 // One band-product launch.  Triangle mode (diag = 0): band b sums the pairs
@@ -91,7 +108,7 @@ struct BandArgs {
     int64_t m_pad, n_pad;
     int32_t *P;   // [S][n_pad][m_pad] (triangle mode)
     uint8_t *R;   // [S][n_pad][m_pad] (diagonal mode)
-    int *status;
+    SplitHeader *hdr;   // of the call: give_up() when a wait runs out
     int diag;
     int split;    // triangle mode: work items of one band each (else all bands of a tile)
     int tri;      // diagonal / magnitude mode: 1 / 2 = only the upper / lower triangle

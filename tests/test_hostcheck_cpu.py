@@ -11,6 +11,8 @@ compiled as host code with nvcc.
   overflow to a correctly signed infinity.
 * two_sum (dd_arith.cuh), which orders its operands by their leading words:
   equal to Knuth's TwoSum over the whole binary64 range (hostcheck/two_sum.cu).
+* A device wait that gives up takes its call's certificate back, so that the
+  plain kernel computes C (hostcheck/give_up.cu).
 """
 from __future__ import annotations
 
@@ -70,6 +72,15 @@ def test_prod_error_equals_the_fma(tmp_path):
     assert r.returncode == 0, r.stdout + r.stderr
     pairs, bad = (int(x) for x in r.stdout.split()[1::2])
     assert pairs == 6000000 and bad == 0
+
+
+def test_a_wait_that_gave_up_leaves_c_to_the_plain_kernel(tmp_path):
+    exe = str(tmp_path / "give_up")
+    _build(os.path.join(HERE, "hostcheck", "give_up.cu"), exe, shared=False)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    cases, bad = (int(x) for x in r.stdout.split()[1::2])
+    assert cases == 21 and bad == 0
 
 
 def test_words_to_dd_rounding(tmp_path):
