@@ -1120,6 +1120,13 @@ struct PanelWs {
     PanelCand cand[2][kPanelMaxG];
 };
 
+// A wait of this CTA gave up, or it saw that another's had: its rows are not
+// finished.  Every such CTA says so, as the others may have got past the last
+// column without looking at the abort word.
+__device__ __forceinline__ void panel_gave_up(int64_t *info) {
+    atomicExch(reinterpret_cast<unsigned long long *>(info), ~0ull);   // -1
+}
+
 // Thread 0 of each CTA: arrive, then wait for all G arrivals of barrier b
 // (b = 1, 2, ...).  false: the wait gave up or another CTA did.
 __device__ bool panel_grid_sync(PanelWs *ws, int G, unsigned int b) {
@@ -1221,7 +1228,7 @@ __global__ void __launch_bounds__(kPanelThreads) getrf_panel_kernel(
         if (tid == 0) s_stop = panel_grid_sync(ws, G, (unsigned int)(jj + 1)) ? 0 : 1;
         __syncthreads();
         if (s_stop) {
-            if (c == 0 && tid == 0) *info = -1;
+            if (tid == 0) panel_gave_up(info);
             return;
         }
         // 2. warp 0: the pivot, the best published key (the same in every
@@ -1483,7 +1490,7 @@ __global__ void __launch_bounds__(kPanelThreads) getrf_panel_smem_kernel(
         }
         __syncthreads();
         if (s_stop) {
-            if (c == 0 && tid == 0) *info = -1;
+            if (tid == 0) panel_gave_up(info);
             return;
         }
         const int64_t p = s_p;               // >= j: every column has rows j .. m-1
