@@ -1,6 +1,7 @@
 // Binary floating point with a 128-bit significand held in four 32-bit
 // integer registers: the exact rounding of the residue (CRT) form's
-// reconstructed integer to dd.
+// reconstructed integer to dd, and that of the digit form's recombined one
+// (signed160_to_dd, which keeps all 160 bits).
 //
 // The reconstructed product Z 2^s is an exact multiword integer; its leading
 // 128 bits are taken with integer instructions and rounded to the nearest dd
@@ -248,6 +249,73 @@ BF_HD void signed_words_to_dd(const uint32_t (&S)[NW], int s, double &hi, double
     const uint64_t nh = ((uint64_t)(n2 >> 11) << 32) | nl;
     lo = bitsd((((uint64_t)(uint32_t)(e - 53 - lz2 + 1022) << 52) + nh + (up2 ? 1 : 0)) |
                ((uint64_t)((mask & 1u) ^ (up ? 1u : 0u)) << 63));
+}
+
+// The nearest dd of V 2^s for a two's complement V of six words, |V| < 2^160:
+// hi = RN(V 2^s), lo = RN(V 2^s - hi), every bit of V taking part (barring
+// results near the ends of the exponent range).  The magnitude's five words
+// are formed first, so both signs go the same way: 128 leading bits and a tail
+// word of those below.  Written out is the usual case (V's leading bit in its
+// fifth word, the remainder's among its first 32, exponents well inside the
+// normal range); the general path covers the rest.
+BF_HD void signed160_to_dd(const uint32_t (&S)[6], int s, double &hi, double &lo) {
+    const uint32_t neg = S[5] >> 31, mask = 0u - neg;
+    uint32_t z[5], c = neg;
+#pragma unroll
+    for (int t = 0; t < 5; ++t) {
+        const uint64_t v = (uint64_t)(S[t] ^ mask) + c;
+        z[t] = (uint32_t)v;
+        c = (uint32_t)(v >> 32);
+    }
+    const int lz = clz32(z[4]);
+    const int e = 159 - lz + s;
+    const uint32_t m3 = fshl(z[3], z[4], lz), m2 = fshl(z[2], z[3], lz), m1 = fshl(z[1], z[2], lz),
+                   m0 = fshl(z[0], z[1], lz), mt = fshl(0u, z[0], lz);
+    // hi: the leading 53 bits, rounded by the next one and the rest
+    const uint32_t r2 = m2 & 0x7FFu;
+    const uint64_t r0 = ((uint64_t)m0 << 32) | mt;
+    const bool rest = (m1 | m0 | mt) != 0;
+    const uint32_t ml = (m3 << 21) | (m2 >> 11);
+    const bool up = (r2 >> 10) && ((r2 & 0x3FFu) != 0 || rest || (ml & 1u));
+    // lo: the remainder (107 bits), or 2^107 minus it when rounded up
+    const uint64_t l0t = up ? 0 - r0 : r0;
+    const uint32_t l0 = (uint32_t)(l0t >> 32), lt = (uint32_t)l0t;
+    const uint32_t l1 = up ? 0u - m1 - (r0 != 0) : m1;
+    const uint32_t l2 = up ? 0x800u - r2 - rest : r2;
+    const uint32_t a2 = (l2 << 21) | (l1 >> 11), a1 = (l1 << 21) | (l0 >> 11),
+                   a0 = (l0 << 21) | (lt >> 11), at = lt << 21;
+    const uint32_t lneg = neg ^ (up ? 1u : 0u);
+    if (z[4] == 0 || a2 == 0 || e < -900 || e > 1000) {
+        if (z[4] == 0) {   // 128 bits: to_dd has them all
+            const uint32_t w[4] = {z[0], z[1], z[2], z[3]};
+            to_dd(from_words<4>(w, neg, s), hi, lo);
+            return;
+        }
+        hi = make_double((((uint64_t)m3 << 21) | (m2 >> 11)) + (up ? 1 : 0), e - 52, neg);
+        uint32_t m[4] = {lt, l0, l1, l2};
+        const int lz2 = clz128(m);
+        if (lz2 == 128) {
+            lo = 0.0;
+            return;
+        }
+        shl128(m, lz2);
+        uint64_t mh = ((uint64_t)m[3] << 21) | (m[2] >> 11);
+        if (((m[2] >> 10) & 1u) && (((m[2] & 0x3FFu) | m[1] | m[0]) != 0 || (mh & 1u))) mh += 1;
+        // the remainder's leading bit is bit 127 - lz2 of the frame 2^(e - 159)
+        lo = make_double(mh, e - 159 + (127 - lz2) - 52, lneg);
+        return;
+    }
+    const uint64_t mh = ((uint64_t)(m3 >> 11) << 32) | ml;   // 2^52 <= mh < 2^53
+    hi = bitsd((((uint64_t)(uint32_t)(e + 1022) << 52) + mh + (up ? 1 : 0)) |
+               ((uint64_t)neg << 63));
+    const int lz2 = clz32(a2);
+    const uint32_t n2 = fshl(a1, a2, lz2), n1 = fshl(a0, a1, lz2), n0 = fshl(at, a0, lz2),
+                   nt = fshl(0u, at, lz2);
+    const uint32_t nl = (n2 << 21) | (n1 >> 11);
+    const bool up2 = ((n1 >> 10) & 1u) && (((n1 & 0x3FFu) | n0 | nt) != 0 || (nl & 1u));
+    const uint64_t nh = ((uint64_t)(n2 >> 11) << 32) | nl;
+    lo = bitsd((((uint64_t)(uint32_t)(e - 53 - lz2 + 1022) << 52) + nh + (up2 ? 1 : 0)) |
+               ((uint64_t)lneg << 63));
 }
 
 #undef BF_HD

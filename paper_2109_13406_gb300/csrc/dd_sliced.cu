@@ -985,11 +985,15 @@ struct RecArgs {
 // V = sum_b P_b 256^(S-1-b) as a two's complement integer of six words: four
 // bands at a time make a signed 64-bit digit of base 2^32 (|P_b| < 2^31), the
 // carries run up the digits; S is padded to 16 bands, so the value is V
-// 256^(16 - S).  Rounded to the nearest dd by integer operations (as the
-// residue form's), then the alpha / beta epilogue.  Bound by HBM: 4 S bytes of
-// band sums, C and the result per entry.  192-bit shifts per band and a
-// rounding through the FP64 pipe's conversions took 150 us at 2048 x 2048
-// (S = 14), this 103 (161 and 115 with alpha).
+// 256^(16 - S), below 2^152.  Rounded to the nearest dd by integer operations,
+// all of V's bits among them, then the alpha / beta epilogue.  Bound by integer
+// issue, and with general alpha and beta by the FP64 pipe, against 45 us of
+// HBM time at 2048 x 2048 (S = 14: 4 S bytes of band sums and the result per
+// entry): there this phase takes 96 us with alpha = 1 and beta = 0, 103 with
+// general alpha, 195 with both.  A rounding written for the residue form's
+// words, whose straight-line path no negative sum could take, made it 111,
+// 117 and 199; 192-bit shifts per band and a rounding through the FP64 pipe's
+// conversions 150 and 161.
 __global__ void __launch_bounds__(256) recombine_kernel(const RecArgs p) {
     chain_begin();
     const PlanPick pk = plan_choice(p.plan);
@@ -1022,7 +1026,7 @@ __global__ void __launch_bounds__(256) recombine_kernel(const RecArgs p) {
         Z[5] = (uint32_t)(carry >> 32);
         const int sc = scale_exponent(__ldg(p.rmax + i)) + scale_exponent(__ldg(p.cmax + j)) - 136;
         dd r;
-        bigf::signed_words_to_dd<6>(Z, sc, r.hi, r.lo);
+        bigf::signed160_to_dd(Z, sc, r.hi, r.lo);
         if (!p.alpha_one) r = mul(dd{p.alpha.hi, p.alpha.lo}, r);
         if (!p.beta_zero) r = add_sloppy(r, mul(dd{p.beta.hi, p.beta.lo}, c));
         p.ch[off] = r.hi;

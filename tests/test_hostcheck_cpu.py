@@ -9,6 +9,9 @@ compiled as host code with nvcc.
   value when Z has at most 128 significant bits, and |hi + lo - Z 2^s| stays
   within (2^-106 + 2^-126) |Z 2^s| (plus the subnormal spacing), with
   overflow to a correctly signed infinity.
+* The digit form's rounding of the recombined integer V 2^s: hi and lo are the
+  nearest binary64 numbers of the value and of what hi leaves, both signs
+  (hostcheck/bands_dd.cu).
 * two_sum (dd_arith.cuh), which orders its operands by their leading words:
   equal to Knuth's TwoSum over the whole binary64 range (hostcheck/two_sum.cu).
 * A device wait that gives up takes its call's certificate back, so that the
@@ -138,3 +141,42 @@ def test_signed_words_to_dd_is_the_general_rounding(tmp_path):
         lib.words_to_dd(words, neg, s, a)
         lib.signed_words_to_dd(words, neg, s, b)
         assert bytes(a) == bytes(b), (hex(Z), neg, s, list(a), list(b))
+
+
+def test_bands_to_dd_is_the_nearest_dd(tmp_path):
+    """V of up to 159 bits, as 14 or 15 bands of digit products give it: hi is
+    V 2^s rounded to nearest and lo the rest rounded to nearest, whatever lies
+    below the leading 128 bits.  Ties of both roundings that only the tail
+    decides, all-one and zero words, both signs; exponents past the normal
+    range within two subnormal units, or an infinity of V's sign."""
+    so = str(tmp_path / "bands_dd.so")
+    _build(os.path.join(HERE, "hostcheck", "bands_dd.cu"), so, shared=True)
+    lib = ctypes.CDLL(so)
+    U6 = ctypes.c_uint32 * 6
+    D2 = ctypes.c_double * 2
+    lib.bands_to_dd.argtypes = [U6, ctypes.c_int, D2]
+    g = random.Random(13)
+    fill = [0, 0xFFFFFFFF, 0x80000000, 1, 0x7FF, 0x400, 0x800]
+    for it in range(60000):
+        nbits = g.choice([0, 1, 53, 54, 96, 107, 127, 128, 129, 140, 145, 150, 157, 158, 159])
+        Z = sum((g.choice(fill) if g.random() < 0.3 else g.getrandbits(32)) << (32 * t)
+                for t in range(5)) & ((1 << nbits) - 1)
+        if nbits:
+            Z |= 1 << (nbits - 1)
+        if nbits > 128 and g.random() < 0.5:
+            # a tie of hi (or one of lo) in the leading 128 bits, 0 or 1 below
+            low = nbits - 53 if g.random() < 0.5 else nbits - 53 - g.randint(53, 75)
+            Z = (Z >> low << low) + (1 << (low - 1)) + g.choice([-1, 0, 1])
+        s = g.choice([g.randint(-300, 50), g.randint(-1200, -1000), g.randint(700, 1100)])
+        V = -Z if g.random() < 0.5 else Z
+        out = D2()
+        lib.bands_to_dd(U6(*[(V >> (32 * t)) & 0xFFFFFFFF for t in range(6)]), s, out)
+        x = Fraction(V) * Fraction(2) ** s
+        if abs(x) >= Fraction(2) ** 1024 * (1 - Fraction(2) ** -54):
+            assert math.isinf(out[0]) and (out[0] < 0) == (V < 0)
+            continue
+        hi, lo = Fraction(out[0]), Fraction(out[1])
+        if x == 0 or abs(x) > Fraction(2) ** -860:
+            assert out[0] == float(x) and out[1] == float(x - hi), (hex(V), s, list(out))
+        else:
+            assert abs(x - hi - lo) <= abs(x) * Fraction(2) ** -106 + Fraction(2) ** -1073
