@@ -315,8 +315,8 @@ __device__ __forceinline__ dd div(dd a, dd b) {
     return q;
 }
 
-// The exponent field of x lies in [128, 1918]: products, quotients and
-// remainders of such numbers with 2^-53-sized factors stay normal.
+// The exponent field of x lies in [128, 1918] (2^-895 to 2^896): its parts
+// 2^-106 below it and its reciprocal are normal.
 __device__ __forceinline__ bool mid_range(double x) {
     return (((unsigned int)__double2hiint(x) >> 20) & 0x7FFu) - 128u <= 1790u;
 }
@@ -326,9 +326,13 @@ __device__ __forceinline__ bool mid_range(double x) {
 // (one FMA) times y corrects it, so the result is a / b rounded once, but for
 // near-ties, and a / b itself whenever that is a binary64 number (Markstein,
 // "Computation of elementary functions on the IBM RISC System/6000
-// processor", 1990).  Three FP64 instructions on the dependent chain, where
-// the division takes as long as nine (576 cycles of a warp).  Operands near
-// the ends of the exponent range, zeros and non-finite ones are divided.
+// processor", 1990), as long as a / b is normal.  Operands of opposite extremes
+// are not singled out: where a / b is below the normal range the result is
+// within a subnormal unit of it, and where it overflows the result is a NaN
+// (which the remainder makes of div_rcp's quotient in any case).  Three FP64
+// instructions on the dependent chain, where the division takes as long as nine
+// (576 cycles of a warp).  Operands near the ends of the exponent range, zeros
+// and non-finite ones are divided.
 __device__ __forceinline__ double quotient(double a, double b, double y) {
     if (!(mid_range(a) && mid_range(b))) return __ddiv_rn(a, b);
     const double q = __dmul_rn(a, y);

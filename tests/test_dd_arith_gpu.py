@@ -156,3 +156,38 @@ def test_division_and_root_over_the_exponent_range(cuda_lib, ea, eb):
     r = q * 2.0 ** (ea // 2)
     zh, zl = run(cuda_lib, "sqrt", (r * r, z0))
     assert np.array_equal(zh, r) and not zl.any()
+
+
+@pytest.mark.parametrize("eq,eb", [(0, -980), (0, 960), (-880, 950), (880, -960), (-850, -100),
+                                   (60, 890), (-440, -440), (440, 440), (-790, 830), (300, -700)])
+def test_exact_quotients_inside_and_outside_the_middle_range(cuda_lib, eq, eb):
+    """Quotients that are binary64 numbers come out exact where a, b or both
+    lie outside the range in which div_rcp multiplies by the reciprocal, and
+    where they lie at its opposite ends."""
+    n = 500
+    g = datagen.rng(920)
+    q = g.integers(1, 2 ** 26, n) * np.where(g.random(n) < 0.5, -1.0, 1.0) * 2.0 ** eq
+    b = g.integers(1, 2 ** 26, n) * np.where(g.random(n) < 0.5, -1.0, 1.0) * 2.0 ** eb
+    a = q * b
+    assert all(Fraction(x) == Fraction(y) * Fraction(z) for x, y, z in zip(a, q, b))
+    z0 = np.zeros(n)
+    zh, zl = run(cuda_lib, "divr", (a, z0), (b, z0))
+    assert np.array_equal(zh, q) and not zl.any()
+
+
+def test_quotients_past_the_ends_of_the_range(cuda_lib):
+    """Operands inside the middle range whose quotient is not a normal number:
+    below it within two subnormal units, above it not finite."""
+    n = 500
+    x, y = operands(921, n), operands(922, n)
+    for ea, eb in ((-700, 500), (-560, 480), (-500, 830)):
+        a, b = tuple(v * 2.0 ** ea for v in x), tuple(v * 2.0 ** eb for v in y)
+        zh, zl = run(cuda_lib, "divr", a, b)
+        for i in range(n):
+            ex = exact("divr", a[0][i], a[1][i], b[0][i], b[1][i])
+            if abs(ex) < Fraction(2) ** -1022:
+                got = Fraction(float(zh[i])) + Fraction(float(zl[i]))
+                assert abs(got - ex) <= Fraction(2) ** -1073
+    a, b = tuple(v * 2.0 ** 700 for v in x), tuple(v * 2.0 ** -500 for v in y)
+    zh, zl = run(cuda_lib, "divr", a, b)
+    assert not np.isfinite(zh).any()
