@@ -235,3 +235,40 @@ def test_alpha_zero_reports_no_product(cuda_lib):
     c = datagen.gemm_case(860, "N", "N", 30, 20, 40, alpha=(0.0, 0.0))
     _, _, rep = run_form(cuda_lib, "crt", c)
     assert rep["form"] == 0 and rep["width_bits"] == 0
+
+
+@pytest.mark.parametrize("pad", [0, 1])
+def test_large_fallback_equals_the_plain_kernel(cuda_lib, pad):
+    """No width certifies and the output has 152 or more 64 x 64 tiles: the
+    plain kernel behind the call is the TMA-staged one (1216 x 512, even
+    leading dimensions) or has 64 x 64 register-staged tiles (1216 x 1024, odd
+    ones).  The same bits as mp_dd_Rgemm, which takes smaller tiles."""
+    mp = cuda_lib
+    m, n, k = 1216, 1024 if pad else 512, 40
+    c = adversarial_case(870, m + pad, n, k + pad)
+    c.m, c.k = m, k
+    got, _, rep = run_form(mp, "crt", c)
+    assert rep["width_bits"] == 0
+    A, B, C = dev(c.A), dev(c.B), dev(c.C)
+    mp.mp_dd_Rgemm("N", "N", m, n, k, c.alpha, A, m + pad, B, k + pad, c.beta, C, m + pad)
+    want = host(C, m, n)
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    g = datagen.rng(871)
+    rows, cols = g.integers(0, m, 300), g.integers(0, n, 300)
+    rows[:30], cols[30:60] = m - 1, n - 1
+    assert check_against_exact(c, got, rows, cols) <= 1.0
+
+
+@pytest.mark.parametrize("uplo", ["U", "L"])
+def test_large_rsyrk_fallback_equals_the_plain_kernel(cuda_lib, uplo):
+    """The same for the Rsyrk triangle: 325 tiles of 64 x 64 at n = 1600."""
+    mp = cuda_lib
+    n, k = 1600, 40
+    A = _syrk_stress(872, n, k, 2.0 ** -45)
+    C = datagen.dd_matrix(datagen.rng(873), n, n)
+    got, rep = run_syrk_crt(mp, uplo, "N", n, k, (1.5, 0.0), A, (0.0, 0.0), C)
+    assert rep["width_bits"] == 0
+    dA, dC = dev(A), dev(C)
+    mp.mp_dd_Rsyrk(uplo, "N", n, k, (1.5, 0.0), dA, n, (0.0, 0.0), dC, n)
+    want = host(dC, n, n)
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
