@@ -968,7 +968,11 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
 
     const int a_rc = p.ta ? 0 : 1, b_rc = p.tb ? 1 : 0;
     int rc;
-    sliced_timing_mark(0, st);
+    // (an update inside a solve or factorisation is not one of the timed calls)
+    auto mark = [&](int phase) {
+        if (p.tight == 0.0) sliced_timing_mark(phase, st);
+    };
+    mark(0);
     const SplitOperand oa{p.ah, p.al, p.lda, a_rc, p.m, L.m_pad, rmax, w + L.off_ma, 0};
     const SplitOperand ob{p.bh, p.bl, p.ldb, b_rc, p.n, L.n_pad, cmax, w + L.off_mb, 0};
     // (the Rsyrk form has one operand: its maxima and planes serve as both)
@@ -979,7 +983,7 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
         return rc;
     if ((rc = launch_residues(oa, RA, sym ? nullptr : &ob, RB, p.k, L.k_pad, plan, st))) return rc;
 
-    sliced_timing_mark(1, st);
+    mark(1);
     CUtensorMap tmA, tmB;
     if ((rc = make_tmap(&tmA, RA, (int64_t)L.N * L.m_pad, L.k_pad, kBandTM))) return rc;
     if ((rc = make_tmap(&tmB, RB, (int64_t)L.N * L.n_pad, L.k_pad, TN))) return rc;
@@ -1004,7 +1008,7 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
         ba.run_kb[i] = (1 << 24) / (r * r) / kBandTK;   // r^2 64 run_kb <= 2^24
     }
     if ((rc = launch_band(tmA, tmB, ba, TN, st, &tmB_half))) return rc;
-    sliced_timing_mark(2, st);
+    mark(2);
 
     // CRT constants of every candidate
     CrtArgs ca{};
@@ -1052,7 +1056,7 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
                                       : launch_chained(crt_kernel<9, 9>, nb, 256, 0, st, ca);
     if ((rc = chained_ok(le, "crt_kernel"))) return rc;
     rc = launch_plain_fallback(p, plan, st);
-    sliced_timing_mark(3, st);
+    mark(3);
     return rc;
 }
 

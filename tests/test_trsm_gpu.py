@@ -212,3 +212,35 @@ def test_tensor_core_updates(cuda_lib, side, uplo, transa, diag, form):
         for P in (*c.B, *X):
             P[~np.isfinite(P)] = 0.0
     assert trsm_residual_over_bound(c, X, rows, cols) <= 0.1
+
+
+def test_updates_are_not_in_the_phase_log(cuda_lib):
+    """The phase log holds the split-precision calls, not the tensor-core
+    updates that Rtrsm, Rgetrf and Rgetrs make between them (order 512 with
+    512 right-hand sides: the 256 x 512 x 256 update of a solve, 471 us on the
+    FP64 pipe by the launch's count, runs in residue form)."""
+    mp = cuda_lib
+    n = 512
+    c = datagen.trsm_case(862, "L", "L", "N", "N", n, n)
+    A, B = dev(c.A), dev(c.B)
+    g = datagen.rng(863)
+    F, P, Q = (dev(datagen.dd_matrix(g, n, n)) for _ in range(3))
+    ipiv = torch.empty(n, dtype=torch.int64, device="cuda")
+    info = torch.empty(1, dtype=torch.int64, device="cuda")
+    ws = mp.workspace(mp.mp_dd_Rgemm_crt_workspace(64, 64, 64))
+
+    def product():
+        mp.mp_dd_Rgemm_crt("N", "N", 64, 64, 64, (1.0, 0.0), P, n, P, n, (0.0, 0.0), Q, n, ws,
+                           ws.numel())
+
+    mp.mp_dd_sliced_timing(True)
+    try:
+        product()
+        mp.mp_dd_Rtrsm("L", "L", "N", "N", n, n, c.alpha, A, n, B, n)
+        product()
+        mp.mp_dd_Rgetrf(n, n, F, n, ipiv, info)
+        mp.mp_dd_Rgetrs("N", n, n, F, n, ipiv, B, n)
+        log = mp.mp_dd_sliced_phase_log()
+    finally:
+        mp.mp_dd_sliced_timing(False)
+    assert len(log) == 2 and all(t > 0 for row in log for t in row)
