@@ -244,7 +244,10 @@ int mp_dd_Rsyrk_host(const char *uplo, const char *trans, int64_t n, int64_t k, 
  * a pool of the library that keeps at most 2 GiB between calls) cannot be had.  Accuracy: the componentwise backward error of
  * substitution, |op(A) X - alpha B| <= 4 (n_A + 2) 2^-104 (|op(A)||X| +
  * |alpha B|), n_A the order of A; a zero diagonal entry gives Inf/NaN as
- * DTRSM does (no check).  Asynchronous on the current stream.
+ * DTRSM does (no check).  Within it, a right-hand side's low-order bits may
+ * depend on how many others there are, on their values (one operand width
+ * serves an update) and on which of the two forms the above leaves an update
+ * to; up to 95 right-hand sides there is one form and they depend on neither.  Asynchronous on the current stream.
  * Errors: -1 side, -2 uplo, -3 transa, -4 diag, -5 m < 0, -6 n < 0,
  * -8 A planes NULL, -9 lda < max(1, order of A), -10 B planes NULL,
  * -11 ldb < max(1, m) (DTRSM's numbering). */
@@ -264,7 +267,8 @@ int mp_dd_Rtrsm(const char *side, const char *uplo, const char *transa, const ch
  * j > 0 when U(j, j) is exactly zero (the factorisation completes, as in
  * LAPACK).  Recursive column splitting (LAPACK's dgetrf2): the updates are
  * dd Rtrsm and dd Rgemm products (the large ones on the tensor cores, as in
- * mp_dd_Rtrsm), the leaves panels of at most 32 columns,
+ * mp_dd_Rtrsm, whose note on the low-order bits holds here too), the leaves
+ * panels of at most 32 columns,
  * each one cooperative launch with its rows spread over the SMs.  A
  * panel's grid-barrier waits are bounded (~2 s, which co-resident CTAs
  * never reach); a wait that gives up stops the panel and sets *info = -1.
@@ -279,7 +283,8 @@ int mp_dd_Rgetrf(int64_t m, int64_t n, mp_dd_mat A, int64_t lda, int64_t *ipiv,
 /* Rgetrs (DGETRS semantics): solve A X = B (trans 'N') or A^T X = B ('T';
  * 'C' is 'T') with the factors and ipiv (device) of mp_dd_Rgetrf on the
  * n x n A; B (n x nrhs) is overwritten by X.  Row interchanges, then unit
- * lower and upper dd Rtrsm (reverse order for 'T').  Asynchronous.
+ * lower and upper dd Rtrsm (reverse order for 'T'; its note on the low-order
+ * bits holds here too).  Asynchronous.
  * Errors: -1 trans, -2 n < 0, -3 nrhs < 0, -4 A NULL, -5 lda < max(1, n),
  * -6 ipiv NULL, -7 B NULL, -8 ldb < max(1, n). */
 int mp_dd_Rgetrs(const char *trans, int64_t n, int64_t nrhs, mp_dd_cmat A, int64_t lda,

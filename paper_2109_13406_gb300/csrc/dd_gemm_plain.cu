@@ -358,8 +358,11 @@ int launch_plain_fallback(const GemmArgs &p, const SplitPlan &plan, cudaStream_t
 // with 500 right-hand sides: 71.0 ms with every update on the FP64 pipe
 // (9.75 instructions a multiply-add), 31.9 so.
 // The inner dimension and both outer ones have to reach kUpdateMin: below it
-// the time is latency either way, and a solve's or a factorisation's result
-// then does not depend on how many columns go with it.
+// the time is latency either way, and so solves of up to 95 right-hand sides
+// never leave the FP64 pipe and each one's result is its own.  From there on the
+// estimates depend on the number of columns, and the operand width on all of
+// their values, so a right-hand side's low bits can differ with the others that
+// go with it (within the bound of either form).
 // With `tight` = 2 the residue form's operand rounding stays within 2 u^2
 // (|A||B| + |C|) entry by entry, and its other roundings within 4 u^2, against
 // the plain kernel's sum of k roundings of up to ~8 u^2; a call whose operands
