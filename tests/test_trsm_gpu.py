@@ -273,3 +273,33 @@ def test_right_hand_sides_alone_and_with_others(cuda_lib, side, uplo, transa):
         outs[w] = tuple(x[:, :6] if side == "L" else x[:6] for x in X)
     for a, b in zip(outs[6], outs[95]):
         assert np.array_equal(a, b)
+
+
+def test_updates_in_blocks_of_the_scratch_limit(cuda_lib):
+    """X op(A) = alpha B of order 512 with 160000 rows of B: the 160000 x 256 x
+    256 update's workspace is above 4 GiB, so it runs in two blocks of at most
+    80128 rows.  The rows at both ends and on either side of the border meet a
+    tenth of the bound of substitution (three updates of 6u^2 and 64 steps of
+    8u^2 against 16 * 514 u^2: 0.065)."""
+    mp = cuda_lib
+    m, n = 160000, 512
+    assert mp.mp_dd_Rgemm_crt_workspace(m, 256, 256) > 4 << 30
+    assert mp.mp_dd_Rgemm_crt_workspace(80128, 256, 256) <= 4 << 30
+    c = datagen.trsm_case(866, "R", "U", "N", "N", 8, n)
+    gen = torch.Generator(device="cuda").manual_seed(867)
+    hi, lo = (torch.empty(n, m, dtype=torch.float64, device="cuda").uniform_(-1, 1, generator=gen)
+              for _ in range(2))
+    lo *= hi * 2.0 ** -54
+    rows = np.r_[0:40, 80108:80148, m - 40:m]
+    at = torch.from_numpy(rows).cuda()
+
+    def picked():
+        return tuple(np.asfortranarray(x[:, at].cpu().numpy().T) for x in (hi, lo))
+
+    c.B, c.m = picked(), len(rows)
+    mp.mp_dd_Rtrsm("R", "U", "N", "N", m, n, c.alpha, dev(c.A), n, (hi, lo), m)
+    torch.cuda.synchronize()
+    g = datagen.rng(868)
+    r = np.tile(np.arange(len(rows)), 10)
+    cols = np.where(g.random(len(r)) < 0.7, g.integers(256, n, len(r)), g.integers(0, n, len(r)))
+    assert trsm_residual_over_bound(c, picked(), r, cols) <= 0.1
