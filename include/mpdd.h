@@ -135,13 +135,13 @@ int mp_dd_Rgemm(const char *transa, const char *transb, int64_t m, int64_t n, in
 
 /* Operand staging of the plain Rgemm / Rsyrk kernel (no counterpart in the
  * manual; process-wide, for tuning and testing).  mode 0 (the default):
- * Rgemm products large enough for 64 x 64 output tiles whose A and B planes
- * start on 16-byte boundaries with even leading dimensions are computed by
- * a kernel whose op(A) / op(B) panels arrive by TMA tile copies into a ring
- * of shared-memory stages (mbarrier-synchronised, one producer warp, eight
- * computing warps); the others (thin products, the Rsyrk triangle) by the
- * register-staged kernels on the tile size that fills the SMs best.  mode 1: register staging only.  mode 2: TMA
- * staging wherever its alignment rules allow, whatever the size.  Every
+ * register-staged kernels on the tile size that fills the SMs best; behind a
+ * split-precision product large enough for 64 x 64 tiles, whose plain kernel
+ * mostly has nothing to do, the TMA-staged one.  mode 1: register staging
+ * only.  mode 2: op(A) / op(B) panels by TMA tile copies into a ring of
+ * shared-memory stages (mbarrier-synchronised, one producer warp, eight
+ * computing warps) wherever its alignment rules allow (A and B planes on
+ * 16-byte boundaries, even leading dimensions), whatever the size.  Every
  * mode gives bitwise the same results (the per-entry operation sequence is
  * the same).  Returns 0, or -1 for another mode. */
 int mp_dd_set_plain_staging(int mode);
@@ -364,7 +364,7 @@ typedef struct {
 /* One launch: one CTA per diagonal block.  Errors: -1 count, -2 descs. */
 int mp_dd_potrf_diag_batch(int64_t count, const mp_dd_potrf_diag_desc *descs);
 
-/* One launch over count descriptors, 4 to 32 right-hand-side columns per
+/* One launch over count descriptors, 2 to 32 right-hand-side columns per
  * CTA (chosen from count and max_nrhs; the result does not depend on it);
  * max_nrhs is the largest nrhs in the batch.  Errors: -1, -2, -3. */
 int mp_dd_trsm_batch(int64_t count, const mp_dd_trsm_desc *descs, int64_t max_nrhs);
@@ -673,13 +673,14 @@ int mp_dd_peak_fp64(double *rate);
  * fp16 tcgen05 path is compared.  Synchronous.  Returns 0 or an error. */
 int mp_dd_peak_imma(double *rate);
 
-/* Time the dd multiply-add (the plain kernel's operation sequence, 4 x 4
- * accumulators per thread, renormalised every 4 steps) on operands that stay
+/* Time the dd multiply-add with every operation on the FP64 pipe (4 x 4
+ * accumulators per thread, renormalised by FastTwoSum every 4 steps: 9.75
+ * instructions a step) on operands that stay
  * in registers and change every step by integer operations only, filling
  * every SM, and report the rate in dd multiply-adds per second (twice it in
- * dd-flop/s) in *rate: the ceiling of the all-FP64 form on this GPU's FP64
- * pipe.  (The GEMM kernels form the sums' rounding errors on the integer pipe,
- * to the same bits, and run above it.)  Synchronous.  Returns 0 or an error. */
+ * dd-flop/s) in *rate: the ceiling of that form on this GPU's FP64 pipe.  (The
+ * GEMM kernels form the rounding errors of sums and products on the integer
+ * pipe, to the same bits, renormalise by TwoSum, and run above it.)  Synchronous.  Returns 0 or an error. */
 int mp_dd_peak_ddmac(double *rate);
 
 #ifdef __cplusplus

@@ -99,11 +99,13 @@ __device__ __forceinline__ void mac(dd &acc, dd a, dd b) {
 
 // GEMM-loop multiply-add with deferred renormalisation: the leading parts
 // are summed with TwoSum (exact), the TwoSum error and the product's low
-// part are added into acc.lo, and the FastTwoSum is left to renorm(), which
-// the GEMM kernels call after every kRenormEvery steps of k (at l = 3, 7, 11,
-// ... counted from the start of k, so every kernel renormalises at the same
-// places).  4 + 3 + 2 = 9 FP64 operations per step, 9.75 with the
-// renormalisation (3 + 1 + 2 and 0.25 with the errors on the integer pipe).  Between renormalisations |acc.lo| stays within a few
+// part are added into acc.lo, and the renormalisation is left until after
+// every kRenormEvery steps of k (at l = 3, 7, 11, ... counted from the start of
+// k, so every kernel renormalises at the same places): TwoSum in the GEMM
+// kernels (renorm_mixed and renorm_exact, the same bits), FastTwoSum (renorm)
+// in the Cholesky diagonal block and the 64-row solves.  4 + 3 + 2 = 9 FP64
+// operations per step, 9.75 with the renormalisation (3 + 1 + 2 and 0.25 with
+// the errors on the integer pipe).  Between renormalisations |acc.lo| stays within a few
 // ulps of acc.hi, so each step's rounding error is at most ~(G+4) u^2
 // (|acc| + |a b|) with G = 4: within the Rgemm bound 4 k 2^-104 (...).  A
 // zero product leaves the state unchanged, so zero padding of k does not

@@ -830,11 +830,11 @@ int launch_residues(const SplitOperand &a, __half *ra, const SplitOperand *b, __
             for (int64_t r = 1; r <= 16; ++r) {
                 const int64_t ta = ceil_div(ia, r), tb = slots - ta;
                 if (tb < 1) continue;
-                const int64_t rb = ceil_div(ib, tb), t = r * ca > rb * cb ? r * ca : rb * cb;
+                const int64_t q = ceil_div(ib, tb), t = r * ca > q * cb ? r * ca : q * cb;
                 if (best < 0 || t < best) {
                     best = t;
                     na = ta;
-                    nb = ceil_div(ib, rb);
+                    nb = ceil_div(ib, q);
                 }
             }
         }
@@ -909,8 +909,10 @@ size_t crt_workspace_bytes(int64_t m, int64_t n, int64_t k, bool sym) {
 }
 
 double crt_estimate_us(int64_t m, int64_t n, int64_t k) {
-    // launches and latencies, then reconstruction, residues and products;
-    // measured: 64 x 2048 x 192 66 us, 512^3 80, 1024^3 181, 1501 x 2777 x 1999 757
+    // launches and latencies, then reconstruction, residues and products; fitted
+    // to 64 x 2048 x 192 66 us, 512^3 80, 1024^3 181, 1501 x 2777 x 1999 757, before
+    // the small kernels of a call were shortened (512^3: 58 us), so that products
+    // near the rule's line stay on the FP64 pipe a little longer than they need
     const double dm = (double)m, dn = (double)n, dk = (double)k;
     return 60.0 + 4e-5 * dm * dn + 1.6e-5 * (dm + dn) * dk + 5e-8 * dm * dn * dk;
 }

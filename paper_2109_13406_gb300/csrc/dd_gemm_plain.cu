@@ -342,9 +342,9 @@ int launch_plain_fallback(const GemmArgs &p, const SplitPlan &plan, cudaStream_t
     q.gate = plan.dmin;
     q.gate_below = plan.thr[plan.ncand - 1];
     // with the gate closed every CTA returns at once, so the launch costs
-    // about its CTA count: the persistent TMA-staged kernel where it applies,
-    // else the 64 x 64 tiles whenever they fill the SMs twice (the result
-    // does not depend on the staging or the tile size)
+    // about its CTA count: 64 x 64 tiles, TMA-staged where that applies, else
+    // register-staged whenever they fill the SMs twice (the result does not
+    // depend on the staging or the tile size)
     int rc = 0;
     if (try_launch_gemm_tma(q, stream, &rc)) return rc;
     const int64_t sms = sm_count() > 0 ? sm_count() : 152;

@@ -5,9 +5,9 @@
 // dd_arith.cuh with the renormalisation every 4 steps of k, l = 0 .. k-1 in
 // order -- with the operand panels moved by the tensor memory accelerator:
 //
-//  * one CTA per 64 x 64 output tile (the plain kernel's tile order: groups
-//    of 8 tile columns, or the triangle), one CTA per SM at a time, so the
-//    hardware hands the next tile to whichever SM finishes first;
+//  * one CTA per 64 x 64 output tile (in the plain kernel's order: groups of 8
+//    tile columns, or the triangle), one CTA per SM at a time, so the hardware
+//    hands the next tile to whichever SM finishes first;
 //  * one producer warp issues, for every 16-wide panel of k, four 2-D tile
 //    copies (cp.async.bulk.tensor: the hi and lo planes of op(A) and op(B),
 //    64 x 16 binary64 each) into a ring of kStages stages, completing the
@@ -322,11 +322,12 @@ int plain_staging() { return g_staging.load(); }
 // product, no symmetric operand, alpha != 0) whose planes start on 16-byte
 // boundaries with even leading dimensions (the copy engine's stride rule).
 // Automatically it takes only the gated Rgemm launches behind a certificate
-// that are large enough for 64 x 64 tiles: with the gate closed its one CTA per
-// SM returns at once.  Plain products run faster on the register-staged 16 x
-// 16 tiles, whose six or more warps a partition cover the integer part of the
-// multiply-add that this kernel's two do not (8192 x 8192 x 256: 197 ms against
-// 222).  Returns 1 when it launched (or failed to: *rc), 0 when
+// that fill the SMs with 64 x 64 tiles: with the gate closed, the usual case,
+// every CTA returns at once and the launch costs its CTA count, a sixteenth of
+// the 16 x 16 tiles' (16384 at 8192 x 8192).  With the gate open, as for any plain
+// product, the register-staged 16 x 16 tiles are faster: their six or more warps
+// a partition cover the integer part of the multiply-add that this kernel's two
+// do not (8192 x 8192 x 256: 197 ms against 222).  Returns 1 when it launched (or failed to: *rc), 0 when
 // the caller should use the register-staged kernels.
 int try_launch_gemm_tma(const GemmArgs &p, cudaStream_t st, int *rc) {
     if (g_staging.load() == 1) return 0;

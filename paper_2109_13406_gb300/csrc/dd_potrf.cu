@@ -54,9 +54,10 @@ __host__ __device__ __forceinline__ int64_t uidx(int lower, int64_t i, int64_t j
 // barrier two warps of each CTA take the square root of (j, j), with an
 // approximate reciprocal of it, and divide the row by it (div_rcp), all
 // lanes the same root and each its column; after a block barrier every
-// entry (r, c) with j < r <= c subtracts U(j, r) U(j, c), with the GEMM
-// kernels' deferred renormalisation (every entry has taken exactly j + 1
-// updates after step j, so all renormalise at the same steps).  (With the root
+// entry (r, c) with j < r <= c subtracts U(j, r) U(j, c), the
+// renormalisation (FastTwoSum) deferred to every 4th step (every entry has
+// taken exactly j + 1 updates after step j, so all renormalise at the same
+// steps).  (With the root
 // and the quotients formed by their holders and sent to the others, a step
 // had two cluster barriers: 150 us a block, 135 so.)
 //
@@ -296,8 +297,8 @@ __host__ __device__ constexpr size_t trsm_smem_bytes(int cols) {
 // (q < 64 / RG) as dd accumulators in registers.  Step i: the owner of row i
 // finishes x_i (its accumulator, divided by U(i, i)) and publishes it in
 // shared memory; after one barrier every thread subtracts U-entry x_i from
-// its rows still to be solved, with the deferred renormalisation of the GEMM
-// kernels (TwoSum on the leading parts, a FastTwoSum every 4 steps).  U's
+// its rows still to be solved, the renormalisation (FastTwoSum) deferred to
+// every 4th step.  U's
 // triangle sits in shared memory packed in the order the steps read it: by
 // rows for U^T (step i reads U(i, i+1:)), by columns for U (step i reads
 // U(:i-1, i)).  Every row takes the same operations in the same order
@@ -1062,8 +1063,9 @@ __global__ void __launch_bounds__(256) laswp_perm_kernel(double *ah, double *al,
 
 // C(m x n) -= A(m x k) B(k x n), all column-major, for small k or n: one
 // thread per entry of C, multiply-adds l = 0 .. k-1 straight into C's value.
-// (The 64 x 64 tiles of the Rgemm kernel would compute zero-padded products
-// worth up to 16 / k and 64 / n times the useful ones.)
+// (The Rgemm kernel's panels of 16 steps and tiles of 16, 8 or 4 columns would
+// compute zero-padded products worth up to 16 / k and 4 / n times the useful
+// ones.)
 __global__ void __launch_bounds__(256) small_update_kernel(
     int64_t m, int64_t n, int64_t k, const double *__restrict__ ah,
     const double *__restrict__ al, int64_t lda, const double *__restrict__ bh,

@@ -1440,10 +1440,6 @@ int run_sliced(const GemmArgs &p, int slices, void *ws, size_t ws_bytes, cudaStr
 
 namespace {
 
-}  // namespace
-
-namespace {
-
 // Geometry of the triangle table for a launch (ba.tri_on stays 0 when the
 // table does not apply: no triangle, or too many rows for shared memory).
 void tri_prepare(BandArgs &ba, int TN, bool pair) {

@@ -44,7 +44,8 @@ struct GemmArgs {
     double tight = 0.0;
 };
 
-// Plain FP64 dd kernel (64 x 64 output tiles, 4 x 4 dd accumulators per thread).
+// Plain FP64 dd kernel (16 x 16 output tiles, 16 x 8 or 32 x 4 where those are
+// too few to fill the SMs; the TMA-staged form where plain_staging() asks for it).
 int launch_gemm_plain(const GemmArgs &p, cudaStream_t stream);
 // An update of a factorisation or solve: the residue form at dd accuracy
 // (tight) where it is faster and its workspace can be had, else the plain

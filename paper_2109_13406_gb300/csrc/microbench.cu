@@ -6,9 +6,10 @@
 // bounded (x <- x * b + c with |b| < 1) so no operand becomes denormal.
 //
 // dd multiply-add rate: the multiply-add with every operation on the FP64 pipe
-// (mac_deferred, renorm every kRenormEvery steps: 9.75 instructions; the GEMM
-// kernels form rounding errors on the integer pipe, to the same bits, and run
-// above this rate) on a 4 x 4 block of accumulators per
+// (mac_deferred, renorm every kRenormEvery steps: 9.75 instructions, as in the
+// Cholesky diagonal block and the 64-row solves; the GEMM kernels form the same
+// rounding errors on the integer pipe, renormalise by TwoSum and run above this
+// rate) on a 4 x 4 block of accumulators per
 // thread, with operands that change every step through integer operations
 // on their bit patterns (no FP64 instruction and no memory access besides
 // the multiply-adds, and nothing the compiler can hoist): the ceiling of that
