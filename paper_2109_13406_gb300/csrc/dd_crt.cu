@@ -413,8 +413,9 @@ struct CrtArgs {
     const unsigned long long *rmax, *cmax;
     mp_dd alpha, beta;
     int alpha_one, beta_zero;
-    int ab_mode;                          // 0 general; alpha = +-1 and beta = 0 (1) or 1 (2)
-    int alpha_neg;                        // alpha = -1 (modes 1, 2)
+    int ab_mode;                          // 0 general; alpha = +-1 and beta = 0 (1) or 1 (2);
+                                          // 3 (updates): alpha = +-1, general beta
+    int alpha_neg;                        // alpha = -1 (modes 1 to 3)
     double *ch, *cl;
     int64_t ldc;
     int tri;                              // 0: all of C; 1 / 2: upper / lower triangle
@@ -509,7 +510,8 @@ __device__ __forceinline__ void crt_store(const CrtArgs &p, dd v, int64_t off, d
             break;
         default:
             if (UPD && !p.beta_zero)
-                r = add(mul(dd{p.alpha.hi, p.alpha.lo}, v),
+                r = add(p.ab_mode == 3 ? (p.alpha_neg ? dd{-v.hi, -v.lo} : v)
+                                       : mul(dd{p.alpha.hi, p.alpha.lo}, v),
                         mul(dd{p.beta.hi, p.beta.lo}, dd{ch, cl}));
             else if (!p.beta_zero)
                 r = axpby_dd(dd{p.alpha.hi, p.alpha.lo}, v, dd{p.beta.hi, p.beta.lo}, dd{ch, cl});
@@ -552,7 +554,8 @@ __device__ __forceinline__ void crt_pair(const CrtArgs &p, const CrtTables &T, i
             R1[g] = __byte_perm(v[2 * g], v[2 * g + 1], 0x7531);   // entry i + 1
         }
     }
-    const bool use_c = p.ab_mode == 2 || (p.ab_mode == 0 && !p.beta_zero);
+    const bool use_c = p.ab_mode == 2 || (UPD && p.ab_mode == 3) ||
+                       (p.ab_mode == 0 && !p.beta_zero);
     const int64_t off = i + j * p.ldc;
     const int ec = scale_exponent(__ldg(p.cmax + j)) - 2 * W;
     double c0h = 0.0, c0l = 0.0, c1h = 0.0, c1l = 0.0;
@@ -602,7 +605,8 @@ __device__ __forceinline__ void crt_one(const CrtArgs &p, const CrtTables &T, in
     }
 #pragma unroll
     for (int g = 0; g < G; ++g) R[g] = __byte_perm(v[2 * g], v[2 * g + 1], sel);
-    const bool use_c = p.ab_mode == 2 || (p.ab_mode == 0 && !p.beta_zero);
+    const bool use_c = p.ab_mode == 2 || (UPD && p.ab_mode == 3) ||
+                       (p.ab_mode == 0 && !p.beta_zero);
     const int64_t off = i + j * p.ldc;
     const double ch = use_c ? p.ch[off] : 0.0, cl = use_c ? p.cl[off] : 0.0;
     const int sc = scale_exponent(__ldg(p.rmax + i)) + scale_exponent(__ldg(p.cmax + j)) - 2 * W;
@@ -1034,7 +1038,7 @@ int run_crt(const GemmArgs &p, void *ws, size_t ws_bytes, cudaStream_t st) {
     {
         const bool a_pm1 = p.alpha.lo == 0.0 && (p.alpha.hi == 1.0 || p.alpha.hi == -1.0);
         const bool b_one = p.beta.hi == 1.0 && p.beta.lo == 0.0;
-        ca.ab_mode = a_pm1 && p.beta_zero ? 1 : (a_pm1 && b_one ? 2 : 0);
+        ca.ab_mode = !a_pm1 ? 0 : p.beta_zero ? 1 : b_one ? 2 : p.tight > 0.0 ? 3 : 0;
         ca.alpha_neg = p.alpha.hi < 0.0;
     }
     int nw[kMaxCand] = {0, 0, 0};
